@@ -209,7 +209,7 @@ int lbpf_write_fields(lbpf_ctx* ctx, int domain, const void* phi, const void* u,
 /* Advance every domain by n_steps time steps (n_steps >= 0).  One step is
  * the phase-field scheme of Sec. 3.2 followed by the heat scheme of Sec. 3.1
  * with Q_u = (phi(t + dt) - phi(t)) / (2 dt), one kernel launch for all
- * domains.  On a non-default stream, runs of 16 steps are replayed from CUDA
+ * domains (two where the vector form applies, see LBPF_Q_KERNEL).  On a non-default stream, runs of 16 steps are replayed from CUDA
  * graphs captured on first use (do not call lbpf_step while another capture
  * is active on the context's stream).  Asynchronous on the context's stream
  * (except the first call of a context whose schedule is timed, see
@@ -319,13 +319,18 @@ typedef enum {
     LBPF_Q_TILE_ROWS = 6,      /* tile variant of the step kernel (autotuned): 8, 16 */
     LBPF_Q_SEGMENT = 7,        /* z-planes (3D) or y-rows (2D) per work item          */
     LBPF_Q_BLOCKS = 8,         /* resident blocks of the persistent step launch       */
-    LBPF_Q_KERNEL = 9          /* step kernel: 0 generic (global-memory pulls, the
-                                  default), 1 staged (rows brought to shared memory by
-                                  asynchronous copies; chosen by the environment
-                                  variable LBPF_KERNEL=staged at lbpf_create for 3D
-                                  D3Q15/D3Q19 domains with 16-bit deviation storage,
-                                  nx a multiple of 8 and >= 64, one crystal; same
-                                  results bit for bit, slower on GB300)             */
+    LBPF_Q_KERNEL = 9          /* step kernel: 0 the library's choice (3D contexts with
+                                  16-bit deviation storage whose domains have one crystal,
+                                  no velocity, nx a multiple of 4, >= 8 and not 4 above a
+                                  multiple of 64: two launches a step with four sites a
+                                  thread; otherwise one launch, global-memory pulls), 1
+                                  staged (rows brought to shared memory by asynchronous
+                                  copies; chosen by the environment variable
+                                  LBPF_KERNEL=staged at lbpf_create for 3D D3Q15/D3Q19
+                                  domains with 16-bit deviation storage, nx a multiple of
+                                  8 and >= 64, one crystal; slower on GB300).
+                                  LBPF_KERNEL=generic keeps the one-launch kernel.  Same
+                                  results bit for bit in every case                 */
 } lbpf_query_t;
 
 /* Override the work schedule of the step kernel.  Normally lbpf_create takes

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "staged_kernel.cuh"
+#include "vec_kernel.cuh"
 
 namespace lbpf {
 
@@ -329,6 +330,17 @@ struct LauncherImpl {
                 if (e != cudaSuccess) return e;
             }
         }
+        if constexpr (kVec) {
+            if (v == 0) {
+                cudaError_t e = cudaFuncSetAttribute(phi_vec_kernel<PL, S, false>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)VecSmem<PL>::bytes);
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(phi_vec_kernel<PL, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)VecSmem<PL>::bytes);
+                if (e != cudaSuccess) return e;
+            }
+        }
         const int b0 = (int)smem_v<0>();
         if (v == 1) return cudaFuncSetAttribute(kernel<1>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_v<1>());
         cudaError_t e = cudaFuncSetAttribute(kernel<0, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, b0);
@@ -361,6 +373,49 @@ struct LauncherImpl {
                 cudaGetLastError();
                 return 1;
             }
+        }
+        return nb > 0 ? nb : 1;
+    }
+    // the vector step: 3D, 16-bit deviations
+    static constexpr bool kVec = PL::D == 3 && S::dev;
+    static cudaError_t heat_vec(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s)
+    {
+        if constexpr (kVec) {
+            const int gx = (h.nx / 4 + kHeatX - 1) / kHeatX, gy = (h.ny + kHeatY - 1) / kHeatY;
+            int zlen = 16;
+            while (zlen > 1 && (long long)gx * gy * ((h.nz + zlen - 1) / zlen) < 152 * 8) zlen /= 2;
+            const dim3 grid(gx, gy, (h.nz + zlen - 1) / zlen), block(kHeatX, kHeatY);
+            if (h.bc)
+                heat_vec_kernel<UL, S, true><<<grid, block, 0, s>>>(d, a.cur, a.fcur, a.acur, a.collide, zlen, a.counters);
+            else
+                heat_vec_kernel<UL, S, false><<<grid, block, 0, s>>>(d, a.cur, a.fcur, a.acur, a.collide, zlen, a.counters);
+            return cudaGetLastError();
+        } else {
+            return cudaErrorNotSupported;
+        }
+    }
+    static cudaError_t phi_vec(int walls, const StepArgs& a, int n_blocks, cudaStream_t s)
+    {
+        if constexpr (kVec) {
+            if (walls)
+                phi_vec_kernel<PL, S, true><<<n_blocks, kVecNT, VecSmem<PL>::bytes, s>>>(a);
+            else
+                phi_vec_kernel<PL, S, false><<<n_blocks, kVecNT, VecSmem<PL>::bytes, s>>>(a);
+            return cudaGetLastError();
+        } else {
+            return cudaErrorNotSupported;
+        }
+    }
+    static int vec_blocks_per_sm(int walls)
+    {
+        int nb = 0;
+        if constexpr (kVec) {
+            const cudaError_t e =
+                walls ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, phi_vec_kernel<PL, S, true>, kVecNT,
+                                                                      VecSmem<PL>::bytes)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, phi_vec_kernel<PL, S, false>, kVecNT,
+                                                                      VecSmem<PL>::bytes);
+            if (e != cudaSuccess) cudaGetLastError();
         }
         return nb > 0 ? nb : 1;
     }
@@ -416,6 +471,8 @@ struct LauncherImpl {
     {
         static const Launchers L = {&step,     &smem,           &prepare,  &blocks_per_sm,
                                     kStaged ? &step_staged : nullptr,      &staged_blocks_per_sm,
+                                    kVec ? &heat_vec : nullptr,            &phi_vec,
+                                    &vec_blocks_per_sm,
                                     &heat_sync, &equilibrate,   &read_u,   &read_pop,
                                     &read_as,  PL::Q,          UL::Q,     PL::D};
         return &L;

@@ -1,5 +1,6 @@
 // Host side of the lbpf C ABI: context, device buffers, launches and the
 // lagged/synchronised state of the heat populations.  See include/lbpf.h.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -44,6 +45,7 @@ struct lbpf_ctx {
     int n_items = 0, n_blocks = 0, items_cap = 0;
     int tile_v = 0, seg_len = 0, sms = 1;
     bool staged = false;  // step kernel with bulk-copy staging (staged_kernel.cuh)
+    bool vec = false;     // vector step: two launches, four sites a thread (vec_kernel.cuh)
     int kind = 0;         // step kernel kind: kStepWalls (some domain has walls) | kStepAdvect
     // graphs of kGraphSteps steady-state launches, keyed by (cur, fcur, acur)
     cudaGraphExec_t graphs[8] = {};
@@ -122,7 +124,7 @@ static void free_all(lbpf_ctx* c)
 // ---------------------------------------------------------------------------
 static long long column_units(const lbpf_ctx* c, int v)
 {
-    const int tx = tile_x(c->dim, v), ty = tile_y(c->dim, v);
+    const int tx = c->vec ? kVecTX : tile_x(c->dim, v), ty = c->vec ? kVecTY : tile_y(c->dim, v);
     long long units = 0;
     for (const DomainDev& d : c->dd) {
         const int ny = c->dim == 3 ? d.ny : 1, nz = c->dim == 3 ? d.nz : d.ny;
@@ -133,6 +135,7 @@ static long long column_units(const lbpf_ctx* c, int v)
 
 static int blocks_per_sm(const lbpf_ctx* c, int v)
 {
+    if (c->vec) return c->L->vec_blocks_per_sm(c->kind & kStepWalls);
     return c->staged ? c->L->staged_blocks_per_sm() : c->L->blocks_per_sm(v, c->kind);
 }
 
@@ -142,14 +145,64 @@ static int default_segment(const lbpf_ctx* c, int v)
 {
     if (LBPF_SEGMENT > 0) return LBPF_SEGMENT;
     const double G = (double)blocks_per_sm(c, v) * c->sms;
+    // vector step: below 64 planes a block the waves of equal items do not fill
+    // (64^3: 53.6 us a step in segments, 28.2 balanced), above they do and share
+    // their halo rims better (352^3: 1597 us in segments, 1681 balanced)
+    if (c->vec && (double)column_units(c, v) < 64.0 * G) return 0;
     int L = (int)std::lround(std::sqrt(5.0 * (double)column_units(c, v) / G));
     return L < 8 ? 8 : (L > 256 ? 256 : L);
 }
 
+// Items of equal total work per block: as many whole columns as go round all
+// G blocks evenly, each marched in one piece (neighbouring columns advance
+// together, so their halo rims meet in L2), then the remaining columns, laid
+// end to end, in G runs of equal length (a run that crosses from one column to
+// the next becomes two items), longest first.
+static void balanced_items(const lbpf_ctx* c, int wx, int wy, long long G, std::vector<WorkItem>& items)
+{
+    std::vector<WorkItem> cols;
+    for (int k = 0; k < c->n_domains; ++k) {
+        const DomainDev& d = c->dd[k];
+        const int ny = c->dim == 3 ? d.ny : 1, nz = c->dim == 3 ? d.nz : d.ny;
+        for (int y = 0; y < ny; y += wy)
+            for (int x = 0; x < d.nx; x += wx) cols.push_back(WorkItem{k, x, y, 0, nz, 0});
+    }
+    const size_t whole = c->n_domains == 1 ? cols.size() / (size_t)G * (size_t)G : 0;
+    items.assign(cols.begin(), cols.begin() + whole);
+    long long rest = 0;
+    for (size_t j = whole; j < cols.size(); ++j) rest += cols[j].z1;
+    if (rest > 0) {
+        const long long run = (rest + G - 1) / G < 4 ? 4 : (rest + G - 1) / G;
+        long long left = run;  // of the current run
+        for (size_t j = whole; j < cols.size(); ++j) {
+            const int nz = cols[j].z1;
+            for (int z = 0; z < nz;) {
+                int len = (int)(left < nz - z ? left : nz - z);
+                if (nz - z - len > 0 && nz - z - len < 3) len = nz - z;  // no slivers
+                WorkItem w = cols[j];
+                w.z0 = z;
+                w.z1 = z + len;
+                items.push_back(w);
+                z += len;
+                left -= len;
+                if (left < 3) left = run;
+            }
+        }
+        std::stable_sort(items.begin() + whole, items.end(),
+                         [](const WorkItem& a, const WorkItem& b) { return a.z1 - a.z0 > b.z1 - b.z0; });
+    }
+}
+
+// seg: planes per item, 0 the balanced partition (vector step).
 static int set_schedule(lbpf_ctx* c, int v, int seg)
 {
-    const int wx = tile_x(c->dim, v), wy = tile_y(c->dim, v);
+    const int wx = c->vec ? kVecTX : tile_x(c->dim, v), wy = c->vec ? kVecTY : tile_y(c->dim, v);
+    const long long G = (long long)blocks_per_sm(c, v) * c->sms;
     std::vector<WorkItem> items;
+    if (seg == 0) {
+        balanced_items(c, wx, wy, G, items);
+        seg = (int)(column_units(c, v) / (long long)items.size());
+    } else
     for (int k = 0; k < c->n_domains; ++k) {
         const DomainDev& d = c->dd[k];
         // 2D: the kernel marches the y axis (its z) with one-row tiles
@@ -181,7 +234,6 @@ static int set_schedule(lbpf_ctx* c, int v, int seg)
     CK(cudaMemcpyAsync(c->d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->n_items = (int)items.size();
-    long long G = (long long)blocks_per_sm(c, v) * c->sms;
     c->n_blocks = (int)(G < c->n_items ? G : c->n_items);
     c->tile_v = v;
     c->seg_len = seg;
@@ -209,7 +261,7 @@ static std::string tune_key(const lbpf_ctx* c)
         h *= 1099511628211ULL;
     }
     snprintf(buf, sizeof(buf), "s2-lat%d-prec%d-grad%d-dom%d-%016llx-sm%d-k%d", c->lattice, c->precision, c->grad,
-             c->n_domains, h, c->sms, (c->staged ? 1 : 0) | (c->kind << 1));
+             c->n_domains, h, c->sms, (c->staged ? 1 : 0) | (c->kind << 1) | (c->vec ? 8 : 0));
     return buf;
 }
 
@@ -219,6 +271,18 @@ static std::string tune_cache_path()
     if (p) return p;
     const char* home = getenv("HOME");
     return std::string(home ? home : "/tmp") + "/.cache/lbpf_tune.txt";
+}
+
+// The launches of one time step.
+static cudaError_t issue_step(lbpf_ctx* c, const StepArgs& a)
+{
+    if (c->staged) return c->L->step_staged(a, c->n_blocks, c->stream);
+    if (!c->vec) return c->L->step(c->tile_v, c->kind, a, c->n_blocks, c->stream);
+    for (int k = 0; k < c->n_domains; ++k) {
+        const cudaError_t e = c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream);
+        if (e != cudaSuccess) return e;
+    }
+    return c->L->phi_vec(c->kind & kStepWalls, a, c->n_blocks, c->stream);
 }
 
 // Time a few launches of the current schedule on the live state.  Every trial
@@ -245,9 +309,7 @@ static double time_schedule(lbpf_ctx* c, int launches)
     for (int k = 0; k < launches + 2; ++k) {
         if (cudaMemsetAsync(c->d_counters + c->cur, 0, sizeof(int), c->stream) != cudaSuccess) break;
         cudaEventRecord(e0, c->stream);
-        if ((c->staged ? c->L->step_staged(a, c->n_blocks, c->stream)
-                       : c->L->step(c->tile_v, c->kind, a, c->n_blocks, c->stream)) != cudaSuccess)
-            break;
+        if (issue_step(c, a) != cudaSuccess) break;
         cudaEventRecord(e1, c->stream);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -270,7 +332,7 @@ static int initial_schedule(lbpf_ctx* c)
         char k[200];
         int v, seg;
         while (fscanf(f, "%199s %d %d", k, &v, &seg) == 3)
-            if (key == k && v >= 0 && v < (c->staged || c->kind ? 1 : kNumTileVariants) && seg >= 1) {
+            if (key == k && v >= 0 && v < (c->staged || c->vec || c->kind ? 1 : kNumTileVariants) && seg >= (c->vec ? 0 : 1)) {
                 fclose(f);
                 c->tuned = "cache";
                 return set_schedule(c, v, seg);
@@ -294,9 +356,9 @@ static int autotune(lbpf_ctx* c)
     CK(cudaStreamSynchronize(c->stream));
     double best_t = 1e30, rule_t = 1e30;
     int best_v = 0, best_seg = default_segment(c, 0);
-    for (int v = 0; v < (c->staged || c->kind ? 1 : kNumTileVariants); ++v) {
+    for (int v = 0; v < (c->staged || c->vec || c->kind ? 1 : kNumTileVariants); ++v) {
         const int L0 = default_segment(c, v);
-        const int segs[3] = {L0, L0 / 2 > 8 ? L0 / 2 : 8, L0 * 2};
+        const int segs[3] = {L0, L0 / 2 > 8 ? L0 / 2 : 8, L0 ? L0 * 2 : 32};
         for (int j = 0; j < 3; ++j) {
             int rc = set_schedule(c, v, segs[j]);
             if (rc) return rc;
@@ -323,6 +385,21 @@ static int autotune(lbpf_ctx* c)
         fclose(f);
     }
     return set_schedule(c, best_v, best_seg);
+}
+
+// Whether every domain takes the vector step: 3D in single precision, one
+// crystal, no advection, rows of whole 4-site vectors, and no row segment of
+// a single vector (its two ends need different lanes).
+static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_domains)
+{
+    if (!L->heat_vec) return false;
+    for (int k = 0; k < n_domains; ++k) {
+        const lbpf_domain& d = domains[k];
+        if (d.nx % 4 || d.nx < 8 || d.nx % kVecTX == 4 || (long long)d.nx * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 || d.adv[0] != 0.0 || d.adv[1] != 0.0 ||
+            d.adv[2] != 0.0)
+            return false;
+    }
+    return true;
 }
 
 extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattice, int grad, int precision,
@@ -399,6 +476,9 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
     }
     const double e2u = (dim == 2) ? 1.0 / 3.0 : 1.0 / 4.0;
 
+    const char* kenv = getenv("LBPF_KERNEL");
+    c->vec = vec_applies(L, domains, n_domains) && !(kenv && *kenv);
+
     int rc = LBPF_OK;
     long long max_n = 0;
     c->dd.resize(n_domains);
@@ -441,6 +521,7 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
             if (rc == LBPF_OK && h.use_index) rc = dev_alloc(c, reinterpret_cast<void**>(&h.I[b]), (size_t)h.n);
             if (rc == LBPF_OK && h.advect) rc = dev_alloc(c, &h.U[b], (size_t)h.n * c->rsize);
         }
+        if (rc == LBPF_OK && c->vec) rc = dev_alloc(c, &h.u_work, (size_t)h.n * c->rsize);
         // zero state so that an unseeded domain holds finite values
         for (int b = 0; b < 2 && rc == LBPF_OK; ++b) {
             if (cudaMemsetAsync(h.g[b], 0, (size_t)c->Sg * h.n * c->ssize, c->stream) != cudaSuccess ||
@@ -456,7 +537,6 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
         // the staged kernel (opt-in: it measured slower than the generic one,
         // see staged_kernel.cuh) needs 16-byte aligned row copies (nx a
         // multiple of 8), rows wider than the staged 48-site window, one crystal
-        const char* kenv = getenv("LBPF_KERNEL");
         c->staged = L->step_staged != nullptr && kenv && strcmp(kenv, "staged") == 0;
         for (const DomainDev& h : c->dd)
             if (h.nx % 8 != 0 || h.nx < 64 || h.use_index || h.bc || h.advect) c->staged = false;
@@ -604,10 +684,7 @@ static int launch_step(lbpf_ctx* c)
     a.acur = c->acur;
     a.collide = c->lagged;
     a.grad = c->grad;
-    if (c->staged)
-        CK(c->L->step_staged(a, c->n_blocks, c->stream));
-    else
-        CK(c->L->step(c->tile_v, c->kind, a, c->n_blocks, c->stream));
+    CK(issue_step(c, a));
     c->cur ^= 1;
     c->acur ^= 1;
     if (c->lagged) c->fcur ^= 1;

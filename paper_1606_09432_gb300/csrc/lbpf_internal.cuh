@@ -220,6 +220,7 @@ struct DomainDev {
     int advect;
     double adv[3];
     void* U[2];
+    void* u_work;       // u^n between the two launches of the vector step (vec_kernel.cuh)
 };
 
 // One thread block's work: a column of TX x TY sites over planes [z0, z1).
@@ -250,6 +251,8 @@ constexpr int TX = 32;
 constexpr int kNumTileVariants = 2;
 constexpr int kTileRows[kNumTileVariants] = {8, 16};
 constexpr int kStripX[kNumTileVariants] = {128, 256};
+// Tile of the vector step's phase-field launch (vec_kernel.cuh).
+constexpr int kVecTX = 64, kVecTY = 12;
 constexpr int tile_x(int dim, int v) { return dim == 3 ? TX : kStripX[v]; }
 constexpr int tile_y(int dim, int v) { return dim == 3 ? kTileRows[v] : 1; }
 
@@ -434,6 +437,12 @@ struct Launchers {
     // nullptr where it is not built (2D, full storage, D3Q27).
     cudaError_t (*step_staged)(const StepArgs& a, int n_blocks, cudaStream_t s);
     int (*staged_blocks_per_sm)();
+    // The vector step (vec_kernel.cuh): the heat launch of one domain (its host
+    // copy h for the sizes, d on the device), then the phase-field launch over
+    // the items; nullptr where it is not built (2D, FP64).
+    cudaError_t (*heat_vec)(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s);
+    cudaError_t (*phi_vec)(int walls, const StepArgs& a, int n_blocks, cudaStream_t s);
+    int (*vec_blocks_per_sm)(int walls);
     // Heat step alone, lagged -> synced state of one domain (f^{n-1}, aux^{n-1},
     // phi^n -> f^n [+ aux^n]).
     cudaError_t (*heat_sync)(const DomainDev* d, int cur, int fcur, int acur, cudaStream_t s);

@@ -1,0 +1,97 @@
+"""The vector step (two launches, four sites a thread; 3D, 16-bit deviations)
+against the one-launch step kernel (LBPF_KERNEL=generic).
+
+Both evaluate the same operations in the same order, so the fields and the
+populations must agree bit for bit.  Sizes sit at the edges of the vector
+form's tile (64 x 12 sites, row segments of at least two vectors): the
+smallest rows, one and several segments with short last ones, rows of blocks
+that end inside the domain, and columns of two planes.  Reads between the
+steps put the heat state through both of its forms (synchronised, lagged)."""
+import numpy as np
+import pytest
+
+from helpers import gpu_run
+from paper_1606_09432_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_1606_09432_gb300 import build as B
+    from paper_1606_09432_gb300 import lbpf
+    B.build()
+    lbpf.load()
+    return lbpf
+
+
+SHAPES = [(2, 2, 8), (3, 13, 12), (5, 12, 64), (4, 25, 72), (7, 11, 128), (9, 37, 140), (40, 24, 200)]
+FORM = dict(kind=3, eps=0.02, gamma=-0.02)
+
+
+def smooth_fields(shape, seed):
+    """A wavy interface with a little noise."""
+    rng = np.random.default_rng(seed)
+    waves = [np.cos(2 * np.pi * (np.arange(n) / n + rng.random())) for n in shape]
+    w = waves[0][:, None, None] + waves[1][None, :, None] + waves[2][None, None, :]
+    phi = np.tanh(w) + 0.01 * rng.standard_normal(shape)
+    u = -0.4 + 0.05 * w + 0.01 * rng.standard_normal(shape)
+    return phi.astype(np.float32), u.astype(np.float32)
+
+
+def both(L, monkeypatch, make):
+    out = []
+    for kernel in ("", "generic"):
+        monkeypatch.setenv("LBPF_KERNEL", kernel)
+        out.append(make())
+    return out
+
+
+@pytest.mark.parametrize("precision", [2, 3, 4])
+@pytest.mark.parametrize("lattice", [1, 2, 3])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_vector_step_matches_one_launch_step(L, monkeypatch, shape, lattice, precision):
+    prm = dict(W.C3D_PARAMS, delta=0.4)
+    phi, u = smooth_fields(shape, sum(shape) + lattice)
+    a, b = both(L, monkeypatch, lambda: gpu_run(L, lattice, shape, prm, [FORM], fields=(phi, u), precision=precision))
+    for steps in (1, 1, 2, 21):
+        for s in (a, b):
+            s.step(steps)
+        if steps != 1:
+            for x, y in zip(a.fields(), b.fields()):
+                assert np.array_equal(x, y)
+    for which in (0, 1):
+        assert np.array_equal(a.populations(which), b.populations(which))
+
+
+@pytest.mark.parametrize("bc", [1, 2, 4, 7])
+@pytest.mark.parametrize("lattice,grad", [(1, 0), (2, 0), (3, 0), (1, 1)])
+def test_vector_step_walls_and_gradients(L, monkeypatch, bc, lattice, grad):
+    shape = (9, 14, 76)
+    prm = dict(W.C3D_PARAMS, delta=0.4)
+    phi, u = smooth_fields(shape, bc + 10 * lattice + grad)
+    a, b = both(L, monkeypatch, lambda: gpu_run(L, lattice, shape, prm, [FORM], fields=(phi, u), precision=2, bc=bc,
+                                                grad=grad))
+    for s in (a, b):
+        s.step(17)
+    for x, y in zip(a.fields(), b.fields()):
+        assert np.array_equal(x, y)
+
+
+def test_vector_step_of_several_domains_and_segments(L, monkeypatch):
+    """Two domains in one context, and every item split: same bits as one launch."""
+    def make():
+        doms = [L.make_domain(nx, ny, nz, lam=10.0, delta=0.4, crystals=[L.make_crystal(**FORM)],
+                              **{k: v for k, v in W.C3D_PARAMS.items() if k != "lam"})
+                for nx, ny, nz in ((72, 30, 11), (16, 12, 40))]
+        s = L.Solver(doms, L.LBPF_D3Q15_D3Q7, L.LBPF_GRAD_DD, L.LBPF_FP32_FP16DEV)
+        s.seed([(30.0, 12.0, 5.0, 5.0, 0)], domain=0).seed([(8.0, 6.0, 20.0, 4.0, 0)], domain=1)
+        return s
+    a, b = both(L, monkeypatch, make)
+    a.step(20)
+    L.lbpf_set_schedule(a.ctx, 8, 3)
+    a.step(20)
+    b.step(40)
+    for k in (0, 1):
+        for x, y in zip(a.fields(k), b.fields(k)):
+            assert np.array_equal(x, y)
