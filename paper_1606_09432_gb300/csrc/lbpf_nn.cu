@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "lbpf_nn.cuh"
 
 namespace lbpf_nn {
@@ -71,6 +73,14 @@ __device__ __forceinline__ void umma_commit(uint64_t* mbar)
                  : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ unsigned long long global_ns()
 {
     unsigned long long t;
@@ -78,21 +88,25 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-// Wait for the completion of phase `parity` of an mbarrier, at most ~2 s;
+// Wait for the completion of phase `parity` of an mbarrier, at most ~2 s (each
+// try suspends for at most 0.1 ms);
 // false on expiry.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* mbar, uint32_t parity)
 {
     const uint32_t a = smem_u32(mbar);
-    const unsigned long long t0 = global_ns();
-    for (;;) {
+    unsigned long long t0 = 0;  // the clock is read only once the first waits fail
+    for (int n = 0;; ++n) {
         uint32_t ok;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
             : "=r"(ok)
-            : "r"(a), "r"(parity), "r"(1000000u)
+            : "r"(a), "r"(parity), "r"(100000u)
             : "memory");
         if (ok) return true;
-        if (global_ns() - t0 > 2000000000ull) return false;
+        if (n < 4) continue;
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 2000000000ull) return false;
     }
 }
 
@@ -232,68 +246,194 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols));
 }
 
-// Halo variant of the same convolution for images whose H is a multiple of
-// 16 and W of 8 (with `resident`, every tap's weights are copied once beside
-// the halo and all MMAs follow one barrier): a block owns a 16 x 8 tile (M = 128: tile row = 8-row group,
-// pixel in the row = row of the core matrix), loads the 18 x 10 halo of all
-// cin channels once (FP32 -> BF16, layout [k8][halo pixel][8]), and every tap
-// is a descriptor over that halo: start at the tap's offset, SBO = one halo
-// row (10 pixels x 16 bytes), LBO = one 8-channel slice (180 x 16 bytes).
-// Only the weights stream through the two stage buffers (cp.async).
-constexpr int kHaloY = 18, kHaloX = 10, kHaloP = kHaloY * kHaloX;
+// Halo form of the same convolution for images whose H is a multiple of 16
+// and W of 8.  A tile is 16 x 8 pixels (M = 128: tile row = 8-row group, pixel
+// in the row = row of the core matrix); its 18 x 10 halo of all cin channels
+// is converted to BF16 once (layout [8-channel slice][halo pixel][8]), and
+// every tap is a matrix descriptor over it: start at the tap's offset, SBO =
+// one halo row (10 pixels x 16 bytes), LBO = one slice.  A slice is 181 pixels
+// long (180 used): at 181 x 16 bytes the eight slices a quarter-warp stores
+// fall into different banks (at 180, into two: 4-way conflicts).
+//
+// A block is persistent over tiles and its warps take different parts:
+// warps 0-3 the epilogue (bias, ReLU, coalesced stores), 4-11 load and convert
+// halos (two buffers where they fit), warp 12 issues the MMAs (two
+// accumulators where they fit), 13-20 stream the weights through a ring where
+// they don't all stay resident, a stage (KC channels of one tap) per warp.  Every hand-over is an mbarrier with a bounded
+// wait; on expiry a role sets the error word and leaves, the others follow.
+// MMAs are issued tap by tap, 16 channels at a time, for every tile: the sum's
+// order is that of the gather kernel.
+constexpr int kHaloY = 18, kHaloX = 10, kHaloP = kHaloY * kHaloX, kHaloS = kHaloP + 1;
+constexpr int kEpiT = 128, kLoadT = 256, kWtT = 256;
+constexpr int kMaxWStages = kWtT / 32;  // a warp a slot
+constexpr int kOutPitch = 36;  // floats a pixel of the store staging (32 + 4)
 
-__global__ void __launch_bounds__(kConvM) conv3x3_halo_tc_kernel(const float* __restrict__ x,
-                                                                 const __nv_bfloat16* __restrict__ w,
-                                                                 const float* __restrict__ bias,
-                                                                 float* __restrict__ y, int H, int W, int cin,
-                                                                 int cout_all, int cout, int KC, int relu,
-                                                                 uint32_t tmem_cols, int resident)
+// Channels of the convolution's input: all cin from a, or (b set) the first ca
+// from a at half the resolution (nearest 2x upsampling), the others from b.
+struct ConvSrc {
+    const float* a;
+    const float* b;
+    int ca, cb;
+};
+
+__device__ __forceinline__ const float* src_at(const ConvSrc& s, int img, int y, int x, int H, int W, int c)
 {
-    const int co0 = blockIdx.y * cout;  // output channel tile
+    if (!s.b) return s.a + (((size_t)img * H + y) * W + x) * s.ca + c;
+    if (c < s.ca) return s.a + (((size_t)img * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1)) * s.ca + c;
+    return s.b + (((size_t)img * H + y) * W + x) * s.cb + (c - s.ca);
+}
+
+__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* b)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+
+// Offsets (floats) of the halo pixels from the tile's first pixel in the full
+// resolution source and in the half resolution one, for tiles whose halo does
+// not wrap: filled once a block, so that a piece's address is one table entry.
+__device__ __forceinline__ void fill_halo_table(int* tab, const ConvSrc& s, int W, int t, int nt)
+{
+    for (int hp = t; hp < kHaloP; hp += nt) {
+        const int hy = hp / kHaloX - 1, hx = hp % kHaloX - 1;
+        tab[hp] = (hy * W + hx) * (s.b ? s.cb : s.ca);
+        tab[kHaloP + hp] = s.b ? ((hy >> 1) * (W >> 1) + (hx >> 1)) * s.ca : 0;
+    }
+}
+
+// Halo pixels [r0, r0 + rows) x 10 of tile (img, ty0, tx0), channels c0 ..
+// c0 + 8 k8n, as BF16 into dst ([slice][kHaloS pixels][8]), by threads t of nt:
+// a thread keeps one 8-channel slice and takes every dq-th pixel, six 32-byte
+// pieces in flight.  tab: fill_halo_table of the source.
+__device__ __forceinline__ void load_halo(const ConvSrc& src, const int* tab, unsigned char* dst, int img, int ty0,
+                                          int tx0, int H, int W, int c0, int k8n, int r0, int rows, int t, int nt)
+{
+    constexpr int B = 6;
+    const int dq = nt / k8n;
+    if (t >= dq * k8n) return;
+    const int p0 = t / k8n, k8 = t - p0 * k8n, c = c0 + 8 * k8, end = rows * kHaloX;
+    const bool inside = ty0 > 0 && tx0 > 0 && ty0 + 16 < H && tx0 + 8 < W;
+    const bool half = src.b && c < src.ca;
+    const float* base;
+    if (!src.b)
+        base = src.a + (((size_t)img * H + ty0) * W + tx0) * src.ca + c;
+    else if (half)
+        base = src.a + (((size_t)img * (H >> 1) + (ty0 >> 1)) * (W >> 1) + (tx0 >> 1)) * src.ca + c;
+    else
+        base = src.b + (((size_t)img * H + ty0) * W + tx0) * src.cb + (c - src.ca);
+    const int* tb = tab + (half ? kHaloP : 0) + r0 * kHaloX;
+    unsigned char* o = dst + ((size_t)k8 * kHaloS + p0) * 16;
+    for (int hp = p0; hp < end; hp += B * dq, o += B * dq * 16) {
+        float4 f[B][2];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const int p = hp + j * dq;
+            if (p < end) {
+                const float* g;
+                if (inside) {
+                    g = base + tb[p];
+                } else {
+                    const int hy = p / kHaloX, hx = p - hy * kHaloX;
+                    int gy = ty0 + r0 + hy - 1, gx = tx0 + hx - 1;
+                    gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
+                    gx = gx < 0 ? gx + W : (gx >= W ? gx - W : gx);
+                    g = src_at(src, img, gy, gx, H, W, c);
+                }
+                f[j][0] = __ldg(reinterpret_cast<const float4*>(g));
+                f[j][1] = __ldg(reinterpret_cast<const float4*>(g) + 1);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (hp + j * dq < end)
+                *reinterpret_cast<uint4*>(o + j * dq * 16) =
+                    make_uint4(pack_bf16(f[j][0].x, f[j][0].y), pack_bf16(f[j][0].z, f[j][0].w),
+                               pack_bf16(f[j][1].x, f[j][1].y), pack_bf16(f[j][1].z, f[j][1].w));
+    }
+}
+
+struct HaloArgs {
+    ConvSrc src;
+    const __nv_bfloat16* w;
+    const float* bias;
+    float* y;
+    int H, W, n_tiles, cin, cout_all, cout, KC, relu;
+    int nbuf, nacc, wst;  // halo buffers, accumulators, weight ring stages (0: resident)
+    uint32_t tmem_cols;
+};
+
+// MMAs of one K block (16 k16n channels of one tap), K16 = k16n where it is known
+// at compile time.
+template <int K16>
+__device__ __forceinline__ void umma_block(uint32_t d, uint64_t ad, uint64_t bd, uint32_t bstep, uint32_t idesc, int k16n,
+                                           uint32_t more)
+{
+    if constexpr (K16 > 0) {
+#pragma unroll
+        for (int k = 0; k < K16; ++k) umma_bf16(d, ad + k * (2 * kHaloS), bd + k * bstep, idesc, k > 0 ? 1u : more);
+    } else {
+        for (int k = 0; k < k16n; ++k)
+            umma_bf16(d, ad + k * (2 * kHaloS), bd + (uint64_t)k * bstep, idesc, k > 0 ? 1u : more);
+    }
+}
+
+// STREAM: the weights go through the ring.  K16: 16-channel steps of a K block
+// (KC / 16; resident weights: cin / 16), 0 = any.  One thread issues a tile's
+// MMAs in straight-line code: with a loop over taps and a warp-wide branch in
+// each, an MMA took 150-300 cycles to issue, several times its execution.
+template <int K16, bool STREAM>
+__global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STREAM ? 1 : 2)
+    conv3x3_halo_tc_kernel(const HaloArgs q)
+{
+    constexpr int kHaloThreads = kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0);
+    const int co0 = blockIdx.y * q.cout;  // output channel tile
+    const int cin = q.cin, cout = q.cout, k8n = cin / 8;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[2];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int tiles_x = W / 8, tiles = tiles_x * (H / 16);
-    const int img = blockIdx.x / tiles, t = blockIdx.x - img * tiles;
-    const int ty0 = (t / tiles_x) * 16, tx0 = (t % tiles_x) * 8;
-    const size_t halo_bytes = (size_t)kHaloP * cin * 2, b_bytes = (size_t)cout * KC * 2;
+    __shared__ __align__(8) uint64_t s_hfull[4], s_hempty[4], s_afull[2], s_aempty[2], s_wfull[kMaxWStages],
+        s_wempty[kMaxWStages];
+    __shared__ int s_tab[2 * kHaloP];
+    __shared__ __align__(16) float s_bias[256];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t halo_b = (size_t)kHaloS * 16 * k8n;
+    const size_t wst_b = (size_t)(cout + 1) * q.KC * 2;  // a slice is cout + 1 rows: conflict-free copies
     unsigned char* sH = smem_raw;
-    auto sB = [&](int b) { return smem_raw + halo_bytes + b * b_bytes; };
+    unsigned char* sW = smem_raw + q.nbuf * halo_b;
+    float* sO = reinterpret_cast<float*>(sW + (STREAM ? q.wst * wst_b : (size_t)9 * cin * (cout + 1) * 2));
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(tmem_cols));
+                     "r"(q.tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[1])));
+        for (int k = 0; k < 4; ++k) {
+            mbar_init(&s_hfull[k], kLoadT / q.nbuf);
+            mbar_init(&s_hempty[k], 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(&s_afull[k], 1);
+            mbar_init(&s_aempty[k], kEpiT);
+        }
+        for (int k = 0; k < kMaxWStages; ++k) {
+            mbar_init(&s_wfull[k], 32);
+            mbar_init(&s_wempty[k], 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    const int k8n = cin / 8;
-    if (resident) {  // every tap's weights, [tap][k8][co][8], copied beside the halo
-        for (int e = tid; e < 9 * k8n * cout; e += kConvM) {
+    fill_halo_table(s_tab, q.src, q.W, tid, kHaloThreads);
+    for (int c = tid; c < cout; c += kHaloThreads) s_bias[c] = q.bias ? q.bias[co0 + c] : 0.f;
+    if (!STREAM) {  // every tap's weights, [tap][slice][co][8], once per block
+        for (int e = tid; e < 9 * k8n * cout; e += kHaloThreads) {
             const int co = e % cout, r = e / cout, k8 = r % k8n, tap = r / k8n;
-            const __nv_bfloat16* g = w + ((size_t)tap * cout_all + co0 + co) * cin + 8 * k8;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sB(0) + (size_t)e * 16)), "l"(g));
+            const __nv_bfloat16* g = q.w + ((size_t)tap * q.cout_all + co0 + co) * cin + 8 * k8;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sW + ((size_t)r * (cout + 1) + co) * 16)),
+                         "l"(g));
         }
         asm volatile("cp.async.commit_group;");
-    }
-    // halo: (pixel, 8-channel slice) pieces, FP32 -> BF16
-    const float* ximg = x + (size_t)img * H * W * cin;
-    for (int e = tid; e < kHaloP * k8n; e += kConvM) {
-        const int hp = e / k8n, k8 = e - hp * k8n;
-        const int hy = hp / kHaloX, hx = hp - hy * kHaloX;
-        int gy = ty0 + hy - 1, gx = tx0 + hx - 1;
-        gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
-        gx = gx < 0 ? gx + W : (gx >= W ? gx - W : gx);
-        const float4* src = reinterpret_cast<const float4*>(ximg + ((size_t)gy * W + gx) * cin + 8 * k8);
-        const float4 f0 = __ldg(src), f1 = __ldg(src + 1);
-        *reinterpret_cast<uint4*>(sH + ((size_t)k8 * kHaloP + hp) * 16) =
-            make_uint4(pack_bf16(f0.x, f0.y), pack_bf16(f0.z, f0.w), pack_bf16(f1.x, f1.y), pack_bf16(f1.z, f1.w));
-    }
-    if (resident) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -301,93 +441,180 @@ __global__ void __launch_bounds__(kConvM) conv3x3_halo_tc_kernel(const float* __
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = s_tmem;
+    const int tiles_x = q.W / 8, tiles_img = tiles_x * (q.H / 16);
+    const int nkb = cin / q.KC;
+    auto split = [&](int t, int& img, int& ty0, int& tx0) {
+        img = t / tiles_img;
+        const int r = t - img * tiles_img, by = r / tiles_x;
+        ty0 = by * 16;
+        tx0 = (r - by * tiles_x) * 8;
+    };
 
-    const int nkb = cin / KC, S = 9 * nkb;
-    const uint32_t idesc = umma_idesc_bf16(kConvM, cout);
-    const uint32_t h0 = smem_u32(sH);
-    bool ok = true;
-    int issued = 0;
-    if (resident) {  // all MMAs after the one barrier, one commit
-        if (tid == 0) {
-            const uint32_t b0 = smem_u32(sB(0));
-            for (int tap = 0; tap < 9; ++tap) {
-                const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                const uint32_t tap_off = (uint32_t)(((1 + dy) * kHaloX + (1 + dx)) * 16);
-                for (int k16 = 0; k16 < cin / 16; ++k16) {
-                    const uint64_t ad = umma_desc(h0 + (uint32_t)(2 * k16) * kHaloP * 16 + tap_off, kHaloP * 16,
-                                                  kHaloX * 16);
-                    const uint64_t bd = umma_desc(b0 + (uint32_t)((tap * k8n + 2 * k16) * cout * 16), cout * 16, 128);
-                    umma_bf16(tmem, ad, bd, idesc, (tap > 0 || k16 > 0) ? 1u : 0u);
+    if (warp < 4) {  // epilogue: TMEM lanes 32 warp .. are the warp's 32 pixels (4 tile rows)
+        float* st = sO + warp * 32 * kOutPitch;
+        int k = 0;
+        for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x, ++k) {
+            const int acc = k % q.nacc;
+            if (!mbar_wait_bounded(&s_afull[acc], (k / q.nacc) & 1)) {
+                atomicOr(&g_conv_error, 32);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            int img, ty0, tx0;
+            split(t, img, ty0, tx0);
+            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * cout);
+            float* yt = q.y + (((size_t)img * q.H + ty0 + 4 * warp) * q.W + tx0) * q.cout_all;
+            for (int c0 = 0; c0 < cout; c0 += 32) {
+                const int cw = cout - c0 < 32 ? cout - c0 : 32;  // 16 or 32 channels
+                for (int c = 0; c < cw; c += 16) {
+                    uint32_t r[16];
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                        "[%16];"
+                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                          "=r"(r[15])
+                        : "r"(ta + (uint32_t)(c0 + c)));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const float4 bq = *reinterpret_cast<const float4*>(s_bias + c0 + c + j);
+                        float4 v = make_float4(__uint_as_float(r[j]) + bq.x, __uint_as_float(r[j + 1]) + bq.y,
+                                               __uint_as_float(r[j + 2]) + bq.z, __uint_as_float(r[j + 3]) + bq.w);
+                        if (q.relu)
+                            v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+                        *reinterpret_cast<float4*>(st + lane * kOutPitch + c + j) = v;
+                    }
+                }
+                if (c0 + 32 >= cout) {  // the accumulator is read: the next tile may overwrite it
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    mbar_arrive(&s_aempty[acc]);
+                }
+                __syncwarp();
+                // the warp's 32 pixels, four tile rows, cw channels each: whole
+                // 64- or 128-byte pieces per pixel
+                const int sh = cw == 32 ? 3 : 2, ppi = 32 >> sh;  // pixels a pass
+                float* og = yt + co0 + c0 + 4 * (lane & ((1 << sh) - 1));
+                const float* sg = st + 4 * (lane & ((1 << sh) - 1));
+#pragma unroll 4
+                for (int px = lane >> sh; px < 32; px += ppi)
+                    *reinterpret_cast<float4*>(og + (size_t)((px >> 3) * q.W + (px & 7)) * q.cout_all) =
+                        *reinterpret_cast<const float4*>(sg + px * kOutPitch);
+                __syncwarp();
+            }
+        }
+    } else if (warp < 12) {
+        // halo loaders: one group of warps per buffer, each on its own tiles, so
+        // that the loads of nbuf tiles are in flight
+        const int gt = kLoadT / q.nbuf, buf = (tid - kEpiT) / gt, g = (tid - kEpiT) - buf * gt;
+        int use = 0;
+        for (long long t = blockIdx.x + (long long)buf * gridDim.x; t < q.n_tiles; t += (long long)q.nbuf * gridDim.x, ++use) {
+            if (use > 0 && !mbar_wait_bounded(&s_hempty[buf], (use - 1) & 1)) {
+                atomicOr(&g_conv_error, 16);
+                break;
+            }
+            int img, ty0, tx0;
+            split((int)t, img, ty0, tx0);
+            load_halo(q.src, s_tab, sH + buf * halo_b, img, ty0, tx0, q.H, q.W, 0, k8n, 0, kHaloY, g, gt);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&s_hfull[buf]);
+        }
+    } else if (warp == 12) {
+        if (elect_one()) {
+            const uint32_t idesc = umma_idesc_bf16(kConvM, cout), bstep = 2 * (cout + 1);
+            const int k16n = q.KC / 16;
+            const uint64_t w0 = umma_desc(smem_u32(sW), (cout + 1) * 16, 128);
+            int buf = 0, acc = 0, st = 0;  // halo buffer, accumulator and weight slot, with their phases
+            uint32_t hpar = 0, apar = 1, wpar = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < q.n_tiles && ok; t += gridDim.x) {
+                if (!mbar_wait_bounded(&s_aempty[acc], apar) || !mbar_wait_bounded(&s_hfull[buf], hpar)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                // descriptors advance by adding to their address field (16-byte units)
+                const uint32_t d = tmem + (uint32_t)(acc * cout);
+                const uint64_t a0 = umma_desc(smem_u32(sH + buf * halo_b), kHaloS * 16, kHaloX * 16);
+                if constexpr (!STREAM) {
+                    const int n16 = K16 ? K16 : cin / 16;
+                    uint64_t bd = w0;
+#pragma unroll
+                    for (int tap = 0; tap < 9; ++tap) {
+                        umma_block<K16>(d, a0 + (tap / 3) * kHaloX + tap % 3, bd, bstep, idesc, n16, tap > 0 ? 1u : 0u);
+                        bd += (uint64_t)n16 * bstep;
+                    }
+                } else {
+                    for (int tap = 0; tap < 9 && ok; ++tap) {
+                        uint64_t ad = a0 + (uint64_t)((tap / 3) * kHaloX + tap % 3);
+                        for (int kb = 0; kb < nkb; ++kb) {
+                            if (!mbar_wait_bounded(&s_wfull[st], wpar)) {
+                                ok = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;");
+                            umma_block<K16>(d, ad, w0 + (uint64_t)st * (wst_b >> 4), bstep, idesc, k16n,
+                                            (tap | kb) ? 1u : 0u);
+                            umma_commit(&s_wempty[st]);
+                            ad += (uint64_t)k16n * (2 * kHaloS);
+                            if (++st == q.wst) {
+                                st = 0;
+                                wpar ^= 1;
+                            }
+                        }
+                    }
+                }
+                umma_commit(&s_hempty[buf]);
+                umma_commit(&s_afull[acc]);
+                if (++buf == q.nbuf) {
+                    buf = 0;
+                    hpar ^= 1;
+                }
+                if (++acc == q.nacc) {
+                    acc = 0;
+                    apar ^= 1;
                 }
             }
-            umma_commit(&s_mbar[0]);
+            if (!ok) atomicOr(&g_conv_error, 64);
         }
-        issued = 1;
-    }
-    for (int s = 0; s < S && ok && !resident; ++s) {
-        const int buf = s & 1, tap = s / nkb, c0 = (s - tap * nkb) * KC;
-        if (s >= 2 && !mbar_wait_bounded(&s_mbar[buf], ((s - 2) >> 1) & 1)) {
-            atomicOr(&g_conv_error, 16);
-            ok = false;
-            break;
-        }
-        for (int e = tid; e < cout * (KC / 8); e += kConvM) {
-            const int co = e % cout, k8 = e / cout;
-            const __nv_bfloat16* g = w + ((size_t)tap * cout_all + co0 + co) * cin + c0 + 8 * k8;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             smem_u32(sB(buf) + (size_t)k8 * cout * 16 + co * 16)),
-                         "l"(g));
-        }
-        asm volatile("cp.async.commit_group;");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-            const uint32_t tap_off = (uint32_t)(((1 + dy) * kHaloX + (1 + dx)) * 16);
-            const uint32_t b0 = smem_u32(sB(buf));
-            for (int k16 = 0; k16 < KC / 16; ++k16) {
-                const int k8 = c0 / 8 + 2 * k16;
-                const uint64_t ad = umma_desc(h0 + (uint32_t)k8 * kHaloP * 16 + tap_off, kHaloP * 16, kHaloX * 16);
-                const uint64_t bd = umma_desc(b0 + k16 * 2 * cout * 16, cout * 16, 128);
-                umma_bf16(tmem, ad, bd, idesc, (s > 0 || k16 > 0) ? 1u : 0u);
+        __syncwarp();
+    } else if (STREAM && warp - 13 < q.wst) {
+        // weight stream: warp j owns ring slot j and fills the stages j, j + wst,
+        // ... (one owner a slot: a slot's phases are waited for in order)
+        const int st = warp - 13;
+        int my_tiles = 0;
+        for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x) ++my_tiles;
+        const int S = 9 * nkb, total = my_tiles * S, k8s = q.KC / 8;
+        // the lanes' pieces: k8s slices of a row, rpp rows a pass (k8s = 2, 4, 8;
+        // 6 leaves two lanes idle)
+        const int rpp = 32 / k8s, k8 = lane % k8s, r0 = lane / k8s;
+        int use = 0;
+        for (int ws = st; ws < total; ws += q.wst, ++use) {
+            if (use > 0 && !mbar_wait_bounded(&s_wempty[st], (use - 1) & 1)) {
+                if (lane == 0) atomicOr(&g_conv_error, 128);
+                break;
             }
-            umma_commit(&s_mbar[buf]);
-        }
-        issued = s + 1;
-    }
-    bool done = false;
-    if (issued > 0) {
-        const int last = issued - 1;
-        done = mbar_wait_bounded(&s_mbar[last & 1], (last >> 1) & 1);
-        if (!done) atomicOr(&g_conv_error, 32);
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok && done) {
-        const int m = tid, py = m >> 3, px = m & 7;
-        float* out = y + (((size_t)img * H + ty0 + py) * W + tx0 + px) * cout_all + co0;
-        for (int c = 0; c < cout; c += 8) {
-            uint32_t r[8];
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7])
-                         : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                v[j] = __uint_as_float(r[j]) + (bias ? bias[co0 + c + j] : 0.f);
-                if (relu) v[j] = fmaxf(v[j], 0.f);
+            const int s = ws % S, tap = s / nkb, c0 = (s - tap * nkb) * q.KC;
+            const __nv_bfloat16* g = q.w + ((size_t)tap * q.cout_all + co0 + r0) * cin + c0 + 8 * k8;
+            uint32_t o = smem_u32(sW + st * wst_b) + (k8 * (cout + 1) + r0) * 16;
+            if (r0 < rpp) {
+#pragma unroll 4
+                for (int co = r0; co < cout; co += rpp) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o), "l"(g));
+                    o += rpp * 16;
+                    g += (size_t)rpp * cin;
+                }
             }
-            reinterpret_cast<float4*>(out + c)[0] = make_float4(v[0], v[1], v[2], v[3]);
-            reinterpret_cast<float4*>(out + c)[1] = make_float4(v[4], v[5], v[6], v[7]);
+            asm volatile("cp.async.commit_group;");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&s_wfull[st]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(q.tmem_cols));
 }
 
 // Input channels a stage: all of them up to 64, else the largest of 64, 48,
@@ -400,52 +627,127 @@ static int conv_kc(int cin)
     return 16;
 }
 
+// Largest dynamic shared memory a block may opt into, less the kernels' own
+// static part.
+constexpr size_t kSmemMax = 224 * 1024;
+
+// Raises a kernel's dynamic shared memory limit, once per device (done: the
+// kernel's own flags).
+constexpr int kMaxDevices = 64;
+template <class K>
+static cudaError_t opt_in(K kernel, std::atomic<bool> (&done)[kMaxDevices])
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    if (known && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_relaxed);
+    return e;
+}
+static std::atomic<bool> g_gather_ready[kMaxDevices], g_wgrad_ready[kMaxDevices],
+    g_wgrad9_ready[kMaxDevices], g_wgrad3_ready[kMaxDevices];
+
+template <int K16, bool STREAM>
+static cudaError_t launch_halo(const HaloArgs& q, dim3 grid, size_t smem, cudaStream_t s)
+{
+    static std::atomic<bool> ready[kMaxDevices];
+    const cudaError_t e = opt_in(conv3x3_halo_tc_kernel<K16, STREAM>, ready);
+    if (e != cudaSuccess) return e;
+    conv3x3_halo_tc_kernel<K16, STREAM><<<grid, kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), smem, s>>>(q);
+    return cudaGetLastError();
+}
+
+// Plan of the halo kernel: false where it does not apply.
+static bool halo_plan(HaloArgs& q, size_t& smem, int& per_sm)
+{
+    if (q.H % 16 || q.W % 8) return false;
+    const size_t halo = (size_t)kHaloS * 16 * (q.cin / 8), out = (size_t)4 * 32 * kOutPitch * 4;
+    const size_t all_w = (size_t)9 * q.cin * (q.cout + 1) * 2, st = (size_t)(q.cout + 1) * q.KC * 2;
+    q.nacc = q.cout <= 128 ? 2 : 1;
+    // four halo buffers where two blocks an SM hold them, else two
+    q.nbuf = 4 * halo + all_w + out <= 110 * 1024 ? 4 : 2;
+    q.wst = 0;
+    smem = q.nbuf * halo + all_w + out;
+    if (smem > kSmemMax) {
+        // the weights stream; a second halo buffer only beside four stages
+        q.nbuf = 2 * halo + 4 * st + out <= kSmemMax ? 2 : 1;
+        if (q.nbuf * halo + 3 * st + out > kSmemMax) return false;
+        const size_t n = (kSmemMax - q.nbuf * halo - out) / st;
+        q.wst = (int)(n < kMaxWStages ? n : kMaxWStages);
+        smem = q.nbuf * halo + q.wst * st + out;
+    }
+    q.tmem_cols = 32;
+    while ((int)q.tmem_cols < q.nacc * q.cout) q.tmem_cols <<= 1;
+    // blocks an SM: shared memory, and 512 columns of tensor memory between them
+    per_sm = (int)(228 * 1024 / (smem + 2048));
+    const int by_tmem = 512 / (int)q.tmem_cols;
+    if (per_sm > by_tmem) per_sm = by_tmem;
+    if (per_sm > 2) per_sm = 2;  // registers
+    if (per_sm < 1 || q.wst) per_sm = 1;
+    const size_t least = (size_t)(228 * 1024) / (per_sm + 1) - 1024;  // no more blocks than that fit
+    if (smem < least) smem = least;
+    return true;
+}
+
+cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, const __nv_bfloat16* w, const float* bias,
+                            float* y, int N, int H, int W, int cout_all, int relu, cudaStream_t s)
+{
+    const int cin = ca + cb;
+    // output channels in equal tiles of at most 256 (one MMA's N), multiples of 16
+    const int n_tiles = (cout_all + 255) / 256;
+    if (cin % 16 || ca % 8 || cout_all % (16 * n_tiles) || cin < 16 || cout_all < 16 || H < 1 || W < 1)
+        return cudaErrorInvalidValue;
+    HaloArgs q;
+    q.src = ConvSrc{a, b, ca, cb};
+    q.w = w;
+    q.bias = bias;
+    q.y = y;
+    q.H = H;
+    q.W = W;
+    q.cin = cin;
+    q.cout_all = cout_all;
+    q.cout = cout_all / n_tiles;
+    q.KC = conv_kc(cin);
+    q.relu = relu;
+    size_t smem = 0;
+    int per_sm = 1;
+    if (halo_plan(q, smem, per_sm)) {
+        const long long tiles = (long long)N * (H / 16) * (W / 8);
+        if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+        q.n_tiles = (int)tiles;
+        long long blocks = 152LL * per_sm / n_tiles;
+        if (blocks < 1) blocks = 1;
+        if (blocks > tiles) blocks = tiles;
+        const dim3 grid((unsigned)blocks, n_tiles);
+        if (q.wst) return q.KC == 64 ? launch_halo<4, true>(q, grid, smem, s) : launch_halo<0, true>(q, grid, smem, s);
+        switch (cin / 16) {
+        case 1: return launch_halo<1, false>(q, grid, smem, s);
+        case 2: return launch_halo<2, false>(q, grid, smem, s);
+        case 3: return launch_halo<3, false>(q, grid, smem, s);
+        case 4: return launch_halo<4, false>(q, grid, smem, s);
+        default: return launch_halo<0, false>(q, grid, smem, s);
+        }
+    }
+    if (b) return cudaErrorInvalidValue;
+    const int cout = q.cout, KC = q.KC;
+    smem = 2 * ((size_t)kConvM * KC * 2 + (size_t)cout * KC * 2);
+    cudaError_t e = opt_in(conv3x3_tc_kernel, g_gather_ready);
+    if (e != cudaSuccess) return e;
+    uint32_t cols = 32;
+    while ((int)cols < cout) cols <<= 1;
+    const long long P = (long long)N * H * W;
+    const long long blocks = (P + kConvM - 1) / kConvM;
+    conv3x3_tc_kernel<<<dim3((unsigned)blocks, n_tiles), kConvM, smem, s>>>(a, w, bias, y, P, H, W, cin, cout_all, cout,
+                                                                            KC, relu, cols);
+    return cudaGetLastError();
+}
+
 cudaError_t conv3x3_fwd(const float* x, const __nv_bfloat16* w, const float* bias, float* y, int N, int H, int W,
                         int cin, int cout_all, int relu, cudaStream_t s)
 {
-    // output channels in equal tiles of at most 256 (one MMA's N), multiples of 16
-    const int n_tiles = (cout_all + 255) / 256;
-    if (cin % 16 || cout_all % (16 * n_tiles) || cin < 16 || cout_all < 16 || H < 1 || W < 1)
-        return cudaErrorInvalidValue;
-    const int cout = cout_all / n_tiles;
-    const int KC = conv_kc(cin);
-    const size_t smem = 2 * ((size_t)kConvM * KC * 2 + (size_t)cout * KC * 2);
-    static int attr_bytes = 0;
-    if ((int)smem > attr_bytes) {
-        cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_bytes = (int)smem;
-    }
-    uint32_t cols = 32;
-    while ((int)cols < cout) cols <<= 1;
-    // halo tiles where the image divides into 16 x 8 tiles and the halo of
-    // all channels fits beside the two weight buffers
-    const size_t halo_smem = (size_t)kHaloP * cin * 2 + 2 * (size_t)cout * KC * 2;
-    // every tap's weights beside the halo when both fit in 64 KB (3 blocks an
-    // SM): measured 206 -> 192 us for 32 -> 32 channels at 1024^2, 45 -> 32 us
-    // for a batch of 8 at 128^2; at 97 KB (64 -> 64) it was 4 % slower
-    const size_t res_smem = (size_t)kHaloP * cin * 2 + 9 * (size_t)cin * cout * 2;
-    const int resident = res_smem <= 64 * 1024 ? 1 : 0;
-    const size_t hsm = resident ? res_smem : halo_smem;
-    if (H % 16 == 0 && W % 8 == 0 && halo_smem <= 200 * 1024) {
-        static int halo_attr = 0;
-        if ((int)hsm > halo_attr) {
-            cudaError_t e =
-                cudaFuncSetAttribute(conv3x3_halo_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm);
-            if (e != cudaSuccess) return e;
-            halo_attr = (int)hsm;
-        }
-        const long long blocks = (long long)N * (H / 16) * (W / 8);
-        conv3x3_halo_tc_kernel<<<dim3((unsigned)blocks, n_tiles), kConvM, hsm, s>>>(x, w, bias, y, H, W, cin,
-                                                                                    cout_all, cout, KC, relu, cols,
-                                                                                    resident);
-        return cudaGetLastError();
-    }
-    const long long P = (long long)N * H * W;
-    const long long blocks = (P + kConvM - 1) / kConvM;
-    conv3x3_tc_kernel<<<dim3((unsigned)blocks, n_tiles), kConvM, smem, s>>>(x, w, bias, y, P, H, W, cin, cout_all,
-                                                                            cout, KC, relu, cols);
-    return cudaGetLastError();
+    return conv3x3_fwd_src(x, nullptr, cin, 0, w, bias, y, N, H, W, cout_all, relu, s);
 }
 
 int conv_error()
@@ -636,11 +938,250 @@ __global__ void __launch_bounds__(kConvM) conv3x3_wgrad_tc_kernel(const float* _
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols));
 }
 
-cudaError_t conv3x3_wgrad(const float* x, const float* dy, float* dw, int N, int H, int W, int cin, int cout,
-                          cudaStream_t s)
+// Halo form of the weight gradient (H a multiple of 16, W of 8): no transposed
+// gathers.  Both operands are MN-major in shared memory as they lie in the
+// image: A = dy of a 16 x 8 tile, [8-channel slice][pixel][8] (M = 128 output
+// channels; rows beyond cout read whatever follows and are never stored), B =
+// x of the tile's halo in the same layout, a tap's pixels being a start offset
+// as in the forward kernel; K = 16 pixels, two tile rows, a call (K groups of 8
+// pixels: 128 bytes apart in A, one halo row apart in B; slices are the M and N
+// groups).  A block takes `taps` taps (all nine, or the three of one row dy) of
+// one output-channel tile and nci input channels, keeps their accumulators in
+// tensor memory (taps x nci <= 512 columns) over all its tiles and adds them to
+// dw once at the end, four floats an atomic.  Warps 0-3 load and convert dy,
+// warps 4-11 x (two buffers), warp 12 issues the MMAs, warps 0-3 store.
+constexpr int kWgDyT = 128, kWgXT = 256, kWgLoadT = kWgDyT + kWgXT, kWgThreads = kWgLoadT + 32;
+constexpr int kDyS = kConvM + 1;  // pixels a dy slice (129 x 16 bytes: conflict-free stores)
+
+struct WgradArgs {
+    ConvSrc src;
+    const float* dy;
+    float* dw;
+    int H, W, n_tiles, cin, cout, nci, vec;
+    size_t buf_b;  // bytes of one buffer (dy, then x)
+    uint32_t tmem_cols;
+};
+
+template <int TAPS>
+__global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_halo_kernel(const WgradArgs q)
 {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint32_t s_tmem;
+    __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_done;
+    __shared__ int s_tab[2 * kHaloP];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_ntiles = q.cin / q.nci;
+    const int co0 = ((int)blockIdx.y / n_ntiles) * kConvM, ci0 = ((int)blockIdx.y % n_ntiles) * q.nci;
+    const int tap0 = blockIdx.z * TAPS;
+    const int mco = min(kConvM, q.cout - co0), m8 = mco / 8, n8 = q.nci / 8;
+    const size_t dy_b = (size_t)kDyS * 16 * m8;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(q.tmem_cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(&s_full[k], kWgLoadT);
+            mbar_init(&s_empty[k], 1);
+        }
+        mbar_init(&s_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    fill_halo_table(s_tab, q.src, q.W, tid, kWgThreads);
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = s_tmem;
+    const int tiles_x = q.W / 8, tiles_img = tiles_x * (q.H / 16);
+    // taps of one row dy need the halo rows 1 + dy .. 16 + dy only
+    const int r0 = TAPS == 3 ? tap0 / 3 : 0, rows = TAPS == 3 ? 16 : kHaloY;
+
+    bool ok = true;
+    if (warp < kWgLoadT / 32) {
+        int k = 0;
+        for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x, ++k) {
+            const int buf = k & 1, use = k >> 1;
+            if (use > 0 && !mbar_wait_bounded(&s_empty[buf], (use - 1) & 1)) {
+                atomicOr(&g_conv_error, 4);
+                ok = false;
+                break;
+            }
+            const int img = t / tiles_img, r = t - img * tiles_img, by = r / tiles_x;
+            const int ty0 = by * 16, tx0 = (r - by * tiles_x) * 8;
+            unsigned char* sA = smem_raw + buf * q.buf_b;
+            if (warp < 4) {
+                // dy of the tile: a thread keeps one 8-channel slice, six pieces in flight
+                constexpr int B = 6;
+                const int dq = kWgDyT / m8, p0 = tid / m8, c8 = tid - p0 * m8;
+                const float* base = q.dy + (((size_t)img * q.H + ty0) * q.W + tx0) * q.cout + co0 + 8 * c8;
+                unsigned char* o = sA + ((size_t)c8 * kDyS + p0) * 16;
+                for (int px = p0; px < kConvM && p0 < dq; px += B * dq, o += B * dq * 16) {
+                    float4 f[B][2];
+#pragma unroll
+                    for (int j = 0; j < B; ++j) {
+                        const int p = px + j * dq;
+                        if (p < kConvM) {
+                            const float4* g = reinterpret_cast<const float4*>(
+                                base + (size_t)((p >> 3) * q.W + (p & 7)) * q.cout);
+                            f[j][0] = __ldg(g);
+                            f[j][1] = __ldg(g + 1);
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < B; ++j)
+                        if (px + j * dq < kConvM)
+                            *reinterpret_cast<uint4*>(o + j * dq * 16) =
+                                make_uint4(pack_bf16(f[j][0].x, f[j][0].y), pack_bf16(f[j][0].z, f[j][0].w),
+                                           pack_bf16(f[j][1].x, f[j][1].y), pack_bf16(f[j][1].z, f[j][1].w));
+                }
+            } else {
+                load_halo(q.src, s_tab, sA + dy_b, img, ty0, tx0, q.H, q.W, ci0, n8, r0, rows, tid - kWgDyT, kWgXT);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&s_full[buf]);
+        }
+    } else {
+        if (elect_one()) {
+            // as umma_idesc_bf16, A and B MN-major (bits 15, 16)
+            const uint32_t idesc = umma_idesc_bf16(kConvM, q.nci) | (1u << 15) | (1u << 16);
+            int k = 0;
+            for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x, ++k) {
+                const int buf = k & 1;
+                if (!mbar_wait_bounded(&s_full[buf], (k >> 1) & 1)) {
+                    atomicOr(&g_conv_error, 256);
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t sa = smem_u32(smem_raw + buf * q.buf_b);
+                const uint64_t a0 = umma_desc(sa, 128, kDyS * 16);
+                const uint32_t more = k > 0 ? 1u : 0u;
+                // halo rows start at r0: a row of taps (TAPS = 3) reads rows 0 .. 15
+                const uint64_t b0 = umma_desc(sa + (uint32_t)dy_b, kHaloX * 16, kHaloS * 16);
+#pragma unroll
+                for (int tp = 0; tp < TAPS; ++tp) {
+                    const uint64_t bt = b0 + (TAPS == 9 ? (tp / 3) * kHaloX + tp % 3 : tp);
+                    const uint32_t d = tmem + (uint32_t)(tp * q.nci);
+#pragma unroll
+                    for (int k16 = 0; k16 < 8; ++k16)
+                        umma_bf16(d, a0 + k16 * 16, bt + k16 * 2 * kHaloX, idesc, k16 > 0 ? 1u : more);
+                }
+                umma_commit(&s_empty[buf]);
+            }
+            umma_commit(&s_done);
+        }
+        __syncwarp();
+    }
+    if (warp < 4) {
+        const bool any = (int)blockIdx.x < q.n_tiles;
+        const bool done = mbar_wait_bounded(&s_done, 0);
+        if (!done) atomicOr(&g_conv_error, 8);
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (ok && done && any) {
+            const int co = co0 + tid;  // this thread's TMEM lane = D row
+            for (int tp = 0; tp < TAPS; ++tp)
+                for (int c = 0; c < q.nci; c += 16) {
+                    uint32_t r[16];
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                        "[%16];"
+                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                          "=r"(r[15])
+                        : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(tp * q.nci + c)));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (tid < mco) {
+                        float* d = q.dw + ((size_t)(tap0 + tp) * q.cout + co) * q.cin + ci0 + c;
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4) {
+                            const float4 v = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
+                                                         __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+                            if (q.vec) {
+                                atomicAdd(reinterpret_cast<float4*>(d + j), v);
+                            } else {
+                                atomicAdd(d + j, v.x);
+                                atomicAdd(d + j + 1, v.y);
+                                atomicAdd(d + j + 2, v.z);
+                                atomicAdd(d + j + 3, v.w);
+                            }
+                        }
+                    }
+                }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(q.tmem_cols));
+}
+
+// Launches the halo form where it applies; false otherwise.
+static bool wgrad_halo(const ConvSrc& src, const float* dy, float* dw, int N, int H, int W, int cin, int cout,
+                       cudaStream_t s, cudaError_t& err)
+{
+    const uintptr_t al = (uintptr_t)src.a | (uintptr_t)src.b | (uintptr_t)dy;
+    if (H % 16 || W % 8 || src.ca % 8 || (al & 15)) return false;
+    WgradArgs q;
+    q.src = src;
+    q.dy = dy;
+    q.dw = dw;
+    q.H = H;
+    q.W = W;
+    q.cin = cin;
+    q.cout = cout;
+    q.vec = ((uintptr_t)dw & 15) == 0;
+    // all nine taps where their accumulators fit, else one row of three
+    const int taps = cin <= 48 ? 9 : 3;
+    int nt = 1;
+    while (cin % (16 * nt) || cin / nt > 160) {
+        if (++nt > cin / 16) return false;
+    }
+    q.nci = cin / nt;
+    const int n_mtiles = (cout + kConvM - 1) / kConvM, mco = cout < kConvM ? cout : kConvM;
+    q.buf_b = (size_t)kDyS * 16 * (mco / 8) + (size_t)kHaloS * 16 * (q.nci / 8);
+    // an A descriptor spans the slices of 128 channels, valid or not
+    size_t smem = 2 * q.buf_b;
+    const size_t span = q.buf_b + (size_t)kDyS * 16 * 16;
+    if (smem < span) smem = span;
+    if (smem > kSmemMax) return false;
+    q.tmem_cols = 32;
+    while ((int)q.tmem_cols < taps * q.nci) q.tmem_cols <<= 1;
+    int per_sm = (int)(228 * 1024 / (smem + 2048));
+    const int by_tmem = 512 / (int)q.tmem_cols;
+    if (per_sm > by_tmem) per_sm = by_tmem;
+    if (per_sm > 2) per_sm = 2;  // registers
+    if (per_sm < 1) per_sm = 1;
+    const size_t least = (size_t)(228 * 1024) / (per_sm + 1) - 1024;  // no more blocks than that fit
+    if (smem < least) smem = least;
+    const long long tiles = (long long)N * (H / 16) * (W / 8);
+    if (tiles > 0x7fffffff) return false;
+    q.n_tiles = (int)tiles;
+    const int groups = n_mtiles * nt * (9 / taps);
+    long long chunks = 152LL * per_sm / groups;
+    if (chunks < 1) chunks = 1;
+    if (chunks > tiles) chunks = tiles;
+    const dim3 grid((unsigned)chunks, n_mtiles * nt, 9 / taps);
+    err = taps == 9 ? opt_in(conv3x3_wgrad_halo_kernel<9>, g_wgrad9_ready)
+                    : opt_in(conv3x3_wgrad_halo_kernel<3>, g_wgrad3_ready);
+    if (err != cudaSuccess) return true;
+    if (taps == 9)
+        conv3x3_wgrad_halo_kernel<9><<<grid, kWgThreads, smem, s>>>(q);
+    else
+        conv3x3_wgrad_halo_kernel<3><<<grid, kWgThreads, smem, s>>>(q);
+    err = cudaGetLastError();
+    return true;
+}
+
+cudaError_t conv3x3_wgrad_src(const float* a, const float* b, int ca, int cb, const float* dy, float* dw, int N, int H,
+                              int W, int cout, cudaStream_t s)
+{
+    const int cin = ca + cb;
     const int n_ntiles = (cin + 255) / 256;
     if (cin % 16 || cout % 16 || cin < 16 || cout < 16 || cin % (16 * n_ntiles)) return cudaErrorInvalidValue;
+    cudaError_t e = cudaSuccess;
+    if (wgrad_halo(ConvSrc{a, b, ca, cb}, dy, dw, N, H, W, cin, cout, s, e)) return e;
+    if (b) return cudaErrorInvalidValue;
     const int nci = cin / n_ntiles, n_mtiles = (cout + kConvM - 1) / kConvM;
     const long long P = (long long)N * H * W;
     // about four blocks an SM in all: pixel chunks of a multiple of 64
@@ -649,18 +1190,19 @@ cudaError_t conv3x3_wgrad(const float* x, const float* dy, float* dw, int N, int
     KP = ((KP + kWgK - 1) / kWgK) * kWgK;
     chunks = (P + KP - 1) / KP;
     const size_t smem = 2 * ((size_t)kConvM * kWgK * 2 + (size_t)nci * kWgK * 2);
-    static int attr_bytes = 0;
-    if ((int)smem > attr_bytes) {
-        cudaError_t e =
-            cudaFuncSetAttribute(conv3x3_wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_bytes = (int)smem;
-    }
+    e = opt_in(conv3x3_wgrad_tc_kernel, g_wgrad_ready);
+    if (e != cudaSuccess) return e;
     uint32_t cols = 32;
     while ((int)cols < nci) cols <<= 1;
     dim3 grid((unsigned)chunks, (unsigned)(n_mtiles * n_ntiles), 9);
-    conv3x3_wgrad_tc_kernel<<<grid, kConvM, smem, s>>>(x, dy, dw, P, H, W, cin, cout, nci, KP, cols);
+    conv3x3_wgrad_tc_kernel<<<grid, kConvM, smem, s>>>(a, dy, dw, P, H, W, cin, cout, nci, KP, cols);
     return cudaGetLastError();
+}
+
+cudaError_t conv3x3_wgrad(const float* x, const float* dy, float* dw, int N, int H, int W, int cin, int cout,
+                          cudaStream_t s)
+{
+    return conv3x3_wgrad_src(x, nullptr, cin, 0, dy, dw, N, H, W, cout, s);
 }
 
 // Elementwise and small kernels -------------------------------------------------
