@@ -727,6 +727,7 @@ cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, cons
         case 2: return launch_halo<2, false>(q, grid, smem, s);
         case 3: return launch_halo<3, false>(q, grid, smem, s);
         case 4: return launch_halo<4, false>(q, grid, smem, s);
+        case 6: return launch_halo<6, false>(q, grid, smem, s);
         default: return launch_halo<0, false>(q, grid, smem, s);
         }
     }
@@ -945,9 +946,9 @@ __global__ void __launch_bounds__(kConvM) conv3x3_wgrad_tc_kernel(const float* _
 // x of the tile's halo in the same layout, a tap's pixels being a start offset
 // as in the forward kernel; K = 16 pixels, two tile rows, a call (K groups of 8
 // pixels: 128 bytes apart in A, one halo row apart in B; slices are the M and N
-// groups).  A block takes `taps` taps (all nine, or the three of one row dy) of
+// groups).  A block takes TAPS taps (all nine, or the three of one row dy) of
 // one output-channel tile and nci input channels, keeps their accumulators in
-// tensor memory (taps x nci <= 512 columns) over all its tiles and adds them to
+// tensor memory (TAPS x nci <= 512 columns) over all its tiles and adds them to
 // dw once at the end, four floats an atomic.  Warps 0-3 load and convert dy,
 // warps 4-11 x (two buffers), warp 12 issues the MMAs, warps 0-3 store.
 constexpr int kWgDyT = 128, kWgXT = 256, kWgLoadT = kWgDyT + kWgXT, kWgThreads = kWgLoadT + 32;
@@ -969,7 +970,7 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_halo_kernel(const Wg
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_full[2], s_empty[2], s_done;
     __shared__ int s_tab[2 * kHaloP];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int n_ntiles = q.cin / q.nci;
     const int co0 = ((int)blockIdx.y / n_ntiles) * kConvM, ci0 = ((int)blockIdx.y % n_ntiles) * q.nci;
     const int tap0 = blockIdx.z * TAPS;
@@ -1207,200 +1208,235 @@ cudaError_t conv3x3_wgrad(const float* x, const float* dy, float* dw, int N, int
 
 // Elementwise and small kernels -------------------------------------------------
 
-__global__ void bias_grad_kernel(const float* dy, float* db, long long P, int c)
-{
-    // one block per channel
-    const int ch = blockIdx.x;
-    float acc = 0.f;
-    for (long long p = threadIdx.x; p < P; p += blockDim.x) acc += dy[p * c + ch];
-    __shared__ float red[256];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) db[ch] += red[0];
-}
-
-cudaError_t bias_grad(const float* dy, float* db, long long P, int c, cudaStream_t s)
-{
-    bias_grad_kernel<<<c, 256, 0, s>>>(dy, db, P, c);
-    return cudaGetLastError();
-}
-
-__global__ void relu_bwd_kernel(const float* y, float* dy, long long n)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        if (!(y[i] > 0.f)) dy[i] = 0.f;
-}
-
 static int eblocks(long long n)
 {
     long long b = (n + 255) / 256;
     return (int)(b < 1 ? 1 : (b > 152 * 32 ? 152 * 32 : b));
 }
 
-cudaError_t relu_bwd(const float* y, float* dy, long long n, cudaStream_t s)
-{
-    relu_bwd_kernel<<<eblocks(n), 256, 0, s>>>(y, dy, n);
-    return cudaGetLastError();
-}
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
-// 2 x 2 average pool (NHWC) and its gradient.
-__global__ void pool_fwd_kernel(const float* x, float* y, int N, int H, int W, int c)
+// Sum of v over the block's threads with the same tid % q4 (q4 a power of two
+// dividing 256), added to out[4 (tid % q4) ..] by the first q4 threads.
+__device__ __forceinline__ void block_sum4(float4 v, int q4, float* out, float4* red)
 {
-    const int Ho = H / 2, Wo = W / 2;
-    const long long total = (long long)N * Ho * Wo * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = i % c;
-        long long r = i / c;
-        const int xo = r % Wo;
-        r /= Wo;
-        const int yo = r % Ho;
-        const int n = (int)(r / Ho);
-        const float* b = x + (((size_t)n * H + 2 * yo) * W + 2 * xo) * c + ch;
-        y[i] = 0.25f * (b[0] + b[c] + b[(size_t)W * c] + b[(size_t)W * c + c]);
+    __syncthreads();
+    red[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 128; o >= q4; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] = add4(red[threadIdx.x], red[threadIdx.x + o]);
+        __syncthreads();
+    }
+    if ((int)threadIdx.x < q4) {
+        const float4 t = red[threadIdx.x];
+        atomicAdd(out + 4 * threadIdx.x, t.x);
+        atomicAdd(out + 4 * threadIdx.x + 1, t.y);
+        atomicAdd(out + 4 * threadIdx.x + 2, t.z);
+        atomicAdd(out + 4 * threadIdx.x + 3, t.w);
     }
 }
 
-__global__ void pool_bwd_kernel(const float* dy, float* dx, int N, int H, int W, int c)
+// Gradient before a layer's ReLU and the layer's bias gradient, in one pass:
+//   dst[p][ch] = y[p][ch] > 0 ? g[p][ch] : 0,   db[ch] += sum_p dst[p][ch],
+// where g is, by `from`:
+//   kFromSame   src[p][ch] (dst may be src);
+//   kFromUp     the sum over the pixel's 2 x 2 children in src (N, 2H, 2W, sc),
+//               channel ch (backward of the nearest upsampling);
+//   kFromPool   0.25 src[parent][ch] (N, H/2, W/2, c: backward of the pooling)
+//               + skip[p][so + ch] (N, H, W, sc: the decoder's skip gradient).
+// Bound by memory: 12 to 17 bytes an element.  A thread keeps one channel quad
+// (c / 4 a power of two) and sums it over its pixels; a block adds once.
+// Replaces a ReLU, a pooling or upsampling, an addition and a one-block-a-channel
+// sum (for 16 channels at 8 x 128^2: 76 us of 90, now 8 in all).
+enum { kFromSame, kFromUp, kFromPool };
+template <int FROM>
+__global__ void __launch_bounds__(256) act_bwd_kernel(const float* y, const float* src, const float* skip, float* dst,
+                                                      float* db, long long P, int H, int W, int c, int sc, int so)
 {
-    const long long total = (long long)N * H * W * c;
-    const int Wo = W / 2, Ho = H / 2;
+    __shared__ float4 red[256];
+    const int q4 = c / 4, ch = 4 * ((int)threadIdx.x % q4), ppb = 256 / q4;
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long p = (long long)blockIdx.x * ppb + threadIdx.x / q4; p < P; p += (long long)gridDim.x * ppb) {
+        float4 g;
+        if (FROM == kFromSame) {
+            g = ld4(src + p * c + ch);
+        } else {
+            const int x = (int)(p % W);
+            const long long r = p / W;
+            const int yy = (int)(r % H);
+            const long long n = r / H;
+            if (FROM == kFromUp) {
+                const float* b = src + ((n * 2 * H + 2 * yy) * 2 * W + 2 * x) * sc + ch;
+                const size_t row = (size_t)2 * W * sc;
+                g = add4(add4(add4(ld4(b), ld4(b + sc)), ld4(b + row)), ld4(b + row + sc));
+            } else {
+                const float4 a = ld4(src + ((n * (H / 2) + yy / 2) * (W / 2) + x / 2) * c + ch);
+                g = make_float4(0.25f * a.x, 0.25f * a.y, 0.25f * a.z, 0.25f * a.w);
+                if (skip) g = add4(g, ld4(skip + p * sc + so + ch));
+            }
+        }
+        const float4 v = ld4(y + p * c + ch);
+        if (!(v.x > 0.f)) g.x = 0.f;
+        if (!(v.y > 0.f)) g.y = 0.f;
+        if (!(v.z > 0.f)) g.z = 0.f;
+        if (!(v.w > 0.f)) g.w = 0.f;
+        st4(dst + p * c + ch, g);
+        sum = add4(sum, g);
+    }
+    block_sum4(sum, q4, db, red);
+}
+
+static int act_blocks(long long P, int c)
+{
+    const long long b = (P + 256 / (c / 4) - 1) / (256 / (c / 4));
+    return (int)(b < 1 ? 1 : (b > 152 * 4 ? 152 * 4 : b));
+}
+
+cudaError_t act_bwd(const float* y, float* dy, float* db, long long P, int c, cudaStream_t s)
+{
+    act_bwd_kernel<kFromSame><<<act_blocks(P, c), 256, 0, s>>>(y, dy, nullptr, dy, db, P, 1, 1, c, 0, 0);
+    return cudaGetLastError();
+}
+cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* db, int N, int H, int W, int c, int sc,
+                       cudaStream_t s)
+{
+    const long long P = (long long)N * H * W;
+    act_bwd_kernel<kFromUp><<<act_blocks(P, c), 256, 0, s>>>(y, src, nullptr, dst, db, P, H, W, c, sc, 0);
+    return cudaGetLastError();
+}
+cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* db, int N, int H, int W,
+                         int c, int sc, int so, cudaStream_t s)
+{
+    const long long P = (long long)N * H * W;
+    act_bwd_kernel<kFromPool><<<act_blocks(P, c), 256, 0, s>>>(y, src, skip, dst, db, P, H, W, c, sc, so);
+    return cudaGetLastError();
+}
+
+// 2 x 2 average pool (NHWC), a channel quad a thread.
+__global__ void pool_fwd_kernel(const float* x, float* y, int N, int H, int W, int c)
+{
+    const int Ho = H / 2, Wo = W / 2, q4 = c / 4;
+    const long long total = (long long)N * Ho * Wo * q4;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
-        const int ch = i % c;
-        long long r = i / c;
-        const int xx = r % W;
-        r /= W;
-        const int yy = r % H;
-        const int n = (int)(r / H);
-        dx[i] = 0.25f * dy[(((size_t)n * Ho + yy / 2) * Wo + xx / 2) * c + ch];
+        const int ch = 4 * (int)(i % q4);
+        long long r = i / q4;
+        const int xo = (int)(r % Wo);
+        r /= Wo;
+        const int yo = (int)(r % Ho);
+        const long long n = r / Ho;
+        const float* b = x + ((n * H + 2 * yo) * W + 2 * xo) * c + ch;
+        const float4 t = add4(add4(add4(ld4(b), ld4(b + c)), ld4(b + (size_t)W * c)), ld4(b + (size_t)W * c + c));
+        st4(y + 4 * i, make_float4(0.25f * t.x, 0.25f * t.y, 0.25f * t.z, 0.25f * t.w));
     }
 }
 
 cudaError_t pool_fwd(const float* x, float* y, int N, int H, int W, int c, cudaStream_t s)
 {
-    pool_fwd_kernel<<<eblocks((long long)N * H * W * c / 4), 256, 0, s>>>(x, y, N, H, W, c);
-    return cudaGetLastError();
-}
-cudaError_t pool_bwd(const float* dy, float* dx, int N, int H, int W, int c, cudaStream_t s)
-{
-    pool_bwd_kernel<<<eblocks((long long)N * H * W * c), 256, 0, s>>>(dy, dx, N, H, W, c);
+    pool_fwd_kernel<<<eblocks((long long)N * H * W * c / 16), 256, 0, s>>>(x, y, N, H, W, c);
     return cudaGetLastError();
 }
 
-// Nearest 2x upsample of `a` (N, H/2, W/2, ca) concatenated with the skip `b`
-// (N, H, W, cb) into y (N, H, W, ca + cb), and the backward split.
-__global__ void upcat_fwd_kernel(const float* a, const float* b, float* y, int N, int H, int W, int ca, int cb)
+// The head, forward: out[p] = b + w x[p] (2 outputs, FP32), the first times the
+// interface gate 1 - phi^2 (xin[p][0] = phi), so that the network changes phi
+// only in the diffuse interface.  Written to out, and to y when given.
+__global__ void head_fwd_kernel(const float* x, const float* w, const float* b, const float* xin, int cx, float* out,
+                                float* y, long long P, int c)
 {
-    const int c = ca + cb;
-    const long long total = (long long)N * H * W * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = i % c;
-        const long long p = i / c;
-        const int xx = p % W;
-        const long long r = p / W;
-        const int yy = r % H;
-        const int n = (int)(r / H);
-        y[i] = ch < ca ? a[(((size_t)n * (H / 2) + yy / 2) * (W / 2) + xx / 2) * ca + ch] : b[p * cb + (ch - ca)];
-    }
-}
-
-__global__ void upcat_bwd_kernel(const float* dy, float* da, float* db, int N, int H, int W, int ca, int cb)
-{
-    // da: sum over the 2 x 2 children; db: copy
-    const int c = ca + cb;
-    const long long total_a = (long long)N * (H / 2) * (W / 2) * ca;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total_a;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = i % ca;
-        long long r = i / ca;
-        const int xo = r % (W / 2);
-        r /= (W / 2);
-        const int yo = r % (H / 2);
-        const int n = (int)(r / (H / 2));
-        const float* b0 = dy + (((size_t)n * H + 2 * yo) * W + 2 * xo) * c + ch;
-        da[i] = b0[0] + b0[c] + b0[(size_t)W * c] + b0[(size_t)W * c + c];
-    }
-    const long long total_b = (long long)N * H * W * cb;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total_b;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = i % cb;
-        const long long p = i / cb;
-        db[i] = dy[p * c + ca + ch];
-    }
-}
-
-cudaError_t upcat_fwd(const float* a, const float* b, float* y, int N, int H, int W, int ca, int cb, cudaStream_t s)
-{
-    upcat_fwd_kernel<<<eblocks((long long)N * H * W * (ca + cb)), 256, 0, s>>>(a, b, y, N, H, W, ca, cb);
-    return cudaGetLastError();
-}
-cudaError_t upcat_bwd(const float* dy, float* da, float* db, int N, int H, int W, int ca, int cb, cudaStream_t s)
-{
-    upcat_bwd_kernel<<<eblocks((long long)N * H * W * cb), 256, 0, s>>>(dy, da, db, N, H, W, ca, cb);
-    return cudaGetLastError();
-}
-
-// 1 x 1 convolution (FP32): y[p][co] = b[co] + sum_ci w[co][ci] x[p][ci].
-__global__ void conv1x1_fwd_kernel(const float* x, const float* w, const float* b, float* y, long long P, int cin,
-                                   int cout)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * cout;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int co = i % cout;
-        const long long p = i / cout;
-        float acc = b[co];
-        for (int ci = 0; ci < cin; ++ci) acc += w[co * cin + ci] * x[p * cin + ci];
-        y[i] = acc;
-    }
-}
-
-// dx[p][ci] = sum_co w[co][ci] dy[p][co]
-__global__ void conv1x1_dgrad_kernel(const float* dy, const float* w, float* dx, long long P, int cin, int cout)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * cin;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ci = i % cin;
-        const long long p = i / cin;
-        float acc = 0.f;
-        for (int co = 0; co < cout; ++co) acc += w[co * cin + ci] * dy[p * cout + co];
-        dx[i] = acc;
-    }
-}
-
-// dw[co][ci] += sum_p dy[p][co] x[p][ci]; one block per (co, ci).
-__global__ void conv1x1_wgrad_kernel(const float* x, const float* dy, float* dw, long long P, int cin, int cout)
-{
-    const int co = blockIdx.x / cin, ci = blockIdx.x % cin;
-    float acc = 0.f;
-    for (long long p = threadIdx.x; p < P; p += blockDim.x) acc += dy[p * cout + co] * x[p * cin + ci];
-    __shared__ float red[256];
-    red[threadIdx.x] = acc;
+    __shared__ float sw[2 * 64];
+    for (int k = threadIdx.x; k < 2 * c; k += blockDim.x) sw[k] = w[k];
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    const float b0 = b[0], b1 = b[1];
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
+        float a0 = b0, a1 = b1;
+        for (int k = 0; k < c; k += 4) {
+            const float4 v = ld4(x + p * c + k);
+            a0 += sw[k] * v.x;
+            a1 += sw[c + k] * v.x;
+            a0 += sw[k + 1] * v.y;
+            a1 += sw[c + k + 1] * v.y;
+            a0 += sw[k + 2] * v.z;
+            a1 += sw[c + k + 2] * v.z;
+            a0 += sw[k + 3] * v.w;
+            a1 += sw[c + k + 3] * v.w;
+        }
+        const float ph = xin[p * cx];
+        a0 *= (1.f - ph) * (1.f + ph);
+        const float2 o = make_float2(a0, a1);
+        reinterpret_cast<float2*>(out)[p] = o;
+        if (y) {  // y: the caller's, any alignment
+            y[2 * p] = a0;
+            y[2 * p + 1] = a1;
+        }
+    }
+}
+
+cudaError_t head_fwd(const float* x, const float* w, const float* b, const float* xin, int cx, float* out, float* y,
+                     long long P, int c, cudaStream_t s)
+{
+    if (c > 64 || c % 4) return cudaErrorInvalidValue;
+    head_fwd_kernel<<<eblocks(P), 256, 0, s>>>(x, w, b, xin, cx, out, y, P, c);
+    return cudaGetLastError();
+}
+
+// The head, backward, with the gate and the last layer's ReLU and bias in the
+// same pass: g = (dy0 (1 - phi^2), dy1); dw += g x^T, db += g; dx = w^T g where
+// x > 0 (x is that layer's output), else 0; db_last += sum dx.
+__global__ void __launch_bounds__(256) head_bwd_kernel(const float* x, const float* dy, const float* w, const float* xin,
+                                                       int cx, float* dx, float* dw, float* db, float* db_last,
+                                                       long long P, int c)
+{
+    __shared__ float4 red[256];
+    const int q4 = c / 4, ch = 4 * ((int)threadIdx.x % q4), ppb = 256 / q4;
+    float w0[4], w1[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        w0[k] = w[ch + k];
+        w1[k] = w[c + ch + k];
+    }
+    float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0, sl = s0, sb = s0;
+    for (long long p = (long long)blockIdx.x * ppb + threadIdx.x / q4; p < P; p += (long long)gridDim.x * ppb) {
+        const float ph = __ldg(xin + p * cx);
+        const float g0 = __ldg(dy + 2 * p) * ((1.f - ph) * (1.f + ph)), g1 = __ldg(dy + 2 * p + 1);
+        const float4 v = ld4(x + p * c + ch);
+        float4 d = make_float4(__fmaf_rn(w1[0], g1, w0[0] * g0), __fmaf_rn(w1[1], g1, w0[1] * g0),
+                               __fmaf_rn(w1[2], g1, w0[2] * g0), __fmaf_rn(w1[3], g1, w0[3] * g0));
+        if (!(v.x > 0.f)) d.x = 0.f;
+        if (!(v.y > 0.f)) d.y = 0.f;
+        if (!(v.z > 0.f)) d.z = 0.f;
+        if (!(v.w > 0.f)) d.w = 0.f;
+        st4(dx + p * c + ch, d);
+        sl = add4(sl, d);
+        s0 = add4(s0, make_float4(g0 * v.x, g0 * v.y, g0 * v.z, g0 * v.w));
+        s1 = add4(s1, make_float4(g1 * v.x, g1 * v.y, g1 * v.z, g1 * v.w));
+        if (ch == 0) {
+            sb.x += g0;
+            sb.y += g1;
+        }
+    }
+    block_sum4(s0, q4, dw, red);
+    block_sum4(s1, q4, dw + c, red);
+    block_sum4(sl, q4, db_last, red);
+    // db: the first quad's threads hold the two sums
+    __syncthreads();
+    red[threadIdx.x] = sb;
+    __syncthreads();
+    for (int o = 128; o >= 1; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] = add4(red[threadIdx.x], red[threadIdx.x + o]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) dw[blockIdx.x] += red[0];
+    if (threadIdx.x == 0) {
+        atomicAdd(db, red[0].x);
+        atomicAdd(db + 1, red[0].y);
+    }
 }
 
-cudaError_t conv1x1_fwd(const float* x, const float* w, const float* b, float* y, long long P, int cin, int cout,
-                        cudaStream_t s)
+cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* dw,
+                     float* db, float* db_last, long long P, int c, cudaStream_t s)
 {
-    conv1x1_fwd_kernel<<<eblocks(P * cout), 256, 0, s>>>(x, w, b, y, P, cin, cout);
-    return cudaGetLastError();
-}
-cudaError_t conv1x1_bwd(const float* x, const float* dy, const float* w, float* dx, float* dw, float* db, long long P,
-                        int cin, int cout, cudaStream_t s)
-{
-    if (dx) conv1x1_dgrad_kernel<<<eblocks(P * cin), 256, 0, s>>>(dy, w, dx, P, cin, cout);
-    conv1x1_wgrad_kernel<<<cin * cout, 256, 0, s>>>(x, dy, dw, P, cin, cout);
-    bias_grad_kernel<<<cout, 256, 0, s>>>(dy, db, P, cout);
+    head_bwd_kernel<<<act_blocks(P, c), 256, 0, s>>>(x, dy, w, xin, cx, dx, dw, db, db_last, P, c);
     return cudaGetLastError();
 }
 
@@ -1475,35 +1511,24 @@ cudaError_t to_bf16(const float* a, __nv_bfloat16* b, long long n, cudaStream_t 
     return cudaGetLastError();
 }
 
-// Pad NHWC channels: y[p][c] = c < cin ? x[p][c] : 0 (cout >= cin).
+// The network input's cin <= 8 channels into the first 8 of 16 (the others were
+// cleared when y was allocated and stay zero): two threads a pixel.
 __global__ void pad_channels_kernel(const float* x, float* y, long long P, int cin, int cout)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * cout;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = i % cout;
-        y[i] = c < cin ? x[(i / cout) * cin + c] : 0.f;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 2 * P; i += (long long)gridDim.x * blockDim.x) {
+        const int c = 4 * (int)(i & 1);
+        const float* b = x + (i >> 1) * cin;
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = c + k < cin ? b[c + k] : 0.f;
+        st4(y + (i >> 1) * cout + c, make_float4(v[0], v[1], v[2], v[3]));
     }
 }
 
 cudaError_t pad_channels(const float* x, float* y, long long P, int cin, int cout, cudaStream_t s)
 {
-    pad_channels_kernel<<<eblocks(P * cout), 256, 0, s>>>(x, y, P, cin, cout);
-    return cudaGetLastError();
-}
-
-}  // namespace lbpf_nn
-
-namespace lbpf_nn {
-
-__global__ void add_kernel(float* a, const float* b, long long n)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        a[i] += b[i];
-}
-
-cudaError_t add_inplace(float* a, const float* b, long long n, cudaStream_t s)
-{
-    add_kernel<<<eblocks(n), 256, 0, s>>>(a, b, n);
+    if (cin > 8 || cout % 4) return cudaErrorInvalidValue;
+    pad_channels_kernel<<<eblocks(2 * P), 256, 0, s>>>(x, y, P, cin, cout);
     return cudaGetLastError();
 }
 
@@ -1588,27 +1613,6 @@ __global__ void range_kernel(const float* phi, long long P, float lo, float hi, 
 cudaError_t range_count(const float* phi, long long P, float lo, float hi, unsigned int* count, cudaStream_t s)
 {
     range_kernel<<<eblocks(P) < 608 ? eblocks(P) : 608, 256, 0, s>>>(phi, P, lo, hi, count);
-    return cudaGetLastError();
-}
-
-}  // namespace lbpf_nn
-
-namespace lbpf_nn {
-
-// Interface gate of the phi output: out[p][0] *= 1 - x[p][0]^2 (x channel 0 is
-// phi), so that the network changes phi only in the diffuse interface.  The
-// same factor scales the gradient.
-__global__ void gate_kernel(const float* x, int cx, float* out, long long P)
-{
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-        const float ph = x[p * cx];
-        out[2 * p] *= (1.f - ph) * (1.f + ph);
-    }
-}
-
-cudaError_t gate(const float* x, int cx, float* out, long long P, cudaStream_t s)
-{
-    gate_kernel<<<eblocks(P), 256, 0, s>>>(x, cx, out, P);
     return cudaGetLastError();
 }
 

@@ -20,29 +20,39 @@ cudaError_t flip_weights(const __nv_bfloat16* w, __nv_bfloat16* wt, int cin, int
 // cores, FP32 accumulation; cin, cout multiples of 16 (cin > 256: of 32).
 cudaError_t conv3x3_wgrad(const float* x, const float* dy, float* dw, int N, int H, int W, int cin, int cout,
                           cudaStream_t s);
-cudaError_t bias_grad(const float* dy, float* db, long long P, int c, cudaStream_t s);
-cudaError_t relu_bwd(const float* y, float* dy, long long n, cudaStream_t s);
+// The same two with the input given in two parts: ca channels at half the
+// resolution (upsampled 2x, nearest), then cb channels (b NULL: cb = 0, a at
+// full resolution).  Two parts need H a multiple of 16 and W of 8.
+cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, const __nv_bfloat16* w, const float* bias,
+                            float* y, int N, int H, int W, int cout, int relu, cudaStream_t s);
+cudaError_t conv3x3_wgrad_src(const float* a, const float* b, int ca, int cb, const float* dy, float* dw, int N, int H,
+                              int W, int cout, cudaStream_t s);
+// Gradient through a layer's ReLU and its bias gradient (act_bwd_kernel): in
+// place; from the 2 x 2 children in src (sc channels a pixel); from the pooled
+// gradient src plus the skip gradient (sc channels a pixel, from so on; may be
+// NULL).  c a power of two, 16 .. 256.
+cudaError_t act_bwd(const float* y, float* dy, float* db, long long P, int c, cudaStream_t s);
+cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* db, int N, int H, int W, int c, int sc,
+                       cudaStream_t s);
+cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* db, int N, int H, int W,
+                         int c, int sc, int so, cudaStream_t s);
 cudaError_t pool_fwd(const float* x, float* y, int N, int H, int W, int c, cudaStream_t s);
-cudaError_t pool_bwd(const float* dy, float* dx, int N, int H, int W, int c, cudaStream_t s);
-cudaError_t upcat_fwd(const float* a, const float* b, float* y, int N, int H, int W, int ca, int cb, cudaStream_t s);
-cudaError_t upcat_bwd(const float* dy, float* da, float* db, int N, int H, int W, int ca, int cb, cudaStream_t s);
-cudaError_t conv1x1_fwd(const float* x, const float* w, const float* b, float* y, long long P, int cin, int cout,
-                        cudaStream_t s);
-cudaError_t conv1x1_bwd(const float* x, const float* dy, const float* w, float* dx, float* dw, float* db, long long P,
-                        int cin, int cout, cudaStream_t s);
+// 1x1 head with the interface gate, c <= 64 channels in, 2 out; y may be NULL.
+cudaError_t head_fwd(const float* x, const float* w, const float* b, const float* xin, int cx, float* out, float* y,
+                     long long P, int c, cudaStream_t s);
+cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* dw,
+                     float* db, float* db_last, long long P, int c, cudaStream_t s);
 cudaError_t mse(const float* p, const float* t, const float* x, int cin, int cout, float alpha, float* dp, double* loss,
                 long long n, cudaStream_t s);
 cudaError_t adam(float* w, const float* g, float* m, float* v, __nv_bfloat16* wb, long long n, float lr, float b1,
                  float b2, float eps, int t, cudaStream_t s);
 cudaError_t to_bf16(const float* a, __nv_bfloat16* b, long long n, cudaStream_t s);
 cudaError_t pad_channels(const float* x, float* y, long long P, int cin, int cout, cudaStream_t s);
-cudaError_t add_inplace(float* a, const float* b, long long n, cudaStream_t s);
 cudaError_t assemble(const float* phi, const float* u, const int* index, const float* tab, int nc, float* x, long long P,
                      cudaStream_t s);
 cudaError_t apply(const float* y, float* phi, float* u, long long P, cudaStream_t s);
 cudaError_t delta(const float* phi0, const float* u0, const float* phi1, const float* u1, float* y, long long P,
                   cudaStream_t s);
-cudaError_t gate(const float* x, int cx, float* out, long long P, cudaStream_t s);
 cudaError_t range_count(const float* phi, long long P, float lo, float hi, unsigned int* count, cudaStream_t s);
 
 }  // namespace lbpf_nn

@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/lbpf.h"
@@ -43,13 +44,13 @@ struct lbpf_net {
     int adam_t = 0;
     float loss_alpha = 0.f;  // interface weight of the training loss
     // activations (N, H >> l, W >> l, c) per level l: encoder convolution
-    // outputs ea, e; pooled input pl (l >= 1); decoder concatenation u and
-    // outputs da, d (l < levels - 1)
+    // outputs ea, e; pooled input pl (l >= 1); decoder outputs da, d (l <
+    // levels - 1; the concatenation of the upsampled level below and the skip is
+    // read in its two parts)
     float *xin = nullptr, *out = nullptr;
-    std::vector<float*> ea, e, pl, u, da, d;
+    std::vector<float*> ea, e, pl, da, d;
     // gradient scratch per level (two of the level's widest channel count)
-    // and the skip gradients of the decoder levels
-    std::vector<float*> ga, gb, gskip;
+    std::vector<float*> ga, gb;
     float* g_out = nullptr;
     double* d_loss = nullptr;
     std::vector<void*> allocs;
@@ -57,6 +58,8 @@ struct lbpf_net {
 
     int ch(int l) const { return base << l; }
     float* top() const { return levels > 1 ? d[0] : e[0]; }
+    // output of the level below decoder level l
+    float* below(int l) const { return l == levels - 2 ? e[l + 1] : d[l + 1]; }
 };
 
 namespace {
@@ -180,12 +183,10 @@ extern "C" int lbpf_net_create_arch(int H, int W, int batch, int levels, int bas
     net->ea.assign(levels, nullptr);
     net->e.assign(levels, nullptr);
     net->pl.assign(levels, nullptr);
-    net->u.assign(levels, nullptr);
     net->da.assign(levels, nullptr);
     net->d.assign(levels, nullptr);
     net->ga.assign(levels, nullptr);
     net->gb.assign(levels, nullptr);
-    net->gskip.assign(levels, nullptr);
     ok = ok && (net->xin = alloc_f(net, P0 * kInPad)) && (net->out = alloc_f(net, P0 * kOut)) &&
          (net->g_out = alloc_f(net, P0 * kOut));
     for (int l = 0; l < levels && ok; ++l) {
@@ -195,8 +196,7 @@ extern "C" int lbpf_net_create_arch(int H, int W, int batch, int levels, int bas
              (net->ga[l] = alloc_f(net, Pl * cw)) && (net->gb[l] = alloc_f(net, Pl * cw));
         if (ok && l > 0) ok = (net->pl[l] = alloc_f(net, Pl * net->ch(l - 1))) != nullptr;
         if (ok && l + 1 < levels)
-            ok = (net->u[l] = alloc_f(net, Pl * cw)) && (net->da[l] = alloc_f(net, Pl * c)) &&
-                 (net->d[l] = alloc_f(net, Pl * c)) && (net->gskip[l] = alloc_f(net, Pl * c));
+            ok = (net->da[l] = alloc_f(net, Pl * c)) && (net->d[l] = alloc_f(net, Pl * c));
     }
     void* dl = nullptr;
     ok = ok && cudaMalloc(&dl, sizeof(double)) == cudaSuccess;
@@ -274,7 +274,7 @@ extern "C" int lbpf_net_set_params(lbpf_net* net, const float* host)
 
 namespace {
 
-int forward(lbpf_net* net, const float* x)
+int forward(lbpf_net* net, const float* x, float* y)
 {
     const int N = net->N, H = net->H, W = net->W, lv = net->levels;
     const long long P0 = (long long)N * H * W;
@@ -295,59 +295,70 @@ int forward(lbpf_net* net, const float* x)
         NK(cv(k + 1, net->ea[l], net->e[l], l));
         k += 2;
     }
-    const float* prev = net->e[lv - 1];
     for (int l = lv - 2; l >= 0; --l) {
-        NK(upcat_fwd(prev, net->e[l], net->u[l], N, H >> l, W >> l, net->ch(l + 1), net->ch(l), s));
-        NK(cv(k, net->u[l], net->da[l], l));
+        const Conv& c = net->conv[k];
+        NK(conv3x3_fwd_src(net->below(l), net->e[l], net->ch(l + 1), net->ch(l), c.wb, net->p + c.off_b, net->da[l], N,
+                           H >> l, W >> l, c.cout, 1, s));
         NK(cv(k + 1, net->da[l], net->d[l], l));
-        prev = net->d[l];
         k += 2;
     }
-    NK(conv1x1_fwd(prev, net->p + net->off_hw, net->p + net->off_hb, net->out, P0, net->ch(0), kOut, s));
-    NK(gate(net->xin, kInPad, net->out, P0, s));
+    NK(head_fwd(net->top(), net->p + net->off_hw, net->p + net->off_hb, net->xin, kInPad, net->out, y, P0, net->ch(0),
+                s));
     return LBPF_OK;
 }
 
-// Backward from g_out (dL/d out); accumulates parameter gradients into g.
-// Mirrors the forward pass: decoder levels from the top down (their skip
-// gradients kept), then the encoder from the deepest level up.
-int backward(lbpf_net* net)
+// Backward from dy (dL/d out); accumulates parameter gradients into g.
+// Mirrors the forward pass: decoder levels from the top down, then the encoder
+// from the deepest level up.  A layer's gradient arrives masked by its ReLU,
+// with its bias gradient already summed (head_bwd, act_bwd*).
+int backward(lbpf_net* net, const float* dy)
 {
     const int N = net->N, H = net->H, W = net->W, lv = net->levels;
     const long long P0 = (long long)N * H * W;
     cudaStream_t s = net->stream;
     float* g = net->g;
-    // through conv k at level l: dY (post-ReLU grad) given, y = its output; writes dX
-    auto cvb = [&](int k, const float* in, const float* y, float* dy, float* dx, int l) -> int {
+    auto bias = [&](int k) { return g + net->conv[k].off_b; };
+    // weight gradient and data gradient (dx may be NULL) of conv k at level l
+    // from the masked gradient dyk of its output
+    auto cvb = [&](int k, const float* a, const float* b, int ca, int cb, const float* dyk, float* dx, int l) -> int {
         const Conv& c = net->conv[k];
         const int h = H >> l, w = W >> l;
-        const long long P = (long long)N * h * w;
-        NK(relu_bwd(y, dy, P * c.cout, s));
-        NK(conv3x3_wgrad(in, dy, g + c.off_w, N, h, w, c.cin, c.cout, s));
-        NK(bias_grad(dy, g + c.off_b, P, c.cout, s));
-        if (dx) NK(conv3x3_fwd(dy, c.wt, nullptr, dx, N, h, w, c.cout, c.cin, 0, s));
+        NK(conv3x3_wgrad_src(a, b, ca, cb, dyk, g + c.off_w, N, h, w, c.cout, s));
+        if (dx) NK(conv3x3_fwd(dyk, c.wt, nullptr, dx, N, h, w, c.cout, c.cin, 0, s));
         return LBPF_OK;
     };
     int rc;
-    NK(gate(net->xin, kInPad, net->g_out, P0, s));  // the gate is linear in the output
-    NK(conv1x1_bwd(net->top(), net->g_out, net->p + net->off_hw, net->ga[0], g + net->off_hw, g + net->off_hb, P0,
-                   net->ch(0), kOut, s));
     int k = (int)net->conv.size();
-    for (int l = 0; l + 1 < lv; ++l) {  // decoder: the gradient of d[l] is in ga[l]
+    NK(head_bwd(net->top(), dy, net->p + net->off_hw, net->xin, kInPad, net->ga[0], g + net->off_hw, g + net->off_hb,
+                bias(k - 1), P0, net->ch(0), s));
+    for (int l = 0; l + 1 < lv; ++l) {  // decoder: the masked gradient of d[l] is in ga[l]
         k -= 2;
-        if ((rc = cvb(k + 1, net->da[l], net->d[l], net->ga[l], net->gb[l], l))) return rc;
-        if ((rc = cvb(k, net->u[l], net->da[l], net->gb[l], net->ga[l], l))) return rc;
-        // u[l] = [up(level l + 1 output), e[l]]
-        NK(upcat_bwd(net->ga[l], net->ga[l + 1], net->gskip[l], N, H >> l, W >> l, net->ch(l + 1), net->ch(l), s));
-    }
-    for (int l = lv - 1; l >= 0; --l) {  // encoder: the gradient of e[l] is in ga[l]
-        k -= 2;
+        const int c = net->ch(l), h = H >> l, w = W >> l;
         const long long Pl = P0 >> (2 * l);
-        if (l + 1 < lv) NK(add_inplace(net->ga[l], net->gskip[l], Pl * net->ch(l), s));
-        if ((rc = cvb(k + 1, net->ea[l], net->e[l], net->ga[l], net->gb[l], l))) return rc;
-        if ((rc = cvb(k, l > 0 ? net->pl[l] : net->xin, net->ea[l], net->gb[l], l > 0 ? net->ga[l] : nullptr, l)))
-            return rc;
-        if (l > 0) NK(pool_bwd(net->ga[l], net->ga[l - 1], N, H >> (l - 1), W >> (l - 1), net->ch(l - 1), s));
+        if ((rc = cvb(k + 1, net->da[l], nullptr, c, 0, net->ga[l], net->gb[l], l))) return rc;
+        NK(act_bwd(net->da[l], net->gb[l], bias(k), Pl, c, s));
+        // gradient of [up(below), e[l]] into ga[l]; its e[l] part stays there
+        // until the encoder reads it
+        if ((rc = cvb(k, net->below(l), net->e[l], net->ch(l + 1), c, net->gb[l], net->ga[l], l))) return rc;
+        NK(act_bwd_up(net->below(l), net->ga[l], net->ga[l + 1], bias(l + 2 < lv ? k - 1 : 2 * lv - 1), N, h / 2, w / 2,
+                      net->ch(l + 1), net->ch(l + 1) + c, s));
+    }
+    for (int l = lv - 1; l >= 0; --l) {  // encoder
+        k -= 2;
+        const int c = net->ch(l), h = H >> l, w = W >> l;
+        const long long Pl = P0 >> (2 * l);
+        float *a = net->ga[l], *b = net->gb[l];
+        if (l + 1 < lv) {  // gradient of e[l]: pooled from level l + 1 (gb[l + 1]) plus the skip's (ga[l])
+            NK(act_bwd_pool(net->e[l], net->gb[l + 1], net->ga[l], net->gb[l], bias(k + 1), N, h, w, c,
+                            net->ch(l + 1) + c, net->ch(l + 1), s));
+            std::swap(a, b);
+        }
+        // the masked gradient of e[l] is in a
+        if ((rc = cvb(k + 1, net->ea[l], nullptr, c, 0, a, b, l))) return rc;
+        NK(act_bwd(net->ea[l], b, bias(k), Pl, c, s));
+        const int cin = net->conv[k].cin;
+        if ((rc = cvb(k, l > 0 ? net->pl[l] : net->xin, nullptr, cin, 0, b, l > 0 ? a : nullptr, l))) return rc;
+        if (l > 0 && a != net->gb[l]) std::swap(net->ga[l], net->gb[l]);  // level l - 1 reads gb[l]
     }
     return LBPF_OK;
 }
@@ -357,21 +368,14 @@ int backward(lbpf_net* net)
 extern "C" int lbpf_net_forward(lbpf_net* net, const float* x, float* y)
 {
     if (!net || !x) return LBPF_EINVAL;
-    int rc = forward(net, x);
-    if (rc) return rc;
-    if (y)
-        NK(cudaMemcpyAsync(y, net->out, sizeof(float) * (size_t)net->N * net->H * net->W * kOut,
-                           cudaMemcpyDeviceToDevice, net->stream));
-    return LBPF_OK;
+    return forward(net, x, y);
 }
 
 extern "C" int lbpf_net_backward(lbpf_net* net, const float* dy)
 {
     if (!net || !dy) return LBPF_EINVAL;
     NK(cudaMemsetAsync(net->g, 0, sizeof(float) * net->n_params, net->stream));
-    NK(cudaMemcpyAsync(net->g_out, dy, sizeof(float) * (size_t)net->N * net->H * net->W * kOut,
-                       cudaMemcpyDeviceToDevice, net->stream));
-    return backward(net);
+    return backward(net, dy);
 }
 
 extern "C" int lbpf_net_set_loss_weight(lbpf_net* net, float alpha)
@@ -384,13 +388,13 @@ extern "C" int lbpf_net_set_loss_weight(lbpf_net* net, float alpha)
 extern "C" int lbpf_net_train_step(lbpf_net* net, const float* x, const float* target, float lr, double* loss)
 {
     if (!net || !x || !target) return LBPF_EINVAL;
-    int rc = forward(net, x);
+    int rc = forward(net, x, nullptr);
     if (rc) return rc;
     const long long n = (long long)net->N * net->H * net->W * kOut;
     NK(cudaMemsetAsync(net->d_loss, 0, sizeof(double), net->stream));
     NK(mse(net->out, target, x, kIn, kOut, net->loss_alpha, net->g_out, net->d_loss, n, net->stream));
     NK(cudaMemsetAsync(net->g, 0, sizeof(float) * net->n_params, net->stream));
-    if ((rc = backward(net))) return rc;
+    if ((rc = backward(net, net->g_out))) return rc;
     net->adam_t += 1;
     NK(adam(net->p, net->g, net->m, net->v, nullptr, net->n_params, lr, 0.9f, 0.999f, 1e-8f, net->adam_t, net->stream));
     if ((rc = refresh_bf16(net))) return rc;
