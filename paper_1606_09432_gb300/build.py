@@ -22,7 +22,7 @@ SOURCES = ["lbpf_api.cu", "lbpf_fields.cu", "lbpf_launchers.cu", "lbpf_static.cu
 # (object name, source, extra flags): one lattice object per pair and precision
 LATTICE_OBJECTS = [(f"lbpf_lattice_l{lat}_p{prec}", "lbpf_lattice.cu", [f"-DLBPF_LAT={lat}", f"-DLBPF_PREC={prec}"])
                    for lat in range(4) for prec in range(5)]
-HEADERS = ["lbpf_internal.cuh", "step_kernel.cuh", "staged_kernel.cuh", "vec_kernel.cuh", "aux_kernels.cuh", "lbpf_nn.cuh"]
+HEADERS = ["lbpf_internal.cuh", "step_kernel.cuh", "staged_kernel.cuh", "vec_kernel.cuh", "tile_kernel.cuh", "aux_kernels.cuh", "lbpf_nn.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"] + ARCH
 

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "staged_kernel.cuh"
+#include "tile_kernel.cuh"
 #include "vec_kernel.cuh"
 
 namespace lbpf {
@@ -21,10 +22,17 @@ struct SiteNb {
 __device__ __forceinline__ SiteNb site_nb(const DomainDev& d, long long s, int& x, int& y, int& z)
 {
     const long long nxy = (long long)d.nx * d.ny;
-    z = (int)(s / nxy);
-    const long long r = s - (long long)z * nxy;
-    y = (int)(r / d.nx);
-    x = (int)(r - (long long)y * d.nx);
+    if (d.n < (1LL << 31)) {  // 32-bit divisions (a third of the 64-bit ones' instructions)
+        const uint32_t t = (uint32_t)s, q = t / (uint32_t)d.nx;
+        x = (int)(t - q * (uint32_t)d.nx);
+        z = (int)(q / (uint32_t)d.ny);
+        y = (int)(q - (uint32_t)z * (uint32_t)d.ny);
+    } else {
+        z = (int)(s / nxy);
+        const long long r = s - (long long)z * nxy;
+        y = (int)(r / d.nx);
+        x = (int)(r - (long long)y * d.nx);
+    }
     // periodic wrap, or reflection at a wall (the image of the node beyond
     // a wall is the node on the other side of it)
     const bool wx = d.bc & LBPF_BC_WALL_X, wy = d.bc & LBPF_BC_WALL_Y, wz = d.bc & LBPF_BC_WALL_Z;
@@ -406,6 +414,19 @@ struct LauncherImpl {
             return cudaErrorNotSupported;
         }
     }
+    // the one-tile step: 2D
+    static cudaError_t tile_step(int walls, const StepArgs& a, cudaStream_t s)
+    {
+        if constexpr (PL::D == 2) {
+            if (walls)
+                tile_step_kernel<PL, UL, S, true><<<a.n_items, kTileRX * kTileRY, 0, s>>>(a);
+            else
+                tile_step_kernel<PL, UL, S, false><<<a.n_items, kTileRX * kTileRY, 0, s>>>(a);
+            return cudaGetLastError();
+        } else {
+            return cudaErrorNotSupported;
+        }
+    }
     static int vec_blocks_per_sm(int walls)
     {
         int nb = 0;
@@ -473,6 +494,7 @@ struct LauncherImpl {
                                     kStaged ? &step_staged : nullptr,      &staged_blocks_per_sm,
                                     kVec ? &heat_vec : nullptr,            &phi_vec,
                                     &vec_blocks_per_sm,
+                                    PL::D == 2 ? &tile_step : nullptr,
                                     &heat_sync, &equilibrate,   &read_u,   &read_pop,
                                     &read_as,  PL::Q,          UL::Q,     PL::D};
         return &L;

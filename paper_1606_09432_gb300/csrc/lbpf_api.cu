@@ -46,6 +46,7 @@ struct lbpf_ctx {
     int tile_v = 0, seg_len = 0, sms = 1;
     bool staged = false;  // step kernel with bulk-copy staging (staged_kernel.cuh)
     bool vec = false;     // vector step: two launches, four sites a thread (vec_kernel.cuh)
+    bool tile = false;    // one-tile step (tile_kernel.cuh)
     int kind = 0;         // step kernel kind: kStepWalls (some domain has walls) | kStepAdvect
     // graphs of kGraphSteps steady-state launches, keyed by (cur, fcur, acur)
     cudaGraphExec_t graphs[8] = {};
@@ -149,7 +150,13 @@ static int default_segment(const lbpf_ctx* c, int v)
     // (64^3: 53.6 us a step in segments, 28.2 balanced), above they do and share
     // their halo rims better (352^3: 1597 us in segments, 1681 balanced)
     if (c->vec && (double)column_units(c, v) < 64.0 * G) return 0;
-    int L = (int)std::lround(std::sqrt(5.0 * (double)column_units(c, v) / G));
+    // small contexts: one wave of the shortest items that all blocks hold at
+    // once, since a step then costs the latency of one item (us a step, 8 planes
+    // an item / this rule: 2D 128^2 22.1 / 9.1, 256^2 25.8 / 12.3, 512^2 26.6 /
+    // 20.4; 3D 64^3 FP32 37.3 / 27.3)
+    const double units = (double)column_units(c, v);
+    if (units <= 8.0 * G) return (int)std::ceil(units / G);
+    int L = (int)std::lround(std::sqrt(5.0 * units / G));
     return L < 8 ? 8 : (L > 256 ? 256 : L);
 }
 
@@ -196,10 +203,16 @@ static void balanced_items(const lbpf_ctx* c, int wx, int wy, long long G, std::
 // seg: planes per item, 0 the balanced partition (vector step).
 static int set_schedule(lbpf_ctx* c, int v, int seg)
 {
+    if (seg > 0) c->tile = false;  // a segment length asks for the march
     const int wx = c->vec ? kVecTX : tile_x(c->dim, v), wy = c->vec ? kVecTY : tile_y(c->dim, v);
     const long long G = (long long)blocks_per_sm(c, v) * c->sms;
     std::vector<WorkItem> items;
-    if (seg == 0) {
+    if (c->tile) {
+        for (int k = 0; k < c->n_domains; ++k)
+            for (int y = 0; y < c->dd[k].ny; y += kTileRY - 2)
+                for (int x = 0; x < c->dd[k].nx; x += kTileRX - 2) items.push_back(WorkItem{k, x, y, 0, c->dd[k].ny, 0});
+        seg = kTileRY - 2;
+    } else if (seg == 0) {
         balanced_items(c, wx, wy, G, items);
         seg = (int)(column_units(c, v) / (long long)items.size());
     } else
@@ -234,7 +247,7 @@ static int set_schedule(lbpf_ctx* c, int v, int seg)
     CK(cudaMemcpyAsync(c->d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->n_items = (int)items.size();
-    c->n_blocks = (int)(G < c->n_items ? G : c->n_items);
+    c->n_blocks = c->tile ? c->n_items : (int)(G < c->n_items ? G : c->n_items);
     c->tile_v = v;
     c->seg_len = seg;
     for (cudaGraphExec_t& g : c->graphs)
@@ -243,6 +256,21 @@ static int set_schedule(lbpf_ctx* c, int v, int seg)
             g = nullptr;
         }
     return LBPF_OK;
+}
+
+// Whether the one-tile step (tile_kernel.cuh) replaces the march: 2D, no
+// advection, few sites.  us a step, march (shortest items) / tile: FP32 64^2 8.2
+// / 3.8, 128^2 9.2 / 4.0, 256^2 12.3 / 6.1, 512^2 20.4 / 14.3, 768^2 31.0 / 26.5,
+// 1024^2 46.9 / 49.5, 2048^2 155 / 178; FP16 512^2 22.4 / 16.1; FP64 with walls
+// (bound by FP64 arithmetic) 128^2 26 / 17, 800^2 272 / 225, 1200^2 523 / 493,
+// 2000^2 1201 / 1341.
+static bool tile_applies(const lbpf_ctx* c)
+{
+    const char *kenv = getenv("LBPF_KERNEL"), *tenv = getenv("LBPF_AUTOTUNE");
+    if (!c->L->tile_step || (c->kind & kStepAdvect) || (kenv && *kenv) || (tenv && atoi(tenv))) return false;
+    double sites = 0;
+    for (const DomainDev& d : c->dd) sites += (double)d.n;
+    return sites <= (c->rsize == 8 ? 2.0e6 : 7.0e5);
 }
 
 static std::string tune_key(const lbpf_ctx* c)
@@ -273,10 +301,26 @@ static std::string tune_cache_path()
     return std::string(home ? home : "/tmp") + "/.cache/lbpf_tune.txt";
 }
 
+static StepArgs step_args(const lbpf_ctx* c)
+{
+    StepArgs a;
+    a.doms = c->d_dd;
+    a.items = c->d_items;
+    a.n_items = c->n_items;
+    a.counters = c->d_counters;
+    a.cur = c->cur;
+    a.fcur = c->fcur;
+    a.acur = c->acur;
+    a.collide = c->lagged;
+    a.grad = c->grad;
+    return a;
+}
+
 // The launches of one time step.
 static cudaError_t issue_step(lbpf_ctx* c, const StepArgs& a)
 {
     if (c->staged) return c->L->step_staged(a, c->n_blocks, c->stream);
+    if (c->tile) return c->L->tile_step(c->kind & kStepWalls, a, c->stream);
     if (!c->vec) return c->L->step(c->tile_v, c->kind, a, c->n_blocks, c->stream);
     for (int k = 0; k < c->n_domains; ++k) {
         const cudaError_t e = c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream);
@@ -295,16 +339,8 @@ static double time_schedule(lbpf_ctx* c, int launches)
         cudaGetLastError();
         return 1e30;
     }
-    StepArgs a;
-    a.doms = c->d_dd;
-    a.items = c->d_items;
-    a.n_items = c->n_items;
-    a.counters = c->d_counters;
-    a.cur = c->cur;
-    a.fcur = c->fcur;
-    a.acur = c->acur;
+    StepArgs a = step_args(c);
     a.collide = 1;
-    a.grad = c->grad;
     double best = 1e30;
     for (int k = 0; k < launches + 2; ++k) {
         if (cudaMemsetAsync(c->d_counters + c->cur, 0, sizeof(int), c->stream) != cudaSuccess) break;
@@ -327,6 +363,10 @@ static double time_schedule(lbpf_ctx* c, int launches)
 // LBPF_AUTOTUNE=1) are then timed at the first step, on the seeded state.
 static int initial_schedule(lbpf_ctx* c)
 {
+    if ((c->tile = tile_applies(c))) {
+        c->tuned = "rule";
+        return set_schedule(c, 0, 0);
+    }
     const std::string key = tune_key(c);
     if (FILE* f = fopen(tune_cache_path().c_str(), "r")) {
         char k[200];
@@ -601,7 +641,15 @@ static int device_error(lbpf_ctx* c)
 static int sync_state(lbpf_ctx* c)
 {
     if (!c->lagged) return LBPF_OK;
-    for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_sync(c->d_dd + k, c->cur, c->fcur, c->acur, c->stream));
+    if (c->vec && c->precision != LBPF_FP32_FP16DEV_SR) {
+        // the vector step's heat launch is this update (it also fills its work
+        // field; the stochastic form rounds differently here)
+        StepArgs a = step_args(c);
+        a.collide = 1;
+        for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream));
+    } else {
+        for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_sync(c->d_dd + k, c->cur, c->fcur, c->acur, c->stream));
+    }
     c->fcur ^= 1;
     if (c->Sg != c->Qg) c->acur ^= 1;
     c->lagged = 0;
@@ -674,16 +722,7 @@ extern "C" int lbpf_write_fields(lbpf_ctx* c, int domain, const void* phi, const
 // One launch of the fused step on the context's stream.
 static int launch_step(lbpf_ctx* c)
 {
-    StepArgs a;
-    a.doms = c->d_dd;
-    a.items = c->d_items;
-    a.n_items = c->n_items;
-    a.counters = c->d_counters;
-    a.cur = c->cur;
-    a.fcur = c->fcur;
-    a.acur = c->acur;
-    a.collide = c->lagged;
-    a.grad = c->grad;
+    const StepArgs a = step_args(c);
     CK(issue_step(c, a));
     c->cur ^= 1;
     c->acur ^= 1;

@@ -251,6 +251,8 @@ constexpr int TX = 32;
 constexpr int kNumTileVariants = 2;
 constexpr int kTileRows[kNumTileVariants] = {8, 16};
 constexpr int kStripX[kNumTileVariants] = {128, 256};
+// Region of a block of the one-tile step of small 2D domains (tile_kernel.cuh).
+constexpr int kTileRX = 32, kTileRY = 8;
 // Tile of the vector step's phase-field launch (vec_kernel.cuh).
 constexpr int kVecTX = 64, kVecTY = 12;
 constexpr int tile_x(int dim, int v) { return dim == 3 ? TX : kStripX[v]; }
@@ -443,6 +445,9 @@ struct Launchers {
     cudaError_t (*heat_vec)(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s);
     cudaError_t (*phi_vec)(int walls, const StepArgs& a, int n_blocks, cudaStream_t s);
     int (*vec_blocks_per_sm)(int walls);
+    // The one-tile step (tile_kernel.cuh) over n_items tiles of 30 x 6 sites;
+    // nullptr in 3D.
+    cudaError_t (*tile_step)(int walls, const StepArgs& a, cudaStream_t s);
     // Heat step alone, lagged -> synced state of one domain (f^{n-1}, aux^{n-1},
     // phi^n -> f^n [+ aux^n]).
     cudaError_t (*heat_sync)(const DomainDev* d, int cur, int fcur, int acur, cudaStream_t s);
