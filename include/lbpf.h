@@ -319,18 +319,17 @@ typedef enum {
     LBPF_Q_TILE_ROWS = 6,      /* tile variant of the step kernel (autotuned): 8, 16 */
     LBPF_Q_SEGMENT = 7,        /* z-planes (3D) or y-rows (2D) per work item          */
     LBPF_Q_BLOCKS = 8,         /* resident blocks of the persistent step launch       */
-    LBPF_Q_KERNEL = 9          /* step kernel: 0 the library's choice (3D contexts with
-                                  16-bit deviation storage whose domains have one crystal,
-                                  no velocity, nx a multiple of 4, >= 8 and not 4 above a
-                                  multiple of 64: two launches a step with four sites a
-                                  thread; otherwise one launch, global-memory pulls), 1
-                                  staged (rows brought to shared memory by asynchronous
-                                  copies; chosen by the environment variable
-                                  LBPF_KERNEL=staged at lbpf_create for 3D D3Q15/D3Q19
-                                  domains with 16-bit deviation storage, nx a multiple of
-                                  8 and >= 64, one crystal; slower on GB300).
-                                  LBPF_KERNEL=generic keeps the one-launch kernel.  Same
-                                  results bit for bit in every case                 */
+    LBPF_Q_KERNEL = 9          /* step kernel: 0 the library's choice, 1 staged.  The choice
+                                  (same results bit for bit): a march over tiles in one
+                                  launch; in 2D with few sites one launch with a block per
+                                  tile; in 3D with 16-bit deviation storage (one crystal, no
+                                  velocity, rows that fill 64-site segments) two launches
+                                  with four sites a thread.  The environment variable
+                                  LBPF_KERNEL at lbpf_create forces generic (the march),
+                                  vector (the last, wherever it can run) or staged (rows
+                                  brought to shared memory by asynchronous copies: 3D
+                                  D3Q15/D3Q19 domains with 16-bit deviation storage, nx a
+                                  multiple of 8 and >= 64, one crystal; slower on GB300) */
 } lbpf_query_t;
 
 /* Override the work schedule of the step kernel.  Normally lbpf_create takes

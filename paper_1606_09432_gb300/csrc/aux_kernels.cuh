@@ -21,17 +21,17 @@ struct SiteNb {
 
 __device__ __forceinline__ SiteNb site_nb(const DomainDev& d, long long s, int& x, int& y, int& z)
 {
-    const long long nxy = (long long)d.nx * d.ny;
+    const long long nxy = (long long)d.px * d.ny;
     if (d.n < (1LL << 31)) {  // 32-bit divisions (a third of the 64-bit ones' instructions)
-        const uint32_t t = (uint32_t)s, q = t / (uint32_t)d.nx;
-        x = (int)(t - q * (uint32_t)d.nx);
+        const uint32_t t = (uint32_t)s, q = t / (uint32_t)d.px;
+        x = (int)(t - q * (uint32_t)d.px);
         z = (int)(q / (uint32_t)d.ny);
         y = (int)(q - (uint32_t)z * (uint32_t)d.ny);
     } else {
         z = (int)(s / nxy);
         const long long r = s - (long long)z * nxy;
-        y = (int)(r / d.nx);
-        x = (int)(r - (long long)y * d.nx);
+        y = (int)(r / d.px);
+        x = (int)(r - (long long)y * d.px);
     }
     // periodic wrap, or reflection at a wall (the image of the node beyond
     // a wall is the node on the other side of it)
@@ -39,11 +39,19 @@ __device__ __forceinline__ SiteNb site_nb(const DomainDev& d, long long s, int& 
     SiteNb nb;
     nb.oxm = (x == 0) ? (wx ? 1 : d.nx - 1) : -1;
     nb.oxp = (x == d.nx - 1) ? (wx ? -1 : -(d.nx - 1)) : 1;
-    nb.oym = (long long)((y == 0) ? (wy ? 1 : d.ny - 1) : -1) * d.nx;
-    nb.oyp = (long long)((y == d.ny - 1) ? (wy ? -1 : -(d.ny - 1)) : 1) * d.nx;
+    nb.oym = (long long)((y == 0) ? (wy ? 1 : d.ny - 1) : -1) * d.px;
+    nb.oyp = (long long)((y == d.ny - 1) ? (wy ? -1 : -(d.ny - 1)) : 1) * d.px;
     nb.ozm = (d.nz == 1) ? 0 : (long long)((z == 0) ? (wz ? 1 : d.nz - 1) : -1) * nxy;
     nb.ozp = (d.nz == 1) ? 0 : (long long)((z == d.nz - 1) ? (wz ? -1 : -(d.nz - 1)) : 1) * nxy;
     return nb;
+}
+
+// Index of array element s among the sites of a dense field, -1 for row padding.
+__device__ __forceinline__ long long dense_index(const DomainDev& d, long long s)
+{
+    if (d.px == d.nx) return s;
+    const long long row = s / d.px, x = s - row * d.px;
+    return x < d.nx ? row * d.nx + x : -1;
 }
 
 // Gradient of phi at site s in lattice units (Sec. 4.2), global-memory stencil.
@@ -102,6 +110,7 @@ __global__ void equilibrate_kernel(const DomainDev* dp, int cur, int fcur, int a
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         const SiteNb nb = site_nb(d, s, x, y, z);
+        if (x >= d.nx) continue;
         R Gx, Gy, Gz;
         site_gradient<PL, R>(phi, s, nb, grad, Gx, Gy, Gz);
         const R ph = phi[s];
@@ -157,6 +166,7 @@ __global__ void heat_sync_kernel(const DomainDev* dp, int cur, int fcur, int acu
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         const SiteNb nb = site_nb(d, s, x, y, z);
+        if (x >= d.nx) continue;
         R fv[UL::Q];
         R u = 0;
         R d0 = 0;
@@ -213,13 +223,15 @@ __global__ void read_u_kernel(const DomainDev* dp, int cur, int fcur, int acur, 
     const R* aux = static_cast<const R*>(d.aux[acur]);
     const R* phi = static_cast<const R*>(d.phi[cur]);
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
+        const long long o = dense_index(d, s);
+        if (o < 0) continue;
         if (!S::dev) {
             R u = 0;
 #pragma unroll
             for (int j = 0; j < UL::Q; ++j) u += to_real(f[(long long)j * n + s]);
-            out[s] = u;
+            out[o] = u;
         } else {
-            out[s] = aux[s] + R(0.5) * phi[s];
+            out[o] = aux[s] + R(0.5) * phi[s];
         }
     }
 }
@@ -238,17 +250,19 @@ __global__ void read_pop_kernel(const DomainDev* dp, int which, int i, int cur, 
     const R* phi = static_cast<const R*>(d.phi[cur]);
     const R* aux = static_cast<const R*>(d.aux[acur]);
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
+        const long long o = dense_index(d, s);
+        if (o < 0) continue;
         if (!S::dev) {
-            out[s] = to_real(p[(long long)i * n + s]);
+            out[o] = to_real(p[(long long)i * n + s]);
         } else {
             const R m = which == 0 ? phi[s] : aux[s] + R(0.5) * phi[s];
             if (i > 0) {
                 const R wi = which == 0 ? R(PL::w(i)) : R(UL::w(i));
-                out[s] = wi * m + to_real(p[(long long)(i - 1) * n + s]);
+                out[o] = wi * m + to_real(p[(long long)(i - 1) * n + s]);
             } else {
                 R d0 = 0;
                 for (int j = 1; j < Q; ++j) d0 -= to_real(p[(long long)(j - 1) * n + s]);
-                out[s] = (which == 0 ? R(PL::w(0)) : R(UL::w(0))) * m + d0;
+                out[o] = (which == 0 ? R(PL::w(0)) : R(UL::w(0))) * m + d0;
             }
         }
     }
@@ -268,6 +282,8 @@ __global__ void read_as_kernel(const DomainDev* dp, int cur, int grad, typename 
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < d.n; s += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         const SiteNb nb = site_nb(d, s, x, y, z);
+        const long long o = dense_index(d, s);
+        if (o < 0) continue;
         const int cryst = d.use_index ? (int)I[s] : 1;
         R a = 1, Nx, Ny, Nz;
         if (cryst > 0 && cryst <= d.n_crystals) {
@@ -275,7 +291,7 @@ __global__ void read_as_kernel(const DomainDev* dp, int cur, int grad, typename 
             site_gradient<PL, R>(phi, s, nb, grad, Gx, Gy, Gz);
             anisotropy<R, PL::D>(d.cr[cryst - 1], Gx, Gy, Gz, a, Nx, Ny, Nz);
         }
-        out[s] = a;
+        out[o] = a;
     }
 }
 
@@ -389,7 +405,7 @@ struct LauncherImpl {
     static cudaError_t heat_vec(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s)
     {
         if constexpr (kVec) {
-            const int gx = (h.nx / 4 + kHeatX - 1) / kHeatX, gy = (h.ny + kHeatY - 1) / kHeatY;
+            const int gx = (h.px / 4 + kHeatX - 1) / kHeatX, gy = (h.ny + kHeatY - 1) / kHeatY;
             int zlen = 16;
             while (zlen > 1 && (long long)gx * gy * ((h.nz + zlen - 1) / zlen) < 152 * 8) zlen /= 2;
             const dim3 grid(gx, gy, (h.nz + zlen - 1) / zlen), block(kHeatX, kHeatY);

@@ -427,19 +427,28 @@ static int autotune(lbpf_ctx* c)
     return set_schedule(c, best_v, best_seg);
 }
 
-// Whether every domain takes the vector step: 3D in single precision, one
-// crystal, no advection, rows of whole 4-site vectors, and no row segment of
-// a single vector (its two ends need different lanes).
+// Whether the context takes the vector step.  It can where every domain is 3D
+// with 16-bit deviations, one crystal, no advection and site indices in 31 bits;
+// it pays where its 64-site row segments are at least 0.6 full and there is work
+// for more than a wave of blocks (FP16, us a step, one launch / vector: 32^3 14.5
+// / 25.1, 64^3 29.7 / 29.1, 96^3 56.0 / 52.8, 128^3 115 / 85, 207x174x190 397 /
+// 296, 351^3 walls 2286 / 1679; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201).
+// LBPF_KERNEL: "vector" wherever it can, any other value never.
 static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_domains)
 {
-    if (!L->heat_vec) return false;
+    const char* kenv = getenv("LBPF_KERNEL");
+    const bool forced = kenv && strcmp(kenv, "vector") == 0;
+    if (!L->heat_vec || (kenv && *kenv && !forced)) return false;
+    double sites = 0, slots = 0;
     for (int k = 0; k < n_domains; ++k) {
         const lbpf_domain& d = domains[k];
-        if (d.nx % 4 || d.nx < 8 || d.nx % kVecTX == 4 || (long long)d.nx * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 || d.adv[0] != 0.0 || d.adv[1] != 0.0 ||
+        if (d.nx < 8 || (long long)((d.nx + 3) / 4 * 4) * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 || d.adv[0] != 0.0 || d.adv[1] != 0.0 ||
             d.adv[2] != 0.0)
             return false;
+        sites += (double)d.nx * d.ny * d.nz;
+        slots += (double)((d.nx + kVecTX - 1) / kVecTX * kVecTX) * d.ny * d.nz;
     }
-    return true;
+    return forced || (sites >= 2e5 && sites >= 0.6 * slots);
 }
 
 extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattice, int grad, int precision,
@@ -517,7 +526,7 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
     const double e2u = (dim == 2) ? 1.0 / 3.0 : 1.0 / 4.0;
 
     const char* kenv = getenv("LBPF_KERNEL");
-    c->vec = vec_applies(L, domains, n_domains) && !(kenv && *kenv);
+    c->vec = vec_applies(L, domains, n_domains);
 
     int rc = LBPF_OK;
     long long max_n = 0;
@@ -531,7 +540,8 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
         h.nz = d.nz;
         h.bc = d.bc;
         if (d.bc) c->kind |= kStepWalls;
-        h.n = (long long)d.nx * d.ny * d.nz;
+        h.px = c->vec ? (d.nx + 3) / 4 * 4 : d.nx;  // rows of whole vectors
+        h.n = (long long)h.px * d.ny * d.nz;
         max_n = h.n > max_n ? h.n : max_n;
         // D_phi = (W0^2/tau0)(dt/dx^2), Eq. (LBE_RelaxationTime)
         h.Dphi = (d.W0 * d.W0 / d.tau0) * (d.dt / (d.dx * d.dx));
@@ -692,6 +702,18 @@ extern "C" int lbpf_seed(lbpf_ctx* c, int domain, const lbpf_seed_t* seeds, int 
     return LBPF_OK;
 }
 
+// Sites of a domain (its arrays may hold row padding besides).
+static long long sites_of(const DomainDev& h) { return (long long)h.nx * h.ny * h.nz; }
+
+// A field of the arithmetic type between arrays of row pitches dp and sp (elements).
+static cudaError_t copy_rows(lbpf_ctx* c, const DomainDev& h, void* dst, int dp, const void* src, int sp,
+                             cudaMemcpyKind kind)
+{
+    const size_t row = (size_t)h.nx * c->rsize, rows = (size_t)h.ny * h.nz;
+    if (dp == sp) return cudaMemcpyAsync(dst, src, row * rows, kind, c->stream);
+    return cudaMemcpy2DAsync(dst, (size_t)dp * c->rsize, src, (size_t)sp * c->rsize, row, rows, kind, c->stream);
+}
+
 extern "C" int lbpf_write_fields(lbpf_ctx* c, int domain, const void* phi, const void* u, const int* index,
                                  int on_device)
 {
@@ -700,10 +722,9 @@ extern "C" int lbpf_write_fields(lbpf_ctx* c, int domain, const void* phi, const
     if (!phi || !u) return fail(c, LBPF_EINVAL, "lbpf_write_fields: phi and u are required");
     if ((rc = sync_state(c))) return rc;
     const DomainDev& h = c->dd[domain];
-    const size_t bytes = (size_t)h.n * c->rsize;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(cudaMemcpyAsync(h.phi[c->cur], phi, bytes, kind, c->stream));
-    CK(cudaMemcpyAsync(h.aux[c->acur], u, bytes, kind, c->stream));
+    CK(copy_rows(c, h, h.phi[c->cur], h.px, phi, h.nx, kind));
+    CK(copy_rows(c, h, h.aux[c->acur], h.px, u, h.nx, kind));
     if (h.use_index) {
         if (index) {
             CK(cudaMemcpyAsync(c->scratch, index, sizeof(int) * h.n, kind, c->stream));
@@ -812,7 +833,7 @@ extern "C" int lbpf_read_fields(lbpf_ctx* c, int domain, unsigned mask, void* ou
     const DomainDev& h = c->dd[domain];
     size_t need = 0;
     for (unsigned bit = 1; bit <= LBPF_READ_INDEX; bit <<= 1)
-        if (mask & bit) need += (size_t)h.n * field_esize(c, bit);
+        if (mask & bit) need += (size_t)sites_of(h) * field_esize(c, bit);
     if (out_bytes < need) return fail(c, LBPF_ERANGE, "lbpf_read_fields: need %zu bytes, got %zu", need, out_bytes);
     if (mask & LBPF_READ_U)
         if ((rc = sync_state(c))) return rc;
@@ -820,7 +841,7 @@ extern "C" int lbpf_read_fields(lbpf_ctx* c, int domain, unsigned mask, void* ou
     char* o = static_cast<char*>(out);
     for (unsigned bit = 1; bit <= LBPF_READ_INDEX; bit <<= 1) {
         if (!(mask & bit)) continue;
-        const size_t bytes = (size_t)h.n * field_esize(c, bit);
+        const size_t bytes = (size_t)sites_of(h) * field_esize(c, bit);
         // fields that need a kernel are written in place (device output) or
         // into the context's scratch and copied from there (host output); the
         // copies run in stream order, so the scratch is free again for the
@@ -828,16 +849,16 @@ extern "C" int lbpf_read_fields(lbpf_ctx* c, int domain, unsigned mask, void* ou
         void* dst = out_on_device ? static_cast<void*>(o) : c->scratch;
         switch (bit) {
         case LBPF_READ_PHI:
-            CK(cudaMemcpyAsync(o, h.phi[c->cur], bytes, kind, c->stream));
+            CK(copy_rows(c, h, o, h.nx, h.phi[c->cur], h.px, kind));
             dst = nullptr;
             break;
         case LBPF_READ_U: CK(c->L->read_u(c->d_dd + domain, c->cur, c->fcur, c->acur, dst, c->stream)); break;
         case LBPF_READ_AS: CK(c->L->read_as(c->d_dd + domain, c->cur, c->grad, dst, c->stream)); break;
         case LBPF_READ_INDEX:
             if (h.use_index)
-                CK(launch_index_to_i32(h.I[c->cur], static_cast<int*>(dst), h.n, c->stream));
+                CK(launch_index_to_i32(h.I[c->cur], static_cast<int*>(dst), sites_of(h), c->stream));
             else
-                CK(launch_fill_i32(static_cast<int*>(dst), 1, h.n, c->stream));
+                CK(launch_fill_i32(static_cast<int*>(dst), 1, sites_of(h), c->stream));
             break;
         }
         if (dst && !out_on_device) CK(cudaMemcpyAsync(o, dst, bytes, cudaMemcpyDeviceToHost, c->stream));
@@ -864,7 +885,7 @@ extern "C" int lbpf_read_populations(lbpf_ctx* c, int domain, int which, void* o
     if (!out || (which != 0 && which != 1)) return fail(c, LBPF_EINVAL, "lbpf_read_populations: bad arguments");
     const DomainDev& h = c->dd[domain];
     const int Q = which == 0 ? c->Qg : c->Qu;
-    const size_t bytes = (size_t)Q * h.n * c->rsize, one = (size_t)h.n * c->rsize;
+    const size_t one = (size_t)sites_of(h) * c->rsize, bytes = (size_t)Q * one;
     if (out_bytes < bytes) return fail(c, LBPF_ERANGE, "lbpf_read_populations: need %zu bytes, got %zu", bytes, out_bytes);
     if ((rc = sync_state(c))) return rc;
     // one population at a time, host reads through the context's scratch
@@ -889,9 +910,10 @@ extern "C" int lbpf_measure(lbpf_ctx* c, int domain, int cx, int cy, int cz, dou
     if ((rc = sync_state(c))) return rc;
     CK(c->L->read_u(c->d_dd + domain, c->cur, c->fcur, c->acur, c->scratch, c->stream));
     double* outp = c->red + 3 * kReduceBlocks;
-    CK(launch_reduce(h.phi[c->cur], c->scratch, h.n, c->precision, c->red, outp, c->stream, h.nx, h.ny, h.nz, h.bc,
-                     c->dim));
-    CK(launch_tips(h.phi[c->cur], h.nx, h.ny, h.nz, cx, cy, cz, c->dim, c->precision, outp + 3, c->stream, h.bc));
+    CK(launch_reduce(h.phi[c->cur], c->scratch, sites_of(h), c->precision, c->red, outp, c->stream, h.nx, h.ny, h.nz,
+                     h.bc, c->dim, h.px));
+    CK(launch_tips(h.phi[c->cur], h.nx, h.ny, h.nz, cx, cy, cz, c->dim, c->precision, outp + 3, c->stream, h.bc,
+                   h.px));
     {
         const int slot = (c->hist_last[domain] + 1) % kHistCap;
         CK(launch_hist_append(outp + 3, (double)c->steps * c->in[domain].dt,
@@ -905,7 +927,7 @@ extern "C" int lbpf_measure(lbpf_ctx* c, int domain, int cx, int cy, int cz, dou
     if (tip6)
         for (int k = 0; k < 6; ++k) tip6[k] = hv[3 + k];
     if ((rc = device_error(c))) return rc;
-    if (solid_fraction) *solid_fraction = hv[0] / (double)h.n;
+    if (solid_fraction) *solid_fraction = hv[0] / (double)sites_of(h);
     if (conserved) *conserved = hv[1];
     if (hv[2] > 0) return fail(c, LBPF_ENONFINITE, "lbpf_measure: %.0f non-finite values in phi or u", hv[2]);
     return LBPF_OK;
@@ -937,7 +959,7 @@ extern "C" int lbpf_tip_radius(lbpf_ctx* c, int domain, int cx, int cy, int cz, 
         return fail(c, LBPF_EINVAL, "lbpf_tip_radius: centre outside the domain");
     double* out = c->red + 3 * kReduceBlocks + 15;
     CK(launch_tip_radius(h.phi[c->cur], h.nx, h.ny, h.nz, cx, cy, cz, dir, J, c->dim, c->precision, out, c->stream,
-                         h.bc));
+                         h.bc, h.px));
     CK(cudaMemcpyAsync(rho, out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return LBPF_OK;
@@ -966,7 +988,7 @@ extern "C" int lbpf_query(const lbpf_ctx* c, int what, double* value)
     double v = 0;
     switch (what) {
     case LBPF_Q_SITES:
-        for (const DomainDev& h : c->dd) v += (double)h.n;
+        for (const DomainDev& h : c->dd) v += (double)sites_of(h);
         break;
     case LBPF_Q_STEPS: v = (double)c->steps; break;
     case LBPF_Q_BYTES_PER_SITE: {
@@ -974,8 +996,8 @@ extern "C" int lbpf_query(const lbpf_ctx* c, int what, double* value)
         // the index field when it is used)
         double idx_sites = 0, all_sites = 0;
         for (const DomainDev& h : c->dd) {
-            all_sites += (double)h.n;
-            if (h.use_index) idx_sites += (double)h.n;
+            all_sites += (double)sites_of(h);
+            if (h.use_index) idx_sites += (double)sites_of(h);
         }
         v = 2.0 * (c->Sg + c->Su) * c->ssize + 4.0 * c->rsize + 2.0 * idx_sites / all_sites;
         break;

@@ -22,12 +22,17 @@ __global__ void seed_kernel(const DomainDev* dp, long long n, int cur, int acur,
     R* phi = static_cast<R*>(d.phi[cur]);
     R* aux = static_cast<R*>(d.aux[acur]);
     int8_t* I = d.I[cur];
-    const long long nxy = (long long)d.nx * d.ny;
+    const long long nxy = (long long)d.px * d.ny;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         const int z = (int)(s / nxy);
         const long long r = s - (long long)z * nxy;
-        const int y = (int)(r / d.nx);
-        const int x = (int)(r - (long long)y * d.nx);
+        const int y = (int)(r / d.px);
+        const int x = (int)(r - (long long)y * d.px);
+        if (x >= d.nx) {  // row padding: finite values
+            phi[s] = R(-1);
+            aux[s] = R(u0);
+            continue;
+        }
         double best = -2.0;
         int bestc = 0;
         for (int j = 0; j < ns; ++j) {
@@ -72,12 +77,12 @@ __device__ __forceinline__ double warp_sum(double v)
 // coordinate at a wall: the site lies on a mirror plane (trapezoid rule).
 template <class R>
 __global__ void __launch_bounds__(256) reduce_kernel(const R* __restrict__ phi, const R* __restrict__ u, long long n,
-                                                     double* partial, int nx, int ny, int nz, int bc, int dim)
+                                                     double* partial, int nx, int ny, int nz, int bc, int dim, int px)
 {
     double sf = 0.0, cs = 0.0, bad = 0.0;
     const long long nxy = (long long)nx * ny;
     for (long long s = blockIdx.x * 256LL + threadIdx.x; s < n; s += (long long)gridDim.x * 256) {
-        const double p = (double)phi[s], v = (double)u[s];
+        const double p = (double)phi[px == nx ? s : s / nx * px + s % nx], v = (double)u[s];
         if (!isfinite(p) || !isfinite(v)) {
             bad += 1.0;
             continue;
@@ -124,17 +129,18 @@ __global__ void reduce_finish_kernel(const double* partial, int nblocks, double*
 }
 
 cudaError_t launch_reduce(const void* phi, const void* u, long long n, int precision, double* partial, double* out,
-                          cudaStream_t s, int nx, int ny, int nz, int bc, int dim)
+                          cudaStream_t s, int nx, int ny, int nz, int bc, int dim, int px)
 {
-    if (bc && (long long)nx * ny * nz != n) return cudaErrorInvalidValue;
+    if (px == 0) px = nx;
+    if ((bc || px != nx) && (long long)nx * ny * nz != n) return cudaErrorInvalidValue;
     if (precision == LBPF_FP64)
         reduce_kernel<double><<<kReduceBlocks, 256, 0, s>>>(static_cast<const double*>(phi),
                                                            static_cast<const double*>(u), n, partial, nx, ny, nz, bc,
-                                                           dim);
+                                                           dim, px);
     else
         reduce_kernel<float><<<kReduceBlocks, 256, 0, s>>>(static_cast<const float*>(phi),
                                                           static_cast<const float*>(u), n, partial, nx, ny, nz, bc,
-                                                          dim);
+                                                          dim, px);
     reduce_finish_kernel<<<1, 96, 0, s>>>(partial, kReduceBlocks, out);
     return cudaGetLastError();
 }
@@ -147,7 +153,7 @@ cudaError_t launch_reduce(const void* phi, const void* u, long long n, int preci
 // together; one warp a ray took 16 us for 512 sites.)
 template <class R>
 __global__ void __launch_bounds__(256) tips_kernel(const R* __restrict__ phi, int nx, int ny, int nz, int cx, int cy,
-                                                   int cz, int dim, double* out, int bc)
+                                                   int cz, int dim, double* out, int bc, int px)
 {
     const int w = blockIdx.x, t = threadIdx.x;
     const int axis = w >> 1, sign = (w & 1) ? -1 : 1;
@@ -158,8 +164,8 @@ __global__ void __launch_bounds__(256) tips_kernel(const R* __restrict__ phi, in
     const int nax = axis == 0 ? nx : (axis == 1 ? ny : nz);
     const int cax = axis == 0 ? cx : (axis == 1 ? cy : cz);
     const int len = (bc >> axis) & 1 ? (sign > 0 ? nax - 1 - cax : cax) : nax / 2;
-    const long long step = axis == 0 ? 1 : (axis == 1 ? nx : (long long)nx * ny);
-    const R* ray = phi + ((long long)cz * ny + cy) * nx + cx - cax * step;  // coordinate 0 of the axis
+    const long long step = axis == 0 ? 1 : (axis == 1 ? px : (long long)px * ny);
+    const R* ray = phi + ((long long)cz * ny + cy) * px + cx - cax * step;  // coordinate 0 of the axis
     auto at = [&](int k) -> double {  // |k| <= nax: one wrap
         int v = cax + sign * k;
         v = v < 0 ? v + nax : (v >= nax ? v - nax : v);
@@ -185,12 +191,13 @@ __global__ void __launch_bounds__(256) tips_kernel(const R* __restrict__ phi, in
 }
 
 cudaError_t launch_tips(const void* phi, int nx, int ny, int nz, int cx, int cy, int cz, int dim, int precision,
-                        double* out, cudaStream_t s, int bc)
+                        double* out, cudaStream_t s, int bc, int px)
 {
+    if (px == 0) px = nx;
     if (precision == LBPF_FP64)
-        tips_kernel<double><<<6, 256, 0, s>>>(static_cast<const double*>(phi), nx, ny, nz, cx, cy, cz, dim, out, bc);
+        tips_kernel<double><<<6, 256, 0, s>>>(static_cast<const double*>(phi), nx, ny, nz, cx, cy, cz, dim, out, bc, px);
     else
-        tips_kernel<float><<<6, 256, 0, s>>>(static_cast<const float*>(phi), nx, ny, nz, cx, cy, cz, dim, out, bc);
+        tips_kernel<float><<<6, 256, 0, s>>>(static_cast<const float*>(phi), nx, ny, nz, cx, cy, cz, dim, out, bc, px);
     return cudaGetLastError();
 }
 
@@ -308,7 +315,7 @@ template <class R>
 // Walled axes: transverse offsets beyond a wall are reflected (the mirror
 // image of the crystal) and the ray runs to the wall.
 __global__ void tip_radius_kernel(const R* __restrict__ phi, int nx, int ny, int nz, int cx, int cy, int cz, int dir,
-                                  int J, int dim, double* out, int bc)
+                                  int J, int dim, double* out, int bc, int px)
 {
     __shared__ double xc[32];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -336,7 +343,7 @@ __global__ void tip_radius_kernel(const R* __restrict__ phi, int nx, int ny, int
         auto at = [&](int k) -> double {
             int p[3] = {c[0], c[1], c[2]};
             p[axis] = ((c[axis] + sign * k) % nn[axis] + nn[axis]) % nn[axis];
-            return (double)phi[((long long)p[2] * ny + p[1]) * nx + p[0]];
+            return (double)phi[((long long)p[2] * ny + p[1]) * px + p[0]];
         };
         int best = -1;
         for (int k = l; k < len; k += 32)
@@ -380,15 +387,16 @@ __global__ void tip_radius_kernel(const R* __restrict__ phi, int nx, int ny, int
 }
 
 cudaError_t launch_tip_radius(const void* phi, int nx, int ny, int nz, int cx, int cy, int cz, int dir, int J, int dim,
-                              int precision, double* out, cudaStream_t s, int bc)
+                              int precision, double* out, cudaStream_t s, int bc, int px)
 {
+    if (px == 0) px = nx;
     const int threads = 32 * (2 * J + 1) * (dim - 1);
     if (precision == LBPF_FP64)
         tip_radius_kernel<double><<<1, threads, 0, s>>>(static_cast<const double*>(phi), nx, ny, nz, cx, cy, cz, dir,
-                                                         J, dim, out, bc);
+                                                         J, dim, out, bc, px);
     else
         tip_radius_kernel<float><<<1, threads, 0, s>>>(static_cast<const float*>(phi), nx, ny, nz, cx, cy, cz, dir, J,
-                                                        dim, out, bc);
+                                                        dim, out, bc, px);
     return cudaGetLastError();
 }
 

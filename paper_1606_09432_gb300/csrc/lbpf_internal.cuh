@@ -198,7 +198,12 @@ struct CrystalDev {
 struct DomainDev {
     int nx, ny, nz;
     int bc;             // LBPF_BC_WALL_* bits (0: periodic)
-    long long n;        // sites
+    // Row pitch and elements of one array: px = nx, n = nx ny nz, except where
+    // the vector step applies (vec_kernel.cuh): there rows are padded to whole
+    // four-site vectors (px >= nx; the padding is never read as a site) and n =
+    // px ny nz.  Kernels of contexts without the vector step use nx as pitch.
+    int px;
+    long long n;
     double Dphi;        // (W0^2 / tau0) (dt / dx^2), Eq. (LBE_RelaxationTime)
     double qphi;        // dt / tau0, source factor of Eq. (LBE_Eq_Phase)
     double lambda;      // coupling, Eq. (LBE_SourceTerm)
@@ -479,14 +484,15 @@ cudaError_t launch_seed(const DomainDev* d, long long n, int cur, int acur, int 
 // out[2] = number of non-finite phi or u values; partial[] holds one pair of
 // FP64 partial sums and a count per block (scratch of 3 * kReduceBlocks).
 constexpr int kReduceBlocks = 304;
+// phi: row pitch px (0: nx, dense); u: dense.
 // With walls (bc != 0) the u - phi/2 sum weights nodes on a wall by 1/2 per
 // walled coordinate (they lie on the mirror planes).
 cudaError_t launch_reduce(const void* phi, const void* u, long long n, int precision, double* partial, double* out,
-                          cudaStream_t s, int nx = 0, int ny = 0, int nz = 0, int bc = 0, int dim = 3);
+                          cudaStream_t s, int nx = 0, int ny = 0, int nz = 0, int bc = 0, int dim = 3, int px = 0);
 // Tip crossings along +-x, +-y, +-z from (cx, cy, cz); out[6].  Rays cover
 // half the domain on periodic axes and run to the wall on walled ones.
 cudaError_t launch_tips(const void* phi, int nx, int ny, int nz, int cx, int cy, int cz, int dim, int precision,
-                        double* out, cudaStream_t s, int bc = 0);
+                        double* out, cudaStream_t s, int bc = 0, int px = 0);
 // Measurement history (time, tip6) per domain and the FP64 tip fits.
 cudaError_t launch_hist_append(const double* tips6, double t, double* slot, cudaStream_t s);
 cudaError_t launch_tip_velocity(const double* hist, int cap, int last, int count, int window, double dx, double* out,
@@ -494,7 +500,7 @@ cudaError_t launch_tip_velocity(const double* hist, int cap, int last, int count
 // Tip radius of the tip along dir (0..5) from rays at transverse offsets
 // |j| <= J (J <= 7 in 3D, <= 15 in 2D); out[0].
 cudaError_t launch_tip_radius(const void* phi, int nx, int ny, int nz, int cx, int cy, int cz, int dir, int J, int dim,
-                              int precision, double* out, cudaStream_t s, int bc = 0);
+                              int precision, double* out, cudaStream_t s, int bc = 0, int px = 0);
 // int8 <-> int32 index copies.
 cudaError_t launch_index_to_i32(const int8_t* in, int* out, long long n, cudaStream_t s);
 cudaError_t launch_index_from_i32(const int* in, int8_t* out, long long n, int n_crystals, cudaStream_t s);

@@ -17,8 +17,10 @@
 // and both launches read and write four sites per instruction, which leaves
 // 375 instructions a site for the phase field.  The work field costs 8 of
 // 104 bytes a site.  Measured, us a step (step_kernel / this): D3Q15 FP16
-// 512^3 5289 / 3605, 256^3 718 / 533, 352^3 with walls 2139 / 1597; 256^3
-// D3Q19 838 / 643, D3Q27 1260 / 1088.  Full (FP32) storage measured 2 % slower
+// 512^3 5289 / 3605, 256^3 718 / 533, 351^3 with walls 2286 / 1679, 207 x 174 x
+// 190 397 / 296; 256^3 D3Q19 838 / 643, D3Q27 1260 / 1088.  Rows that are not
+// whole vectors are padded in memory (DomainDev::px); a row's last partial vector
+// is computed whole, what falls into the padding is never read.  Full (FP32) storage measured 2 % slower
 // this way (the vectors in flight need twice the registers) and stays with
 // step_kernel.
 #pragma once
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
     const int x = ((int)blockIdx.x * kHeatX + (int)threadIdx.x) * 4, y = (int)blockIdx.y * kHeatY + (int)threadIdx.y;
     if (x >= nx || y >= ny) return;
     const int z0 = (int)blockIdx.z * zlen, z1 = min(z0 + zlen, nz);
-    const long long n = d.n, nxy = (long long)nx * ny;
+    const long long n = d.n, nxy = (long long)d.px * ny;
     const bool wX = WALLS && (d.bc & LBPF_BC_WALL_X), wY = WALLS && (d.bc & LBPF_BC_WALL_Y),
                wZ = WALLS && (d.bc & LBPF_BC_WALL_Z);
     const T* __restrict__ fc = static_cast<const T*>(d.f[fcur]);
@@ -141,7 +143,8 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
     float* __restrict__ uo = static_cast<float*>(d.u_work);
     const float ieu = (float)d.inv_eta_u, om_u = 1.f - ieu;
     const uint32_t seed = UsesSR<S>::value ? (uint32_t)counters[2 + cur] : 0u;
-    const long long row = (long long)y * nx + x;  // in-plane offset of the vector
+    const long long row = (long long)y * d.px + x;  // in-plane offset of the vector
+    const int ke = min(3, nx - 1 - x);              // the vector's last site (the rest is row padding)
 
     if (!collide) {
         for (int z = z0; z < z1; ++z) {
@@ -160,9 +163,9 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
         return;
     }
 
-    const int xm = wrap_axis<WALLS>(x - 1, nx, wX), xp = wrap_axis<WALLS>(x + 4, nx, wX);
+    const int xm = wrap_axis<WALLS>(x - 1, nx, wX), xp = wrap_axis<WALLS>(x + ke + 1, nx, wX);
     const int ym = wrap_axis<WALLS>(y - 1, ny, wY), yp = wrap_axis<WALLS>(y + 1, ny, wY);
-    const long long rym = (long long)ym * nx + x, ryp = (long long)yp * nx + x, r0 = (long long)y * nx;
+    const long long rym = (long long)ym * d.px + x, ryp = (long long)yp * d.px + x, r0 = (long long)y * d.px;
     auto load_h = [&](long long s, float (&h)[4], float (&ph)[4]) {
         load4(phi + s, ph);
         load4(auxc + s, h);
@@ -209,9 +212,11 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
         float fv[QU][4], u[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float hs[QU] = {hc[k], k > 0 ? hc[k > 0 ? k - 1 : 0] : hxm, hym[k], k < 3 ? hc[k < 3 ? k + 1 : 3] : hxp,
+            const float hs[QU] = {hc[k], k > 0 ? hc[k > 0 ? k - 1 : 0] : hxm, hym[k],
+                                  k == ke ? hxp : hc[k < 3 ? k + 1 : 3],
                                   hyp[k], hm[k], hp[k]};
-            const float pv[QU] = {d0[k], k > 0 ? l1[k > 0 ? k - 1 : 0] : e1, p2[k], k < 3 ? l3[k < 3 ? k + 1 : 3] : e3,
+            const float pv[QU] = {d0[k], k > 0 ? l1[k > 0 ? k - 1 : 0] : e1, p2[k],
+                                  k == ke ? e3 : l3[k < 3 ? k + 1 : 3],
                                   p4[k], p5[k], p6[k]};
             u[k] = 0.f;
 #pragma unroll
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
         uint32_t hh[4] = {0u, 0u, 0u, 0u};
         if constexpr (UsesSR<S>::value) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) hh[k] = sr_hash((uint32_t)(s + k), seed);
+            for (int k = 0; k < 4; ++k) hh[k] = sr_hash((uint32_t)(((long long)z * ny + y) * nx + x + k), seed);
         }
 #pragma unroll
         for (int j = 1; j < QU; ++j) {
@@ -332,7 +337,8 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
 
     const DomainDev& dm = args.doms[it.dom];
     const int nx = dm.nx, ny = dm.ny, nz = dm.nz;
-    const long long n = dm.n, nxy = (long long)nx * ny;
+    const int P = dm.px;  // row pitch
+    const long long n = dm.n, nxy = (long long)P * ny;
     const int x0 = it.x0, y0 = it.y0, z0 = it.z0, z1 = it.z1;
     const int tw = min(kVecTX, nx - x0), th = min(kVecTY, ny - y0);
     const int tid = threadIdx.x;
@@ -359,22 +365,29 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
     auto co_plane = [&](int z) { return s_co + ((z + 3) % 3) * CP; };
 
     // phi plane z (tile + 2 sites) into its ring slot, by threads t0 of nt (a
-    // multiple of 32): 16-byte chunks of the rows, 16 a row, then the four halo
-    // columns
+    // multiple of 32): 16-byte chunks of the rows, 16 a row, then single columns
     auto copy_phi = [&](int z, int t0, int nt) {
         const float* src = phic + (long long)wz(z) * nxy;
         float* dst = phi_plane(z);
-        const int c = t0 & 15, q = t0 & 3, qx = q < 2 ? 2 + q : 4 + tw + (q - 2);
-        if (4 * c < tw)
+        const int c = t0 & 15;
+        if (4 * c + 4 <= tw)
             for (int r = t0 >> 4; r < th + 4; r += nt >> 4) {
-                const float* g = src + ((long long)wy(y0 + r - 2) * nx + x0 + 4 * c);
+                const float* g = src + ((long long)wy(y0 + r - 2) * P + x0 + 4 * c);
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                                  (unsigned)__cvta_generic_to_shared(dst + r * PX + 4 + 4 * c)),
                              "l"(g));
             }
+        // single columns: the two left of the tile, the sites of a row's last
+        // partial vector and the two right of the tile
+        const int sh = tw & 3 ? 3 : 2, q = t0 & ((1 << sh) - 1);
+        const int qx = q < 2 ? 2 + q : 4 + (tw & ~3) + (q - 2);
+        if (qx >= 4 + tw + 2) {
+            asm volatile("cp.async.commit_group;");
+            return;
+        }
         const int gq = wx(x0 + qx - 4);
-        for (int r = t0 >> 2; r < th + 4; r += nt >> 2) {
-            const float* g = src + ((long long)wy(y0 + r - 2) * nx + gq);
+        for (int r = t0 >> sh; r < th + 4; r += nt >> sh) {
+            const float* g = src + ((long long)wy(y0 + r - 2) * P + gq);
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
                              (unsigned)__cvta_generic_to_shared(dst + r * PX + qx)),
                          "l"(g));
@@ -519,22 +532,22 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
     const int lx = tid & (kVecLX - 1);
     const int cr = tid / kVecLX;
     const bool vtask = !helper && V * lx < tw && cr <= th + 1;
-    const long long urow = (long long)wy(y0 + cr - 1) * nx + x0 + V * lx;
+    const long long urow = (long long)wy(y0 + cr - 1) * P + x0 + V * lx;
     auto load_u = [&](int z, float2(&u)[H]) {
         if (vtask) lds_v(uc + (long long)wz(z) * nxy + urow, u);
     };
     // halo columns: helper thread t the site of row t / 2, side t & 1
     static_assert(HN >= 2 * (kVecTY + 2), "one halo column site a helper thread");
     const bool etask = helper && (hl >> 1) < th + 2;
-    const long long erow = (long long)wy(y0 + (hl >> 1) - 1) * nx + wx(hl & 1 ? x0 + tw : x0 - 1);
+    const long long erow = (long long)wy(y0 + (hl >> 1) - 1) * P + wx(hl & 1 ? x0 + tw : x0 - 1);
     auto load_ue = [&](int z) { return etask ? __ldg(uc + (long long)wz(z) * nxy + erow) : 0.f; };
 
     // The populations that output_plane(z) is the first to touch (plane z, or
     // z + 1 for the directions with e_z = -1), requested into L2.
     // Helper thread t takes row t / 2 of the tile with halo rows, its first
     // line or its last (the same where rows are aligned to lines).
-    const long long prow = (long long)wy(y0 + (hl >> 1) - 1) * nx + x0 + (hl & 1 ? tw - 1 : 0);
-    const bool ptask = etask && (!(hl & 1) || nx % 64 != 0);
+    const long long prow = (long long)wy(y0 + (hl >> 1) - 1) * P + x0 + (hl & 1 ? tw - 1 : 0);
+    const bool ptask = etask && (!(hl & 1) || P % 64 != 0);
     auto prefetch_g = [&](int z) {
         if (!ptask) return;
         const T* pa = gc + ((long long)wz(z) * nxy + prow);
@@ -544,19 +557,20 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
             asm volatile("prefetch.global.L2 [%0];" ::"l"((PL::ez(i) < 0 ? pb : pa) + (long long)(i - 1) * n));
     };
     // phi of plane z into L2, ahead of its copy: thread t half of row t / 2
-    const long long frow = (long long)wy(y0 + (hl >> 1) - 1) * nx + min(x0 + (hl & 1) * 32, nx - 1);
+    const long long frow = (long long)wy(y0 + (hl >> 1) - 1) * P + min(x0 + (hl & 1) * 32, nx - 1);
     auto prefetch_phi = [&](int z) {
         if (etask) asm volatile("prefetch.global.L2 [%0];" ::"l"(phic + ((long long)wz(z) * nxy + frow)));
     };
 
     // output geometry
     const int r = cr;            // tile row
-    const int ll = tw / V - 1;   // last lane of the segment
+    const int ll = (tw - 1) / V;   // last lane of the segment
     const bool live = r < th && lx <= ll;
     const bool first = lx == 0, last = lx == ll;
+    const int ke = (tw - 1) & (V - 1);  // the segment's last site in its vector
     // threads without a vector (beyond the tile) read the nearest one
     const int gy = y0 + min(r, th - 1), gx = x0 + V * min(lx, ll);
-    const uint32_t rowm = (uint32_t)wy(gy - 1) * nx + gx, row0 = (uint32_t)gy * nx + gx, rowp = (uint32_t)wy(gy + 1) * nx + gx;
+    const uint32_t rowm = (uint32_t)wy(gy - 1) * P + gx, row0 = (uint32_t)gy * P + gx, rowp = (uint32_t)wy(gy + 1) * P + gx;
 
     // The first (last) site of each row segment: its new populations with e_x =
     // +1 (-1), whose sources are the halo column.  Helper thread t: row t / 2,
@@ -567,7 +581,7 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
         const uint32_t xd = side ? x0 + tw - 1 : x0, xs = side ? wx(x0 + tw) : wx(x0 - 1);
         const uint32_t zo = (uint32_t)z * (uint32_t)nxy, zm = (uint32_t)wz(z - 1) * (uint32_t)nxy,
                        zp = (uint32_t)wz(z + 1) * (uint32_t)nxy;
-        const uint32_t ym = (uint32_t)wy(y - 1) * nx, yc = (uint32_t)y * nx, yp = (uint32_t)wy(y + 1) * nx;
+        const uint32_t ym = (uint32_t)wy(y - 1) * P, yc = (uint32_t)y * P, yp = (uint32_t)wy(y + 1) * P;
         const float ph = phi_plane(z)[(rr + 2) * PX + 4 + (side ? tw - 1 : 0)];
         T lo[9], gp[9];
 #pragma unroll
@@ -699,7 +713,11 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
                 if (PL::ex(i) == 0) continue;
                 const float t = s_end[(r * 2 + (PL::ex(i) > 0 ? 0 : 1)) * 9 + (PL::ez(i) + 1) * 3 + PL::ey(i) + 1];
                 if (PL::ex(i) > 0 && first) el(gnew[i], 0) = t;
-                if (PL::ex(i) < 0 && last) el(gnew[i], V - 1) = t;
+                if (PL::ex(i) < 0 && last) {
+#pragma unroll
+                    for (int k = 0; k < V; ++k)
+                        if (k == ke) el(gnew[i], k) = t;
+                }
             }
         }
         if (!live) return;
@@ -713,14 +731,19 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
         if constexpr (WALLS) {
             // populations from beyond a wall: mirrored partners, axis by axis
             // (an x wall holds the first or last site of one vector)
-            const bool xl = wX && gx == 0, xh = wX && gx + V == nx, yl = wY && gy == 0, yh = wY && gy == ny - 1,
+            const int kh = nx - 1 - gx;  // element on the high x wall, if 0 .. 3
+            const bool xl = wX && gx == 0, xh = wX && kh < V, yl = wY && gy == 0, yh = wY && gy == ny - 1,
                        zl = wZ && z == 0, zh = wZ && z == nz - 1;
             if (xl | xh | yl | yh | zl | zh) {
 #pragma unroll
                 for (int i = 1; i < QG; ++i) {
                     const int m = reflect_dir<PL>(i, 1);
                     if (PL::ex(i) > 0 && xl) gnew[i][0].x = gnew[m][0].x;
-                    if (PL::ex(i) < 0 && xh) gnew[i][H - 1].y = gnew[m][H - 1].y;
+                    if (PL::ex(i) < 0 && xh) {
+#pragma unroll
+                        for (int k = 0; k < V; ++k)
+                            if (k == kh) el(gnew[i], k) = el(gnew[m], k);
+                    }
                 }
 #pragma unroll
                 for (int h = 0; h < H; ++h) {
@@ -737,8 +760,8 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
                     float2 t = gnew[0][h];
 #pragma unroll
                     for (int i = 1; i < QG; ++i) t = __fadd2_rn(t, gnew[i][h]);
-                    if (yz || (xl && h == 0)) pn[h].x = t.x;
-                    if (yz || (xh && h == H - 1)) pn[h].y = t.y;
+                    if (yz || (xl && h == 0) || (xh && kh == 2 * h)) pn[h].x = t.x;
+                    if (yz || (xh && kh == 2 * h + 1)) pn[h].y = t.y;
                 }
             }
         }
@@ -746,7 +769,7 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
         uint32_t hh[V] = {};
         if constexpr (UsesSR<S>::value) {
 #pragma unroll
-            for (int k = 0; k < V; ++k) hh[k] = sr_hash(s + k, seed);
+            for (int k = 0; k < V; ++k) hh[k] = sr_hash(((uint32_t)z * ny + gy) * nx + gx + k, seed);
         }
 #pragma unroll
         for (int i = 1; i < QG; ++i) {

@@ -1,10 +1,11 @@
 """The vector step (two launches, four sites a thread; 3D, 16-bit deviations)
-against the one-launch step kernel (LBPF_KERNEL=generic).
+against the one-launch step kernel (LBPF_KERNEL=vector and generic).
 
 Both evaluate the same operations in the same order, so the fields and the
 populations must agree bit for bit.  Sizes sit at the edges of the vector
-form's tile (64 x 12 sites, row segments of at least two vectors): the
-smallest rows, one and several segments with short last ones, rows of blocks
+form's tile (64 x 12 sites, rows padded to whole vectors of four): the
+smallest rows, one and several segments with short last ones of every length
+modulo four, rows of blocks
 that end inside the domain, and columns of two planes.  Reads between the
 steps put the heat state through both of its forms (synchronised, lagged)."""
 import numpy as np
@@ -25,7 +26,7 @@ def L():
     return lbpf
 
 
-SHAPES = [(2, 2, 8), (3, 13, 12), (5, 12, 64), (4, 25, 72), (7, 11, 128), (9, 37, 140), (40, 24, 200)]
+SHAPES = [(2, 2, 8), (2, 3, 9), (4, 13, 66), (5, 14, 67), (6, 12, 127), (3, 25, 197), (3, 13, 12), (5, 12, 64), (4, 25, 72), (7, 11, 128), (9, 37, 140), (40, 24, 200)]
 FORM = dict(kind=3, eps=0.02, gamma=-0.02)
 
 
@@ -41,7 +42,7 @@ def smooth_fields(shape, seed):
 
 def both(L, monkeypatch, make):
     out = []
-    for kernel in ("", "generic"):
+    for kernel in ("vector", "generic"):
         monkeypatch.setenv("LBPF_KERNEL", kernel)
         out.append(make())
     return out
@@ -65,9 +66,9 @@ def test_vector_step_matches_one_launch_step(L, monkeypatch, shape, lattice, pre
 
 
 @pytest.mark.parametrize("bc", [1, 2, 4, 7])
-@pytest.mark.parametrize("lattice,grad", [(1, 0), (2, 0), (3, 0), (1, 1)])
-def test_vector_step_walls_and_gradients(L, monkeypatch, bc, lattice, grad):
-    shape = (9, 14, 76)
+@pytest.mark.parametrize("lattice,grad,nx", [(1, 0, 76), (2, 0, 76), (3, 0, 77), (1, 1, 74), (1, 0, 67), (2, 0, 65)])
+def test_vector_step_walls_and_gradients(L, monkeypatch, bc, lattice, grad, nx):
+    shape = (9, 14, nx)
     prm = dict(W.C3D_PARAMS, delta=0.4)
     phi, u = smooth_fields(shape, bc + 10 * lattice + grad)
     a, b = both(L, monkeypatch, lambda: gpu_run(L, lattice, shape, prm, [FORM], fields=(phi, u), precision=2, bc=bc,
@@ -76,6 +77,22 @@ def test_vector_step_walls_and_gradients(L, monkeypatch, bc, lattice, grad):
         s.step(17)
     for x, y in zip(a.fields(), b.fields()):
         assert np.array_equal(x, y)
+
+
+def test_padded_rows_through_every_read(L, monkeypatch):
+    """Rows of 67 sites padded to 68: measurement, tip radius, a_s and the
+    seeded start against the one-launch kernel's dense arrays."""
+    prm = dict(W.C3D_PARAMS, delta=0.4)
+    a, b = both(L, monkeypatch, lambda: gpu_run(L, 1, (40, 37, 67), prm, [FORM], seeds=[(33.0, 18.0, 20.0, 8.0, 0)],
+                                                precision=2))
+    for s in (a, b):
+        s.step(12)
+    ma, mb = a.measure(33, 18, 20), b.measure(33, 18, 20)
+    assert np.array_equal(ma[0], mb[0]) and ma[1] == mb[1] and ma[2] == mb[2]
+    assert a.tip_radius(33, 18, 20, 0) == b.tip_radius(33, 18, 20, 0)
+    assert np.array_equal(a.anisotropy_field(), b.anisotropy_field())
+    assert np.array_equal(a.field(L.LBPF_FIELD_INDEX), b.field(L.LBPF_FIELD_INDEX))
+    assert a.query(L.LBPF_Q_SITES) == b.query(L.LBPF_Q_SITES) == 40 * 37 * 67
 
 
 def test_vector_step_of_several_domains_and_segments(L, monkeypatch):
