@@ -10,6 +10,7 @@
 //   1x1 weights  w[cout][cin]             FP32
 // Convolutions are periodic ("same" size, wrap-around), matching the periodic
 // lattice Boltzmann domains.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -259,7 +260,11 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
 // warps 0-3 the epilogue (bias, ReLU, coalesced stores), 4-11 load and convert
 // halos (two buffers where they fit), warp 12 issues the MMAs (two
 // accumulators where they fit), 13-20 stream the weights through a ring where
-// they don't all stay resident, a stage (KC channels of one tap) per warp.  Every hand-over is an mbarrier with a bounded
+// they don't all stay resident, a stage (KC channels of one tap) per warp, or,
+// where KC is 64 channels, warp 13 alone by one TMA load a stage (rows of 64
+// channels in the 128-byte swizzle; the per-piece copies of the eight warps
+// kept the load/store pipe busy for 1800 cycles a stage, 256^2 128 -> 128 65 us,
+// TMATIME by TMA).  Every hand-over is an mbarrier with a bounded
 // wait; on expiry a role sets the error word and leaves, the others follow.
 // MMAs are issued tap by tap, 16 channels at a time, for every tile: the sum's
 // order is that of the gather kernel.
@@ -380,15 +385,19 @@ __device__ __forceinline__ void umma_block(uint32_t d, uint64_t ad, uint64_t bd,
     }
 }
 
-// STREAM: the weights go through the ring.  K16: 16-channel steps of a K block
+// MODE: the weights stay resident, or go through the ring.  K16: 16-channel steps of a K block
 // (KC / 16; resident weights: cin / 16), 0 = any.  One thread issues a tile's
 // MMAs in straight-line code: with a loop over taps and a warp-wide branch in
 // each, an MMA took 150-300 cycles to issue, several times its execution.
-template <int K16, bool STREAM>
-__global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STREAM ? 1 : 2)
-    conv3x3_halo_tc_kernel(const HaloArgs q)
+enum { kResident, kStream, kTma };  // where the weights come from
+constexpr int halo_threads(int mode) { return kEpiT + kLoadT + 32 + (mode == kStream ? kWtT : mode == kTma ? 32 : 0); }
+
+template <int K16, int MODE>
+__global__ void __launch_bounds__(halo_threads(MODE), MODE == kResident ? 2 : 1)
+    conv3x3_halo_tc_kernel(const HaloArgs q, const __grid_constant__ CUtensorMap wmap)
 {
-    constexpr int kHaloThreads = kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0);
+    constexpr bool STREAM = MODE != kResident;
+    constexpr int kHaloThreads = halo_threads(MODE);
     const int co0 = blockIdx.y * q.cout;  // output channel tile
     const int cin = q.cin, cout = q.cout, k8n = cin / 8;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -399,9 +408,12 @@ __global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STR
     __shared__ __align__(16) float s_bias[256];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t halo_b = (size_t)kHaloS * 16 * k8n;
-    const size_t wst_b = (size_t)(cout + 1) * q.KC * 2;  // a slice is cout + 1 rows: conflict-free copies
+    // a stage: slices of cout + 1 rows (conflict-free copies); TMA: cout rows of
+    // 128 bytes, at a multiple of 1024
+    const size_t wst_b = MODE == kTma ? (size_t)cout * 128 : (size_t)(cout + 1) * q.KC * 2;
     unsigned char* sH = smem_raw;
     unsigned char* sW = smem_raw + q.nbuf * halo_b;
+    if (MODE == kTma) sW += (1024 - (smem_u32(sW) & 1023)) & 1023;
     float* sO = reinterpret_cast<float*>(sW + (STREAM ? q.wst * wst_b : (size_t)9 * cin * (cout + 1) * 2));
 
     if (warp == 0) {
@@ -419,7 +431,7 @@ __global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STR
             mbar_init(&s_aempty[k], kEpiT);
         }
         for (int k = 0; k < kMaxWStages; ++k) {
-            mbar_init(&s_wfull[k], 32);
+            mbar_init(&s_wfull[k], MODE == kTma ? 1 : 32);
             mbar_init(&s_wempty[k], 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -524,6 +536,9 @@ __global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STR
             const uint32_t idesc = umma_idesc_bf16(kConvM, cout), bstep = 2 * (cout + 1);
             const int k16n = q.KC / 16;
             const uint64_t w0 = umma_desc(smem_u32(sW), (cout + 1) * 16, 128);
+            // K-major with the 128-byte swizzle (layout 2 at bit 61): 8-row groups
+            // 1024 bytes apart, 16 channels 32 bytes along the row
+            const uint64_t w128 = umma_desc(smem_u32(sW), 16, 1024) | (2ull << 61);
             int buf = 0, acc = 0, st = 0;  // halo buffer, accumulator and weight slot, with their phases
             uint32_t hpar = 0, apar = 1, wpar = 0;
             bool ok = true;
@@ -553,8 +568,8 @@ __global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STR
                                 break;
                             }
                             asm volatile("tcgen05.fence::after_thread_sync;");
-                            umma_block<K16>(d, ad, w0 + (uint64_t)st * (wst_b >> 4), bstep, idesc, k16n,
-                                            (tap | kb) ? 1u : 0u);
+                            const uint64_t bd = (MODE == kTma ? w128 : w0) + (uint64_t)st * (wst_b >> 4);
+                            umma_block<K16>(d, ad, bd, MODE == kTma ? 2 : bstep, idesc, k16n, (tap | kb) ? 1u : 0u);
                             umma_commit(&s_wempty[st]);
                             ad += (uint64_t)k16n * (2 * kHaloS);
                             if (++st == q.wst) {
@@ -578,7 +593,41 @@ __global__ void __launch_bounds__(kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), STR
             if (!ok) atomicOr(&g_conv_error, 64);
         }
         __syncwarp();
-    } else if (STREAM && warp - 13 < q.wst) {
+    } else if (MODE == kTma) {
+        if (lane == 0) {
+            int my_tiles = 0;
+            for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x) ++my_tiles;
+            int st = 0, s = 0, sent = 0;
+            uint32_t par = 1;
+            bool ok = true;
+            for (int k = 0; k < my_tiles && ok; ++k)
+                for (int tap = 0; tap < 9 && ok; ++tap)
+                    for (int kb = 0; kb < nkb; ++kb, ++sent) {
+                        if (!mbar_wait_bounded(&s_wempty[st], par)) {
+                            atomicOr(&g_conv_error, 128);
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&s_wfull[st])),
+                                     "r"((uint32_t)wst_b)
+                                     : "memory");
+                        asm volatile(
+                            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+                            "%3}], [%4];" ::"r"(smem_u32(sW + st * wst_b)),
+                            "l"(&wmap), "r"(kb * 64), "r"(tap * q.cout_all + co0), "r"(smem_u32(&s_wfull[st]))
+                            : "memory");
+                        if (++st == q.wst) {
+                            st = 0;
+                            par ^= 1;
+                        }
+                    }
+            // on expiry: the copies in flight land before the block ends
+            if (!ok)
+                for (s = sent > q.wst ? sent - q.wst : 0; s < sent; ++s)
+                    mbar_wait_bounded(&s_wfull[s % q.wst], (s / q.wst) & 1);
+        }
+        __syncwarp();
+    } else if (MODE == kStream && warp - 13 < q.wst) {
         // weight stream: warp j owns ring slot j and fills the stages j, j + wst,
         // ... (one owner a slot: a slot's phases are waited for in order)
         const int st = warp - 13;
@@ -649,14 +698,41 @@ static cudaError_t opt_in(K kernel, std::atomic<bool> (&done)[kMaxDevices])
 static std::atomic<bool> g_gather_ready[kMaxDevices], g_wgrad_ready[kMaxDevices],
     g_wgrad9_ready[kMaxDevices], g_wgrad3_ready[kMaxDevices];
 
-template <int K16, bool STREAM>
-static cudaError_t launch_halo(const HaloArgs& q, dim3 grid, size_t smem, cudaStream_t s)
+template <int K16, int MODE>
+static cudaError_t launch_halo(const HaloArgs& q, const CUtensorMap& wmap, dim3 grid, size_t smem, cudaStream_t s)
 {
     static std::atomic<bool> ready[kMaxDevices];
-    const cudaError_t e = opt_in(conv3x3_halo_tc_kernel<K16, STREAM>, ready);
+    const cudaError_t e = opt_in(conv3x3_halo_tc_kernel<K16, MODE>, ready);
     if (e != cudaSuccess) return e;
-    conv3x3_halo_tc_kernel<K16, STREAM><<<grid, kEpiT + kLoadT + 32 + (STREAM ? kWtT : 0), smem, s>>>(q);
+    conv3x3_halo_tc_kernel<K16, MODE><<<grid, halo_threads(MODE), smem, s>>>(q, wmap);
     return cudaGetLastError();
+}
+
+// Tensor map of the weights as rows of cin channels, boxes of cout rows by 64
+// channels; false where it cannot be had (the piecewise stream takes over).
+static bool weight_map(const HaloArgs& q, CUtensorMap& map)
+{
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static std::atomic<void*> fn{nullptr};
+    void* f = fn.load(std::memory_order_relaxed);
+    if (!f) {
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess || !f) {
+            cudaGetLastError();
+            return false;
+        }
+        fn.store(f, std::memory_order_relaxed);
+    }
+    const cuuint64_t dims[2] = {(cuuint64_t)q.cin, (cuuint64_t)9 * q.cout_all}, stride[1] = {(cuuint64_t)q.cin * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)q.cout}, one[2] = {1, 1};
+    return reinterpret_cast<Encode>(f)(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                                       const_cast<__nv_bfloat16*>(q.w), dims, stride, box, one,
+                                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Plan of the halo kernel: false where it does not apply.
@@ -671,12 +747,14 @@ static bool halo_plan(HaloArgs& q, size_t& smem, int& per_sm)
     q.wst = 0;
     smem = q.nbuf * halo + all_w + out;
     if (smem > kSmemMax) {
-        // the weights stream; a second halo buffer only beside four stages
-        q.nbuf = 2 * halo + 4 * st + out <= kSmemMax ? 2 : 1;
-        if (q.nbuf * halo + 3 * st + out > kSmemMax) return false;
-        const size_t n = (kSmemMax - q.nbuf * halo - out) / st;
+        // the weights stream; a second halo buffer only beside four stages (and
+        // 1 KB for the TMA form's alignment)
+        const size_t rest = kSmemMax - out - 1024;
+        q.nbuf = 2 * halo + 4 * st <= rest ? 2 : 1;
+        if (q.nbuf * halo + 3 * st > rest) return false;
+        const size_t n = (rest - q.nbuf * halo) / st;
         q.wst = (int)(n < kMaxWStages ? n : kMaxWStages);
-        smem = q.nbuf * halo + q.wst * st + out;
+        smem = q.nbuf * halo + q.wst * st + out + 1024;
     }
     q.tmem_cols = 32;
     while ((int)q.tmem_cols < q.nacc * q.cout) q.tmem_cols <<= 1;
@@ -721,14 +799,19 @@ cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, cons
         if (blocks < 1) blocks = 1;
         if (blocks > tiles) blocks = tiles;
         const dim3 grid((unsigned)blocks, n_tiles);
-        if (q.wst) return q.KC == 64 ? launch_halo<4, true>(q, grid, smem, s) : launch_halo<0, true>(q, grid, smem, s);
+        CUtensorMap map = {};
+        if (q.wst) {
+            if (q.KC == 64 && weight_map(q, map)) return launch_halo<4, kTma>(q, map, grid, smem, s);
+            return q.KC == 64 ? launch_halo<4, kStream>(q, map, grid, smem, s)
+                              : launch_halo<0, kStream>(q, map, grid, smem, s);
+        }
         switch (cin / 16) {
-        case 1: return launch_halo<1, false>(q, grid, smem, s);
-        case 2: return launch_halo<2, false>(q, grid, smem, s);
-        case 3: return launch_halo<3, false>(q, grid, smem, s);
-        case 4: return launch_halo<4, false>(q, grid, smem, s);
-        case 6: return launch_halo<6, false>(q, grid, smem, s);
-        default: return launch_halo<0, false>(q, grid, smem, s);
+        case 1: return launch_halo<1, kResident>(q, map, grid, smem, s);
+        case 2: return launch_halo<2, kResident>(q, map, grid, smem, s);
+        case 3: return launch_halo<3, kResident>(q, map, grid, smem, s);
+        case 4: return launch_halo<4, kResident>(q, map, grid, smem, s);
+        case 6: return launch_halo<6, kResident>(q, map, grid, smem, s);
+        default: return launch_halo<0, kResident>(q, map, grid, smem, s);
         }
     }
     if (b) return cudaErrorInvalidValue;

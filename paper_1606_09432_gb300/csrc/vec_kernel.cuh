@@ -18,7 +18,7 @@
 // 375 instructions a site for the phase field.  The work field costs 8 of
 // 104 bytes a site.  Measured, us a step (step_kernel / this): D3Q15 FP16
 // 512^3 5289 / 3605, 256^3 718 / 533, 351^3 with walls 2286 / 1679, 207 x 174 x
-// 190 397 / 296; 256^3 D3Q19 838 / 643, D3Q27 1260 / 1088.  Rows that are not
+// 190 397 / 296; 256^3 D3Q19 838 / 643, D3Q27 1260 / 980.  Rows that are not
 // whole vectors are padded in memory (DomainDev::px); a row's last partial vector
 // is computed whole, what falls into the padding is never read.  Full (FP32) storage measured 2 % slower
 // this way (the vectors in flight need twice the registers) and stays with
@@ -567,7 +567,6 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
     const int ll = (tw - 1) / V;   // last lane of the segment
     const bool live = r < th && lx <= ll;
     const bool first = lx == 0, last = lx == ll;
-    const int ke = (tw - 1) & (V - 1);  // the segment's last site in its vector
     // threads without a vector (beyond the tile) read the nearest one
     const int gy = y0 + min(r, th - 1), gx = x0 + V * min(lx, ll);
     const uint32_t rowm = (uint32_t)wy(gy - 1) * P + gx, row0 = (uint32_t)gy * P + gx, rowp = (uint32_t)wy(gy + 1) * P + gx;
@@ -620,16 +619,20 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
         const float* cpp = co_plane(z + 1) + (r + 1) * kVecTX + V * lx;
         float2 ph[H];
         lds_v(phi_plane(z) + (r + 2) * PX + 4 + V * lx, ph);
-        // every population vector of the thread is requested before the first is
-        // used (4 registers a direction, the space the new populations take over
-        // one by one)
+        // the thread's population vectors are requested AHEAD directions before
+        // their use (4 registers a direction, the space the new populations take
+        // over one by one): all at once, but 12 of D3Q27's 26, whose space does
+        // not suffice (256^3 FP16, 12 / all: D3Q15 551 / 549 us, D3Q19 723 / 689,
+        // D3Q27 980 / 1083)
+        constexpr int AHEAD = QG > 19 ? 12 : QG;
         uint2 ra[QG], rb[QG];
         auto request = [&](int i) {
             ra[i] = raw4(gc + (long long)(i - 1) * n + s);
             rb[i] = raw4(gc + (long long)(i - 1) * n + src(PL::ey(i), PL::ez(i)));
         };
 #pragma unroll
-        for (int i = 1; i < QG; ++i) request(i);
+        for (int i = 1; i < QG; ++i)
+            if (i <= AHEAD) request(i);
         // new populations; the rest population comes last (its deviation is
         // minus the sum of the others).  Directions i, i + 1 that differ in the
         // sign of e_x share their coefficient vectors.
@@ -652,6 +655,7 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
             const int ex = PL::ex(i), ey = PL::ey(i), ez = PL::ez(i);
             const float2 w = make_float2(float(PL::w(i)), float(PL::w(i))), one = make_float2(-1.f, -1.f);
             float2 gp[H], gl[H], v[H], gs[H];
+            if (i > 0 && i + AHEAD < QG) request(i + AHEAD);
             if (i > 0) {
                 float2 lo[H];
                 unpack2<T>(ra[i], lo);
@@ -708,6 +712,7 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
         // the end sites' populations from beyond the segment (end_sites)
         asm volatile("bar.sync 1, %0;" ::"n"(kVecLX * (kVecTY + 2)) : "memory");
         if (first || last) {
+            const int ke = (tw - 1) & (V - 1);  // the segment's last site in its vector
 #pragma unroll
             for (int i = 1; i < QG; ++i) {
                 if (PL::ex(i) == 0) continue;
