@@ -318,15 +318,15 @@ struct LauncherImpl {
         return step_kernel<KP, KU, S, TXV<V>, TYV<V>, W, A>;
     }
     template <int V, bool A = false>
-    static constexpr size_t smem_v()
+    static constexpr size_t smem_v(bool index = true)
     {
-        return step_smem_bytes<KP, KU, S, TXV<V>, TYV<V>, A>();
+        return step_smem_bytes<KP, KU, S, TXV<V>, TYV<V>, A>(index);
     }
 
     template <int V, bool W, bool A = false>
     static cudaError_t step_v(const StepArgs& a, int n_blocks, cudaStream_t s)
     {
-        kernel<V, W, A>()<<<n_blocks, TXV<V> * TYV<V>, smem_v<V, A>(), s>>>(a);
+        kernel<V, W, A>()<<<n_blocks, TXV<V> * TYV<V>, smem_v<V, A>(a.index), s>>>(a);
         return cudaGetLastError();
     }
     // Tile variant 0 is built periodic, with walls and with an advective

@@ -313,6 +313,8 @@ static StepArgs step_args(const lbpf_ctx* c)
     a.acur = c->acur;
     a.collide = c->lagged;
     a.grad = c->grad;
+    a.index = 0;
+    for (const DomainDev& d : c->dd) a.index |= d.use_index;
     return a;
 }
 

@@ -245,6 +245,7 @@ struct StepArgs {
     int acur;   // aux buffer read (new = acur ^ 1)
     int collide;
     int grad;   // LBPF_GRAD_DD / LBPF_GRAD_FD
+    int index;  // some domain uses the crystal index
 };
 
 // Tile of one thread block of the step kernel, one thread per site of a tile
@@ -434,7 +435,7 @@ struct Launchers {
     // storage only; the kernel also handles walls).  Kinds other than 0 are
     // built for variant 0 only.
     cudaError_t (*step)(int v, int kind, const StepArgs& a, int n_blocks, cudaStream_t s);
-    // Dynamic shared memory of variant v.
+    // Dynamic shared memory of variant v (the most it asks for).
     size_t (*step_smem)(int v);
     // Opt variant v (every kind built for it) into its dynamic shared memory.
     cudaError_t (*prepare)(int v);

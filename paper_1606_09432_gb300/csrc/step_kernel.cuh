@@ -134,6 +134,16 @@ constexpr size_t stf_bytes(int RP)
                                                          : 0;
 }
 
+// Depth of the phi (and index) ring: planes z .. z+3 are in use while plane z
+// is output, and with deviation storage plane z - 1 too (the output phase reads
+// phi^n at its own plane, so the copy of plane z + 4 must not take its slot).
+// Four planes bring the 3D FP32 blocks to 40 KB without the index planes, four
+// blocks an SM into the 164 KB configuration, and L1 from 60 to 92 KB: us a step,
+// five planes / four: 512^3 D3Q15 6055 / 5767, 351^3 with walls 2472 / 2343, 256^3
+// 788 / 779, D3Q19 889 / 878, D3Q27 1317 / 1305, 207^3 D3Q19 561 / 549.
+template <class S>
+constexpr int phi_ring() { return S::dev ? 5 : 4; }
+
 // One work item: the column (x0, y0) of one domain over planes [z0, z1).
 // WALLS: the domain may have zero-flux walls (mirror planes through the
 // boundary nodes, lbpf.h LBPF_BC_WALL_X): stencil indices beyond a wall are
@@ -164,9 +174,7 @@ __device__ __forceinline__ void step_item(const StepArgs& args, const WorkItem i
     constexpr bool CHUNKED = !XZV;
     constexpr int RX = TXT + 2 * XO, RY = TY + 2 * HL, RP = RX * RY;
     constexpr int CX = TXT + 2, CY = TY + 2 * HC, CP = CX * CY;  // tile + 1-site halo
-    // phi / index ring depth: planes z-1 .. z+3 in use while plane z is output
-    // (the output phase reads phi^n only at its own plane)
-    constexpr int NPH = 5;
+    constexpr int NPH = phi_ring<S>();                      // phi / index ring depth
     constexpr int NH = 4;                                   // h ring depth (z .. z+3)
     constexpr int NC = 3;                                   // coefficient ring depth
     constexpr int NCO = 6;                                  // c1, c2, s, vx, vy, vz
@@ -735,16 +743,19 @@ __global__ void __launch_bounds__(TXT * TY, 1024 / (TXT * TY)) step_kernel(const
     }
 }
 
+// index: some domain uses the crystal index (3D without advection: its planes
+// come last and are left out otherwise).
 template <class PL, class UL, class S, int TXT, int TY, bool ADV = false>
-constexpr size_t step_smem_bytes()
+constexpr size_t step_smem_bytes(bool index = true)
 {
     using R = typename S::Real;
     constexpr int HL = IsXZ<PL>::value ? 0 : 2, HC = IsXZ<PL>::value ? 0 : 1;
     constexpr int XO = (IsXZ<PL>::value || sizeof(R) >= 8) ? 2 : 4;
     constexpr int RP = (TXT + 2 * XO) * (TY + 2 * HL), CP = (TXT + 2) * (TY + 2 * HC);
-    constexpr int NPH = 5, NH = 4, NC = 3;
+    constexpr int NPH = phi_ring<S>(), NH = 4, NC = 3;
     constexpr int COP = 6 * CP;
-    return sizeof(R) * (size_t)(NPH * RP + NH * RP + NC * COP) + (((size_t)NPH * RP + 15) & ~size_t(15)) +
+    const size_t planes = IsXZ<PL>::value || ADV || index ? ((size_t)NPH * RP + 15) & ~size_t(15) : 0;
+    return sizeof(R) * (size_t)(NPH * RP + NH * RP + NC * COP) + planes +
            stf_bytes<UL, S, IsXZ<PL>::value>(RP) + (ADV ? sizeof(R) * (size_t)NH * RP : 0);
 }
 
