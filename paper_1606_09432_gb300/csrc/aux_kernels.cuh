@@ -154,7 +154,7 @@ __global__ void heat_sync_kernel(const DomainDev* dp, int cur, int fcur, int acu
 {
     using R = typename S::Real;
     using T = typename S::T;
-    const DomainDev& d = *dp;
+    const DomainDev& d = dp[blockIdx.y];
     const long long n = d.n;
     const R* phi = static_cast<const R*>(d.phi[cur]);
     const R* auxc = static_cast<const R*>(d.aux[acur]);
@@ -476,9 +476,12 @@ struct LauncherImpl {
         }
         return nb > 0 ? nb : 1;
     }
-    static cudaError_t heat_sync(const DomainDev* d, int cur, int fcur, int acur, cudaStream_t s)
+    static cudaError_t heat_sync(const DomainDev* d, int n, int cur, int fcur, int acur, cudaStream_t s)
     {
-        heat_sync_kernel<PL, UL, S><<<152 * 8, 256, 0, s>>>(d, cur, fcur, acur);
+        for (int k = 0; k < n; k += 65535) {  // one launch for the domains (grid y)
+            const int m = n - k < 65535 ? n - k : 65535;
+            heat_sync_kernel<PL, UL, S><<<dim3(m > 4 ? 152 : 152 * 8, m), 256, 0, s>>>(d + k, cur, fcur, acur);
+        }
         return cudaGetLastError();
     }
     static cudaError_t equilibrate(const DomainDev* d, int cur, int fcur, int acur, int grad, int finalize,

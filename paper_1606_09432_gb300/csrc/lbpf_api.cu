@@ -643,6 +643,7 @@ static int check_ctx(lbpf_ctx* c, int domain)
 // gave up); read after the stream has been synchronised.
 static int device_error(lbpf_ctx* c)
 {
+    if (!c->staged) return LBPF_OK;  // no other kernel sets it
     int w = 0;
     CK(cudaMemcpy(&w, c->d_counters + 4, sizeof(int), cudaMemcpyDeviceToHost));
     if (w) return fail(c, LBPF_ETIMEOUT, "a bounded wait in the step kernel gave up (device error word %d)", w);
@@ -660,7 +661,7 @@ static int sync_state(lbpf_ctx* c)
         a.collide = 1;
         for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream));
     } else {
-        for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_sync(c->d_dd + k, c->cur, c->fcur, c->acur, c->stream));
+        CK(c->L->heat_sync(c->d_dd, c->n_domains, c->cur, c->fcur, c->acur, c->stream));
     }
     c->fcur ^= 1;
     if (c->Sg != c->Qg) c->acur ^= 1;

@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
 // they don't all stay resident, a stage (KC channels of one tap) per warp, or,
 // where KC is 64 channels, warp 13 alone by one TMA load a stage (rows of 64
 // channels in the 128-byte swizzle; the per-piece copies of the eight warps
-// kept the load/store pipe busy for 1800 cycles a stage, 256^2 128 -> 128 65 us,
-// TMATIME by TMA).  Every hand-over is an mbarrier with a bounded
+// kept the load/store pipe busy for 1800 cycles a stage: 256^2 128 -> 128 65 us,
+// 29 us by TMA).  Every hand-over is an mbarrier with a bounded
 // wait; on expiry a role sets the error word and leaves, the others follow.
 // MMAs are issued tap by tap, 16 channels at a time, for every tile: the sum's
 // order is that of the gather kernel.
