@@ -60,7 +60,7 @@ WORKLOADS = {
 DTYPE = {0: "f64", 1: "f32", 2: "f32 arithmetic, f16 storage", 3: "f32 arithmetic, bf16 storage",
          4: "f32 arithmetic, f16 storage (stochastic rounding)"}
 METRIC = "fused phi+u LB step MLUPS"
-KERNEL_SOURCES = ["step_kernel.cuh", "staged_kernel.cuh", "lbpf_internal.cuh"]
+KERNEL_SOURCES = ["step_kernel.cuh", "vec_kernel.cuh", "staged_kernel.cuh", "lbpf_internal.cuh"]
 
 
 def peaks():
@@ -577,7 +577,8 @@ def main():
                    "l2": f"state {s.query(L.LBPF_Q_DEVICE_BYTES) / 1e9:.2f} GB per GPU, larger than L2 (no flush)"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": traffic,
-                     "kernel": "step_kernel", "bytes_per_site": bps,
+                     "kernel": "heat_vec_kernel + phi_vec_kernel" if launches > args.steps else "step_kernel",
+                     "bytes_per_site": bps,
                      "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if pk else "fallback 6.8 TB/s"},
         "gpu_launches": launches,
         "clocks": clk.summary(),

@@ -318,6 +318,8 @@ static StepArgs step_args(const lbpf_ctx* c)
     return a;
 }
 
+static long long launches_per_step(const lbpf_ctx* c) { return c->vec ? c->n_domains + 1 : 1; }
+
 // The launches of one time step.
 static cudaError_t issue_step(lbpf_ctx* c, const StepArgs& a)
 {
@@ -753,7 +755,7 @@ static int launch_step(lbpf_ctx* c)
     if (c->lagged) c->fcur ^= 1;
     c->lagged = 1;
     c->steps += 1;
-    c->kernels += 1;
+    c->kernels += launches_per_step(c);
     return LBPF_OK;
 }
 
@@ -794,7 +796,7 @@ static int graph_batch(lbpf_ctx* c)
     }
     CK(cudaGraphLaunch(ex, c->stream));
     c->steps += kGraphSteps;
-    c->kernels += kGraphSteps;  // each batch is kGraphSteps step-kernel launches
+    c->kernels += kGraphSteps * launches_per_step(c);
     return LBPF_OK;
 }
 
