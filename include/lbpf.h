@@ -342,8 +342,11 @@ typedef enum {
  * sites along x by tile_rows along y; in 2D it is one row of 16 * tile_rows
  * sites (128 or 256) along x.  segment (>= 1) is the number of z-planes (3D)
  * or y-rows (2D) per work item (tile_rows = 16 exists only for periodic
- * domains and the generic kernel).  Results do not depend on the schedule;
- * only speed does.  A performance knob with no counterpart in the paper.
+ * domains and the march).  The four-sites-a-thread form (LBPF_Q_KERNEL) has
+ * one tile, 64 x 12 sites: there tile_rows has no effect.  A context on the
+ * block-per-tile form in 2D goes back to the march, with the schedule given.
+ * Results do not depend on the schedule; only speed does.  A performance knob
+ * with no counterpart in the paper.
  * Errors: LBPF_EINVAL. */
 int lbpf_set_schedule(lbpf_ctx* ctx, int tile_rows, int segment);
 

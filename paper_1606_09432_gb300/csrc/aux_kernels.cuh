@@ -402,21 +402,31 @@ struct LauncherImpl {
     }
     // the vector step: 3D, 16-bit deviations
     static constexpr bool kVec = PL::D == 3 && S::dev;
-    static cudaError_t heat_vec(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s)
+    static cudaError_t heat_vec(const DomainDev* h, const DomainDev* d, int n, const StepArgs& a, cudaStream_t s)
     {
         if constexpr (kVec) {
-            const int gx = (h.px / 4 + kHeatX - 1) / kHeatX, gy = (h.ny + kHeatY - 1) / kHeatY;
-            int zlen = 16;
-            while (zlen > 1 && (long long)gx * gy * ((h.nz + zlen - 1) / zlen) < 152 * 8) zlen /= 2;
-            const dim3 grid(gx, gy, (h.nz + zlen - 1) / zlen), block(kHeatX, kHeatY);
-            if (h.bc)
-                heat_vec_kernel<UL, S, true><<<grid, block, 0, s>>>(d, a.cur, a.fcur, a.acur, a.collide, zlen, a.counters);
-            else
-                heat_vec_kernel<UL, S, false><<<grid, block, 0, s>>>(d, a.cur, a.fcur, a.acur, a.collide, zlen, a.counters);
+            const dim3 block(kHeatX, kHeatY);
+            for (int k = 0; k < n;) {
+                const HeatGrid g = heat_grid(h + k, n - k);
+                if (h[k].bc)
+                    heat_vec_kernel<UL, S, true>
+                        <<<g.grid, block, 0, s>>>(d + k, a.cur, a.fcur, a.acur, a.collide, g.zlen, g.nseg, a.counters);
+                else
+                    heat_vec_kernel<UL, S, false>
+                        <<<g.grid, block, 0, s>>>(d + k, a.cur, a.fcur, a.acur, a.collide, g.zlen, g.nseg, a.counters);
+                k += g.m;
+            }
             return cudaGetLastError();
         } else {
             return cudaErrorNotSupported;
         }
+    }
+    static int heat_vec_launches(const DomainDev* h, int n)
+    {
+        int launches = 0;
+        if constexpr (kVec)
+            for (int k = 0; k < n; ++launches) k += heat_grid(h + k, n - k).m;
+        return launches;
     }
     static cudaError_t phi_vec(int walls, const StepArgs& a, int n_blocks, cudaStream_t s)
     {
@@ -511,7 +521,8 @@ struct LauncherImpl {
     {
         static const Launchers L = {&step,     &smem,           &prepare,  &blocks_per_sm,
                                     kStaged ? &step_staged : nullptr,      &staged_blocks_per_sm,
-                                    kVec ? &heat_vec : nullptr,            &phi_vec,
+                                    kVec ? &heat_vec : nullptr,            &heat_vec_launches,
+                                    &phi_vec,
                                     &vec_blocks_per_sm,
                                     PL::D == 2 ? &tile_step : nullptr,
                                     &heat_sync, &equilibrate,   &read_u,   &read_pop,

@@ -318,7 +318,10 @@ static StepArgs step_args(const lbpf_ctx* c)
     return a;
 }
 
-static long long launches_per_step(const lbpf_ctx* c) { return c->vec ? c->n_domains + 1 : 1; }
+static long long launches_per_step(const lbpf_ctx* c)
+{
+    return c->vec ? c->L->heat_vec_launches(c->dd.data(), c->n_domains) + 1 : 1;
+}
 
 // The launches of one time step.
 static cudaError_t issue_step(lbpf_ctx* c, const StepArgs& a)
@@ -326,10 +329,8 @@ static cudaError_t issue_step(lbpf_ctx* c, const StepArgs& a)
     if (c->staged) return c->L->step_staged(a, c->n_blocks, c->stream);
     if (c->tile) return c->L->tile_step(c->kind & kStepWalls, a, c->stream);
     if (!c->vec) return c->L->step(c->tile_v, c->kind, a, c->n_blocks, c->stream);
-    for (int k = 0; k < c->n_domains; ++k) {
-        const cudaError_t e = c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = c->L->heat_vec(c->dd.data(), c->d_dd, c->n_domains, a, c->stream);
+    if (e != cudaSuccess) return e;
     return c->L->phi_vec(c->kind & kStepWalls, a, c->n_blocks, c->stream);
 }
 
@@ -432,11 +433,11 @@ static int autotune(lbpf_ctx* c)
 }
 
 // Whether the context takes the vector step.  It can where every domain is 3D
-// with 16-bit deviations, one crystal, no advection and site indices in 31 bits;
-// it pays where its 64-site row segments are at least 0.6 full and there is work
+// with 16-bit deviations, one crystal, no advection, site indices in 31 bits and
+// rows and planes within a launch grid's limits; it pays where its 64-site row segments are at least 0.6 full and there is work
 // for more than a wave of blocks (FP16, us a step, one launch / vector: 32^3 14.5
 // / 25.1, 64^3 29.7 / 29.1, 96^3 56.0 / 52.8, 128^3 115 / 85, 207x174x190 397 /
-// 296, 351^3 walls 2286 / 1679; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201).
+// 296, 351^3 walls 2307 / 1682; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201).
 // LBPF_KERNEL: "vector" wherever it can, any other value never.
 static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_domains)
 {
@@ -446,8 +447,8 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
     double sites = 0, slots = 0;
     for (int k = 0; k < n_domains; ++k) {
         const lbpf_domain& d = domains[k];
-        if (d.nx < 8 || (long long)((d.nx + 3) / 4 * 4) * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 || d.adv[0] != 0.0 || d.adv[1] != 0.0 ||
-            d.adv[2] != 0.0)
+        if (d.nx < 8 || (long long)((d.nx + 3) / 4 * 4) * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 ||
+            d.adv[0] != 0.0 || d.adv[1] != 0.0 || d.adv[2] != 0.0 || d.ny > 65535 * kHeatY || d.nz > 65535)
             return false;
         sites += (double)d.nx * d.ny * d.nz;
         slots += (double)((d.nx + kVecTX - 1) / kVecTX * kVecTX) * d.ny * d.nz;
@@ -455,8 +456,10 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
     return forced || (sites >= 2e5 && sites >= 0.6 * slots);
 }
 
-extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattice, int grad, int precision,
-                           void* stream, lbpf_ctx** out)
+// lbpf_create with the vector step where it applies, or (vec false) never.
+// *vec: whether the context was to take it.
+static int create(const lbpf_domain* domains, int n_domains, int lattice, int grad, int precision, void* stream,
+                  bool* vec, lbpf_ctx** out)
 {
     lbpf_ctx* c = nullptr;
     if (!out) return fail(nullptr, LBPF_EINVAL, "lbpf_create: out is NULL");
@@ -530,7 +533,7 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
     const double e2u = (dim == 2) ? 1.0 / 3.0 : 1.0 / 4.0;
 
     const char* kenv = getenv("LBPF_KERNEL");
-    c->vec = vec_applies(L, domains, n_domains);
+    c->vec = *vec = *vec && vec_applies(L, domains, n_domains);
 
     int rc = LBPF_OK;
     long long max_n = 0;
@@ -633,6 +636,18 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
     return LBPF_OK;
 }
 
+extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattice, int grad, int precision,
+                           void* stream, lbpf_ctx** out)
+{
+    bool vec = true;
+    int rc = create(domains, n_domains, lattice, grad, precision, stream, &vec, out);
+    if (rc == LBPF_ENOMEM && vec) {  // its work field and row padding (4 to 8 % of the state) may be what does not fit
+        vec = false;
+        rc = create(domains, n_domains, lattice, grad, precision, stream, &vec, out);
+    }
+    return rc;
+}
+
 static int check_ctx(lbpf_ctx* c, int domain)
 {
     if (!c) return fail(nullptr, LBPF_EINVAL, "context is NULL");
@@ -661,7 +676,7 @@ static int sync_state(lbpf_ctx* c)
         // field; the stochastic form rounds differently here)
         StepArgs a = step_args(c);
         a.collide = 1;
-        for (int k = 0; k < c->n_domains; ++k) CK(c->L->heat_vec(c->dd[k], c->d_dd + k, a, c->stream));
+        CK(c->L->heat_vec(c->dd.data(), c->d_dd, c->n_domains, a, c->stream));
     } else {
         CK(c->L->heat_sync(c->d_dd, c->n_domains, c->cur, c->fcur, c->acur, c->stream));
     }

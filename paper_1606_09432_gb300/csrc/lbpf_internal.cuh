@@ -261,6 +261,7 @@ constexpr int kStripX[kNumTileVariants] = {128, 256};
 constexpr int kTileRX = 32, kTileRY = 8;
 // Tile of the vector step's phase-field launch (vec_kernel.cuh).
 constexpr int kVecTX = 64, kVecTY = 12;
+constexpr int kHeatX = 32, kHeatY = 8;     // block of its heat launch: 128 x 8 sites
 constexpr int tile_x(int dim, int v) { return dim == 3 ? TX : kStripX[v]; }
 constexpr int tile_y(int dim, int v) { return dim == 3 ? kTileRows[v] : 1; }
 
@@ -445,10 +446,12 @@ struct Launchers {
     // nullptr where it is not built (2D, full storage, D3Q27).
     cudaError_t (*step_staged)(const StepArgs& a, int n_blocks, cudaStream_t s);
     int (*staged_blocks_per_sm)();
-    // The vector step (vec_kernel.cuh): the heat launch of one domain (its host
-    // copy h for the sizes, d on the device), then the phase-field launch over
-    // the items; nullptr where it is not built (2D, FP64).
-    cudaError_t (*heat_vec)(const DomainDev& h, const DomainDev* d, const StepArgs& a, cudaStream_t s);
+    // The vector step (vec_kernel.cuh): the heat launches of n domains (their host
+    // copies h for the sizes, d on the device) and how many there are, then the
+    // phase-field launch over the items; heat_vec is nullptr where it is not built
+    // (2D, full storage).
+    cudaError_t (*heat_vec)(const DomainDev* h, const DomainDev* d, int n, const StepArgs& a, cudaStream_t s);
+    int (*heat_vec_launches)(const DomainDev* h, int n);
     cudaError_t (*phi_vec)(int walls, const StepArgs& a, int n_blocks, cudaStream_t s);
     int (*vec_blocks_per_sm)(int walls);
     // The one-tile step (tile_kernel.cuh) over n_items tiles of 30 x 6 sites;

@@ -12,18 +12,21 @@
 //
 // Why: step_kernel is bound by instruction issue (1210 thread-instructions a
 // site with FP16 deviations, 73 % issue-active, 30 % of HBM at 256^3).  Apart,
-// the heat update is computed once per site instead of on every halo (106
+// the heat update is computed once per site instead of on every halo (108
 // instructions a site, bound by HBM: 127 us at 256^3, 66 % of the DRAM rate),
 // and both launches read and write four sites per instruction, which leaves
-// 375 instructions a site for the phase field.  The work field costs 8 of
+// 408 instructions a site for the phase field.  The work field costs 8 of
 // 104 bytes a site.  Measured, us a step (step_kernel / this): D3Q15 FP16
-// 512^3 5289 / 3605, 256^3 718 / 533, 351^3 with walls 2286 / 1679, 207 x 174 x
-// 190 397 / 296; 256^3 D3Q19 838 / 643, D3Q27 1260 / 980.  Rows that are not
+// 512^3 5289 / 3782 (stochastic rounding 7147 / 5936), 256^3 719 / 551, 351^3
+// with walls 2307 / 1682, 207 x 174 x 190 397 / 296; 256^3 D3Q19 838 / 690,
+// D3Q27 1260 / 980.  Rows that are not
 // whole vectors are padded in memory (DomainDev::px); a row's last partial vector
 // is computed whole, what falls into the padding is never read.  Full (FP32) storage measured 2 % slower
 // this way (the vectors in flight need twice the registers) and stays with
 // step_kernel.
 #pragma once
+
+#include <algorithm>
 
 #include "step_kernel.cuh"
 
@@ -117,21 +120,57 @@ __device__ __forceinline__ int wrap_axis(int v, int n, bool wall)
 // A thread owns four sites along x and marches over planes [z0, z1), keeping
 // h = aux + phi / 2 of its own column at z - 1, z, z + 1 in registers; rows
 // y +- 1 and the sites x - 1, x + 4 come from global memory (L1).  With
-// collide == 0 (the state is synchronised) only u^n and aux^n are formed.
-constexpr int kHeatX = 32, kHeatY = 8;  // block: 128 x 8 sites
+// collide == 0 (the state is synchronised) only u^n and aux^n are formed.  One
+// launch covers a group of domains (HeatGrid): nseg runs of zlen planes each in
+// grid z.
+
+// The launch over the first m of n domains: as many in a row, with or without
+// walls alike, as keep at least half of the blocks busy when all get the
+// largest one's, in the grid's limits (vec_applies holds a domain's own ny and
+// nz to them).  A launch a domain costs its latency each time: FP16, us a step,
+// a launch each / grouped (the march): 64 domains of 48^3 513 / 343 (474), 64 of
+// 64^3 930 / 665 (760), 8 of 128^3 581 / 547 (727).
+struct HeatGrid {
+    int m, zlen, nseg;
+    dim3 grid;
+};
+inline HeatGrid heat_grid(const DomainDev* h, int n)
+{
+    HeatGrid g{};
+    long long gx = 0, gy = 0, nz = 0, work = 0;
+    while (g.m < n && (h[g.m].bc != 0) == (h[0].bc != 0)) {
+        const DomainDev& d = h[g.m];
+        const long long bx = (d.px / 4 + kHeatX - 1) / kHeatX, by = (d.ny + kHeatY - 1) / kHeatY;
+        const long long ax = std::max(gx, bx), ay = std::max(gy, by), az = std::max(nz, (long long)d.nz);
+        const long long w = work + bx * by * d.nz;
+        if (g.m > 0 && (ax * ay * az * (g.m + 1) > 2 * w || az * (g.m + 1) > 65535)) break;
+        gx = ax;
+        gy = ay;
+        nz = az;
+        work = w;
+        ++g.m;
+    }
+    g.zlen = 16;
+    while (g.zlen > 1 && gx * gy * ((nz + g.zlen - 1) / g.zlen) * g.m < 152 * 8) g.zlen /= 2;
+    g.nseg = (int)((nz + g.zlen - 1) / g.zlen);
+    g.grid = dim3((unsigned)gx, (unsigned)gy, (unsigned)(g.nseg * g.m));
+    return g;
+}
 
 template <class UL, class S, bool WALLS>
 __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDev* dp, int cur, int fcur, int acur,
-                                                                 int collide, int zlen, const int* counters)
+                                                                 int collide, int zlen, int nseg,
+                                                                 const int* counters)
 {
     using T = typename S::T;
     constexpr int QU = UL::Q;
     static_assert(UL::D == 3 && QU == 7 && S::dev, "D3Q7, 16-bit deviations");
-    const DomainDev& d = *dp;
+    const DomainDev& d = dp[(int)blockIdx.z / nseg];
     const int nx = d.nx, ny = d.ny, nz = d.nz;
     const int x = ((int)blockIdx.x * kHeatX + (int)threadIdx.x) * 4, y = (int)blockIdx.y * kHeatY + (int)threadIdx.y;
     if (x >= nx || y >= ny) return;
-    const int z0 = (int)blockIdx.z * zlen, z1 = min(z0 + zlen, nz);
+    const int z0 = (int)blockIdx.z % nseg * zlen, z1 = min(z0 + zlen, nz);
+    if (z0 >= nz) return;
     const long long n = d.n, nxy = (long long)d.px * ny;
     const bool wX = WALLS && (d.bc & LBPF_BC_WALL_X), wY = WALLS && (d.bc & LBPF_BC_WALL_Y),
                wZ = WALLS && (d.bc & LBPF_BC_WALL_Z);
@@ -289,8 +328,9 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
 // lane shuffle, and the result back by another; the one destination site of a
 // row segment whose source lies beyond the segment is computed apart (warp 6).
 // What bounds it: latency.  16 warps an SM at 128 registers (the populations of
-// four sites in flight) keep 44 % of the issue slots and 55 % of the shared
-// memory pipe busy at 256^3 (404 us, 38 % of the DRAM rate).  Tried: two sites
+// four sites in flight) keep 45 % of the issue slots and 54 % of the shared
+// memory pipe busy at 256^3 (418 us, 35 % of the DRAM rate), the barriers being
+// the largest stall.  Tried: two sites
 // a thread with 64 registers and 32 warps (15 % slower: as many spills and
 // 20 % more instructions), 14 rows with one helper warp (3 % slower at 512^3:
 // that warp was the longest path), loads that skip L1 (10 % slower: spilled

@@ -112,3 +112,59 @@ def test_vector_step_of_several_domains_and_segments(L, monkeypatch):
     for k in (0, 1):
         for x, y in zip(a.fields(k), b.fields(k)):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("shapes,heat_launches", [
+    ([(24, 24, 40)] * 5, 1),  # alike: one heat launch
+    ([(8, 9, 16), (8, 9, 16), (20, 26, 200), (5, 9, 12), (5, 9, 12)], 3),  # ragged: 2 + 2 + 1
+    ([(10, 20, 72, 7), (11, 20, 72, 7), (11, 19, 70, 0)], 2),  # walls and periodic apart
+])
+def test_heat_launch_over_several_domains(L, monkeypatch, shapes, heat_launches):
+    def make():
+        doms = [L.make_domain(s[2], s[1], s[0], lam=10.0, delta=0.4, crystals=[L.make_crystal(**FORM)],
+                              bc=s[3] if len(s) > 3 else 0, **{k: v for k, v in W.C3D_PARAMS.items() if k != "lam"})
+                for s in shapes]
+        s = L.Solver(doms, L.LBPF_D3Q15_D3Q7, L.LBPF_GRAD_DD, L.LBPF_FP32_FP16DEV)
+        for k, sh in enumerate(shapes):
+            s.write_fields(*smooth_fields(sh[:3], k), domain=k)
+        return s
+    a, b = both(L, monkeypatch, make)
+    for n in (1, 4):
+        n0 = a.query(L.LBPF_Q_STEP_KERNELS)
+        a.step(n)
+        b.step(n)
+        assert a.query(L.LBPF_Q_STEP_KERNELS) - n0 == n * (heat_launches + 1)
+        for k in range(len(shapes)):
+            for x, y in zip(a.fields(k), b.fields(k)):
+                assert np.array_equal(x, y)
+
+
+def test_one_launch_step_where_the_work_field_does_not_fit(L, monkeypatch):
+    """A state that fits the device memory only without the vector step's work
+    field is still taken, and gives the same results."""
+    import torch
+    n, prm = 256, dict(W.C3D_PARAMS, delta=0.4)
+    seeds = [(128.0, 128.0, 128.0, 8.0, 0)]
+
+    def make():
+        return gpu_run(L, 1, (n, n, n), prm, [FORM], seeds=seeds, precision=2)
+    a, b = both(L, monkeypatch, make)  # both kernels loaded
+    a.step(3)
+    b.step(3)
+    ref = a.fields()
+    need = b.query(L.LBPF_Q_DEVICE_BYTES)
+    assert a.query(L.LBPF_Q_DEVICE_BYTES) - need > 50e6  # the work field, less a smaller table of items
+    a.close()
+    b.close()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(int(free - need - 40e6), dtype=torch.uint8, device="cuda")
+    monkeypatch.delenv("LBPF_KERNEL")
+    s = make()
+    del hog
+    torch.cuda.empty_cache()
+    n0 = s.query(L.LBPF_Q_STEP_KERNELS)
+    s.step(3)
+    assert s.query(L.LBPF_Q_STEP_KERNELS) - n0 == 3
+    for x, y in zip(ref, s.fields()):
+        assert np.array_equal(x, y)
