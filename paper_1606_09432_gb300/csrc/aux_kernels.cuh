@@ -106,7 +106,7 @@ __global__ void equilibrate_kernel(const DomainDev* dp, int cur, int fcur, int a
     T* g = static_cast<T*>(d.g[cur]);
     T* f = static_cast<T*>(d.f[fcur]);
     int8_t* I = d.I[cur];
-    const R De2 = R(d.Dphi / PL::E2);
+    const R De2 = par_of<R>(d).De2;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         const SiteNb nb = site_nb(d, s, x, y, z);
@@ -117,8 +117,7 @@ __global__ void equilibrate_kernel(const DomainDev* dp, int cur, int fcur, int a
         int cryst = 1;
         if (d.use_index) {
             int Iv = I[s];
-            const double xi = sizeof(R) == 4 ? fmax(d.xi_lu, 1e-6) : d.xi_lu;
-            if (finalize_index && !(ph > R(0) || Gx * Gx + Gy * Gy + Gz * Gz > R(xi * xi))) Iv = 0;
+            if (finalize_index && !(ph > R(0) || Gx * Gx + Gy * Gy + Gz * Gz > par_of<R>(d).xi2)) Iv = 0;
             I[s] = (int8_t)Iv;
             cryst = Iv;
         }
@@ -162,7 +161,7 @@ __global__ void heat_sync_kernel(const DomainDev* dp, int cur, int fcur, int acu
     const T* fc = static_cast<const T*>(d.f[fcur]);
     T* fn = static_cast<T*>(d.f[fcur ^ 1]);
     const R* Uc = static_cast<const R*>(d.U[acur]);
-    const R om = R(1) - R(d.inv_eta_u);
+    const R om = R(1) - par_of<R>(d).inv_eta_u;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         const SiteNb nb = site_nb(d, s, x, y, z);

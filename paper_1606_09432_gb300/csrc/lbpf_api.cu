@@ -557,6 +557,9 @@ static int create(const lbpf_domain* domains, int n_domains, int lattice, int gr
         // kappa = e^2 (eta_u - 1/2) dx^2 / dt, Eq. (ThermalDiffusivity)
         h.inv_eta_u = 1.0 / (d.kappa * d.dt / (e2u * d.dx * d.dx) + 0.5);
         h.xi_lu = d.xi * d.dx;
+        const double De2 = h.Dphi / D2Q9::E2, xi32 = std::max(h.xi_lu, 1e-6);
+        h.r64 = {De2, 1.0 / (De2 + 0.5), h.qphi, h.lambda, h.inv_eta_u, h.xi_lu * h.xi_lu};
+        h.r32 = {(float)De2, (float)h.r64.ieta1, (float)h.qphi, (float)h.lambda, (float)h.inv_eta_u, (float)(xi32 * xi32)};
         // advective heat equilibrium: a = v dt / (dx e^2)
         h.advect = d.adv[0] != 0.0 || d.adv[1] != 0.0 || d.adv[2] != 0.0;
         if (h.advect) c->kind |= kStepAdvect;
@@ -566,9 +569,9 @@ static int create(const lbpf_domain* domains, int n_domains, int lattice, int gr
         for (int j = 0; j < d.n_crystals; ++j) {
             h.cr[j].kind = d.crystals[j].kind;
             h.cr[j].q = d.crystals[j].q;
-            h.cr[j].eps = d.crystals[j].eps;
-            h.cr[j].gamma = d.crystals[j].gamma;
-            h.cr[j].phi0 = d.crystals[j].phi0;
+            const lbpf_crystal& cr = d.crystals[j];
+            h.cr[j].r64 = {cr.eps, cr.gamma, cr.phi0};
+            h.cr[j].r32 = {(float)cr.eps, (float)cr.gamma, (float)cr.phi0};
         }
         for (int b = 0; b < 2 && rc == LBPF_OK; ++b) {
             rc = dev_alloc(c, &h.g[b], (size_t)c->Sg * h.n * c->ssize);

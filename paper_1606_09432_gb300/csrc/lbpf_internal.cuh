@@ -189,10 +189,29 @@ template <class S, int Q> struct NStored { static constexpr int value = S::dev ?
 // ---------------------------------------------------------------------------
 // Per-domain device parameters and buffers.
 // ---------------------------------------------------------------------------
+// Parameters a kernel needs at every site, in both arithmetic types: a double
+// divided or converted per thread or item keeps the FP64 pipe (1/64 of the FP32
+// rate) busy in the FP32 kernels too (us a step: 128^2 FP32 4.4 -> 3.8; 1024^2
+// of two crystals 64 -> 61; 800^2 FP64, where the two reciprocals away from an
+// interface go as well, 228 -> 198).  Rounded on the host as the conversion would.
+template <class R>
+struct CrystalPar {
+    R eps, gamma, phi0;
+};
+template <class R>
+struct DomainPar {
+    R De2;        // Dphi / e^2
+    R ieta1;      // 1 / eta where a_s = 1: 1 / (De2 + 1/2)
+    R qphi, lambda, inv_eta_u;
+    R xi2;        // index threshold on |grad phi|^2, in FP32 not below the
+                  // rounding noise of the gradient (1e-6)
+};
+
 struct CrystalDev {
     int kind;
     int q;
-    double eps, gamma, phi0;
+    CrystalPar<double> r64;
+    CrystalPar<float> r32;
 };
 
 struct DomainDev {
@@ -204,6 +223,8 @@ struct DomainDev {
     // px ny nz.  Kernels of contexts without the vector step use nx as pitch.
     int px;
     long long n;
+    DomainPar<double> r64;  // of the following four
+    DomainPar<float> r32;
     double Dphi;        // (W0^2 / tau0) (dt / dx^2), Eq. (LBE_RelaxationTime)
     double qphi;        // dt / tau0, source factor of Eq. (LBE_Eq_Phase)
     double lambda;      // coupling, Eq. (LBE_SourceTerm)
@@ -227,6 +248,17 @@ struct DomainDev {
     void* U[2];
     void* u_work;       // u^n between the two launches of the vector step (vec_kernel.cuh)
 };
+
+template <class R>
+__host__ __device__ __forceinline__ auto& par_of(const DomainDev& d)
+{
+    if constexpr (sizeof(R) == 8) return d.r64; else return d.r32;
+}
+template <class R>
+__host__ __device__ __forceinline__ auto& par_of(const CrystalDev& c)
+{
+    if constexpr (sizeof(R) == 8) return c.r64; else return c.r32;
+}
 
 // One thread block's work: a column of TX x TY sites over planes [z0, z1).
 struct WorkItem {
@@ -365,13 +397,14 @@ __device__ __forceinline__ void anisotropy(const CrystalDev& c, R Gx, R Gy, R Gz
     Nx = Ny = Nz = R(0);
     a = R(1);
     if (!(g2 > guard2<R>())) return;
-    const R eps = R(c.eps), gam = R(c.gamma);
+    const CrystalPar<R>& cp = par_of<R>(c);
+    const R eps = cp.eps, gam = cp.gamma;
     if (c.kind == LBPF_AS_ANGLE) {
         // Eq. (As_Theta), varphi = atan2(n_y, n_x) with n = -G/|G|;
         // N = a a'(varphi) (-G_y, G_x).
         const R vphi = atan2(-Gy, -Gx);
         R sn, cs;
-        sincos(R(c.q) * (vphi - R(c.phi0)), &sn, &cs);
+        sincos(R(c.q) * (vphi - cp.phi0), &sn, &cs);
         a = R(1) + eps * cs;
         const R ap = -eps * R(c.q) * sn;
         Nx = -a * ap * Gy;

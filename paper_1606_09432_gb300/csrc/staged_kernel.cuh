@@ -208,10 +208,11 @@ __device__ __forceinline__ void staged_item(const StepArgs& args, const WorkItem
         else
             *p = from_real<T, R>(v);
     };
-    const R De2 = R(dm.Dphi / PL::E2);
-    const R qphi = R(dm.qphi);
-    const R lam = R(dm.lambda);
-    const R om_u = R(1) - R(dm.inv_eta_u);
+    const DomainPar<R>& par = par_of<R>(dm);
+    const R De2 = par.De2;
+    const R qphi = par.qphi;
+    const R lam = par.lambda;
+    const R om_u = R(1) - par.inv_eta_u;
     const CrystalDev cr = dm.cr[0];
 
     // periodic wrap of indices at most a few sites outside [0, n)

@@ -239,15 +239,9 @@ __device__ __forceinline__ void step_item(const StepArgs& args, const WorkItem i
         else
             *p = from_real<T, R>(v);
     };
-    const R Dphi = R(dm.Dphi);
-    const R De2 = R(dm.Dphi / PL::E2);
-    const R qphi = R(dm.qphi);
-    const R lam = R(dm.lambda);
-    const R ieu = R(dm.inv_eta_u);
+    const DomainPar<R>& par = par_of<R>(dm);
+    const R De2 = par.De2, qphi = par.qphi, lam = par.lambda, ieu = par.inv_eta_u, xi2 = par.xi2;
     const R om_u = R(1) - ieu;
-    // index threshold; in FP32 not below the rounding noise of the gradient (1e-6)
-    const R xi2 = sizeof(R) == 4 ? R(fmax(dm.xi_lu, 1e-6) * fmax(dm.xi_lu, 1e-6)) : R(dm.xi_lu * dm.xi_lu);
-    (void)Dphi;
 
     // walled axes of the kernel's view (a 2D domain's y axis is the kernel's z)
     const int bcm = WALLS ? dm.bc : 0;
@@ -569,9 +563,12 @@ __device__ __forceinline__ void step_item(const StepArgs& args, const WorkItem i
                 }
             }
 
-            const R A2 = a * a;
-            const R iA2 = recip<R>(A2);
-            const R ieta = recip<R>(A2 * De2 + R(0.5));
+            R iA2 = R(1), ieta = par.ieta1;
+            if (sizeof(R) == 4 || a != R(1)) {  // (FP64 divides: not where there is no interface)
+                const R A2 = a * a;
+                iA2 = recip<R>(A2);
+                ieta = recip<R>(A2 * De2 + R(0.5));
+            }
             const R omp = (R(1) - ph) * (R(1) + ph);
             const R Qphi = (ph - lam * u * omp) * omp;
             const R vf = -De2 * ieta * iA2;

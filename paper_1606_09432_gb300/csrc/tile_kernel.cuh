@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(kTileRX* kTileRY) tile_step_kernel(const StepA
     const int fk = (ly + 1) * FX + lx + 1;  // this site in the frame
     R phy = R(0);
     if (active) {
-        const R ieu = R(dm.inv_eta_u), om_u = R(1) - ieu;
+        const DomainPar<R>& par = par_of<R>(dm);
+        const R ieu = par.inv_eta_u, om_u = R(1) - ieu;
         const R ph = s_phi[fk];
         phy = ph;
         R u = 0;
@@ -218,9 +219,8 @@ __global__ void __launch_bounds__(kTileRX* kTileRY) tile_step_kernel(const StepA
         // crystal index (Sec. 4.3)
         int cryst = 1;
         if (use_index) {
-            const R xi2 = sizeof(R) == 4 ? R(fmax(dm.xi_lu, 1e-6) * fmax(dm.xi_lu, 1e-6)) : R(dm.xi_lu * dm.xi_lu);
             int Iv = Ic[s];
-            if (Iv == 0 && Gx * Gx + Gy * Gy > xi2) {
+            if (Iv == 0 && Gx * Gx + Gy * Gy > par.xi2) {
 #pragma unroll
                 for (int i = 1; i < QG; ++i) {
                     const int v = Ic[site(PL::ex(i), PL::ey(i))];
@@ -236,10 +236,13 @@ __global__ void __launch_bounds__(kTileRX* kTileRY) tile_step_kernel(const StepA
             R n2 = 0;
             anisotropy<R, 2>(dm.cr[cryst - 1], Gx, Gy, R(0), a, Nx, Ny, n2);
         }
-        const R De2 = R(dm.Dphi / PL::E2), qphi = R(dm.qphi), lam = R(dm.lambda);
-        const R A2 = a * a;
-        const R iA2 = recip<R>(A2);
-        const R ieta = recip<R>(A2 * De2 + R(0.5));
+        const R De2 = par.De2, qphi = par.qphi, lam = par.lambda;
+        R iA2 = R(1), ieta = par.ieta1;
+        if (sizeof(R) == 4 || a != R(1)) {  // (FP64 divides: not where there is no interface)
+            const R A2 = a * a;
+            iA2 = recip<R>(A2);
+            ieta = recip<R>(A2 * De2 + R(0.5));
+        }
         const R omp = (R(1) - ph) * (R(1) + ph);
         const R Qphi = (ph - lam * u * omp) * omp;
         const R vf = -De2 * ieta * iA2;

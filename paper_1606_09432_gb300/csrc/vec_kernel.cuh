@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kHeatX* kHeatY) heat_vec_kernel(const DomainDe
     float* __restrict__ auxn = static_cast<float*>(d.aux[acur ^ 1]);
     const float* __restrict__ phi = static_cast<const float*>(d.phi[cur]);
     float* __restrict__ uo = static_cast<float*>(d.u_work);
-    const float ieu = (float)d.inv_eta_u, om_u = 1.f - ieu;
+    const float ieu = d.r32.inv_eta_u, om_u = 1.f - ieu;
     const uint32_t seed = UsesSR<S>::value ? (uint32_t)counters[2 + cur] : 0u;
     const long long row = (long long)y * d.px + x;  // in-plane offset of the vector
     const int ke = min(3, nx - 1 - x);              // the vector's last site (the rest is row padding)
@@ -393,7 +393,7 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
     float* __restrict__ phin = static_cast<float*>(dm.phi[args.cur ^ 1]);
     const float* __restrict__ uc = static_cast<const float*>(dm.u_work);
     const uint32_t seed = UsesSR<S>::value ? (uint32_t)args.counters[2 + args.cur] : 0u;
-    const float De2 = float(dm.Dphi / PL::E2), qphi = float(dm.qphi), lam = float(dm.lambda);
+    const float De2 = dm.r32.De2, qphi = dm.r32.qphi, lam = dm.r32.lambda;
     const bool wX = WALLS && (dm.bc & LBPF_BC_WALL_X), wY = WALLS && (dm.bc & LBPF_BC_WALL_Y),
                wZ = WALLS && (dm.bc & LBPF_BC_WALL_Z);
     const bool dd = args.grad == LBPF_GRAD_DD;
