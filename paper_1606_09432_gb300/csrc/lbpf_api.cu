@@ -259,18 +259,19 @@ static int set_schedule(lbpf_ctx* c, int v, int seg)
 }
 
 // Whether the one-tile step (tile_kernel.cuh) replaces the march: 2D, no
-// advection, few sites.  us a step, march (shortest items) / tile: FP32 64^2 8.2
-// / 3.8, 128^2 9.2 / 4.0, 256^2 12.3 / 6.1, 512^2 20.4 / 14.3, 768^2 31.0 / 26.5,
-// 1024^2 46.9 / 49.5, 2048^2 155 / 178; FP16 512^2 22.4 / 16.1; FP64 with walls
-// (bound by FP64 arithmetic) 128^2 26 / 17, 800^2 272 / 225, 1200^2 523 / 493,
-// 2000^2 1201 / 1341.
+// advection, up to a few million sites.  us a step, march (its best schedule) /
+// tile: FP32 128^2 8.9 / 3.2, 256^2 10.9 / 4.1, 512^2 18.5 / 10.2, 1024^2 45.2 /
+// 37.0, 2048^2 148 / 137, 3000^2 289 / 288, 4096^2 522 / 535, 8000^2 1859 / 2030;
+// with walls 1000^2 49.0 / 45.8, 3000^2 330 / 373; FP16 512^2 19.5 / 10.9, 2048^2
+// 166 / 156, 4096^2 554 / 606; FP64 (bound by FP64 arithmetic) with walls 128^2 28
+// / 14, 800^2 240 / 193, 2000^2 1080 / 1146, periodic 1500^2 612 / 534.
 static bool tile_applies(const lbpf_ctx* c)
 {
     const char *kenv = getenv("LBPF_KERNEL"), *tenv = getenv("LBPF_AUTOTUNE");
     if (!c->L->tile_step || (c->kind & kStepAdvect) || (kenv && *kenv) || (tenv && atoi(tenv))) return false;
     double sites = 0;
     for (const DomainDev& d : c->dd) sites += (double)d.n;
-    return sites <= (c->rsize == 8 ? 2.0e6 : 7.0e5);
+    return sites <= (c->rsize == 8 ? 2.5e6 : c->kind & kStepWalls ? 2.0e6 : 4.5e6);
 }
 
 static std::string tune_key(const lbpf_ctx* c)

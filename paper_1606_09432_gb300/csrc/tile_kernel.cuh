@@ -10,11 +10,12 @@
 //
 // Why: a step of a small domain costs one chain of dependent memory latencies.
 // The march has five of them and a fetched work item per launch, the tile has
-// one: 128^2 FP32 4.0 us a step against 9.2 (22 with the march's former
-// eight-row items), at 512^2 14.3 against 20.4.  The ring of sites around a
+// one: 128^2 FP32 3.2 us a step against 8.9 (22 with the march's former
+// eight-row items), at 512^2 10.2 against 18.5.  The ring of sites around a
 // tile is computed more than once (1.42 coefficients a site), so large domains
-// keep the march (2048^2: 178 against 155 us).  A region of 16 rows measured
-// 5.5 us at 128^2 and 54 at 1024^2 (fewer, longer blocks).
+// keep the march (8000^2: 2030 against 1859 us).  A region of 16 rows measured
+// 4.1 us at 128^2 and 39.4 at 1024^2 (37.0; fewer, longer blocks), in FP64 25.6
+// at 128^2 against 13.9 and 400 at 1200^2 against 420.
 #pragma once
 
 #include "step_kernel.cuh"
