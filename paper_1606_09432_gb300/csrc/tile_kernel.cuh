@@ -1,12 +1,12 @@
 // One-tile form of the fused step for small 2D domains: the arithmetic of
 // step_kernel.cuh, operation by operation, with a block per tile instead of a
 // march (rounded explicitly where an expression leaves a choice, in the way the
-// march's compiled form rounds: the results are the same bits).  A thread owns one site of a 32 x 8 region: it requests everything
-// its site needs from global memory at once (phi and aux of the region plus
-// one site into shared memory, its pulled heat populations, its local and
-// pulled phase-field populations), then heat update, gradient, anisotropy and
-// coefficients of the site, one barrier, and the phase-field update of the
-// inner 30 x (RY - 2) sites.
+// march's compiled form rounds: the results are the same bits).  A thread owns one
+// site of a 32 x 8 region: it requests everything its site needs from global
+// memory at once (phi and aux of the region plus one site into shared memory, its
+// pulled heat populations, its local and pulled phase-field populations), then
+// heat update, gradient, anisotropy and coefficients of the site, one barrier, and
+// the phase-field update of the inner 30 x (RY - 2) sites.
 //
 // Why: a step of a small domain costs one chain of dependent memory latencies.
 // The march has five of them and a fetched work item per launch, the tile has

@@ -12,18 +12,17 @@
 //
 // Why: step_kernel is bound by instruction issue (1210 thread-instructions a
 // site with FP16 deviations, 73 % issue-active, 30 % of HBM at 256^3).  Apart,
-// the heat update is computed once per site instead of on every halo (108
+// the heat update is computed once per site instead of on every halo (111
 // instructions a site, bound by HBM: 127 us at 256^3, 66 % of the DRAM rate),
 // and both launches read and write four sites per instruction, which leaves
 // 408 instructions a site for the phase field.  The work field costs 8 of
 // 104 bytes a site.  Measured, us a step (step_kernel / this): D3Q15 FP16
 // 512^3 5289 / 3782 (stochastic rounding 7147 / 5936), 256^3 719 / 551, 351^3
 // with walls 2307 / 1682, 207 x 174 x 190 397 / 296; 256^3 D3Q19 838 / 690,
-// D3Q27 1260 / 980.  Rows that are not
-// whole vectors are padded in memory (DomainDev::px); a row's last partial vector
-// is computed whole, what falls into the padding is never read.  Full (FP32) storage measured 2 % slower
-// this way (the vectors in flight need twice the registers) and stays with
-// step_kernel.
+// D3Q27 1260 / 980.  Rows that are not whole vectors are padded in memory
+// (DomainDev::px); a row's last partial vector is computed whole, what falls into
+// the padding is never read.  Full (FP32) storage measured 2-8 % slower this way
+// (the vectors in flight need twice the registers) and stays with step_kernel.
 #pragma once
 
 #include <algorithm>
@@ -32,7 +31,6 @@
 
 namespace lbpf {
 
-// Four consecutive stored values.
 // Four consecutive stored deviations are loaded in two steps, so that many
 // loads can be in flight in few registers: raw bits, then the values.
 template <class T>
