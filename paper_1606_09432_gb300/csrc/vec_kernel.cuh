@@ -855,6 +855,9 @@ __device__ __forceinline__ void phi_vec_item(const StepArgs& args, const WorkIte
                 output_plane(z);
             } else {
                 end_sites(z);
+                // lanes without an end site leave end_sites early; the arrival is
+                // one instruction of the whole warp (bar is the aligned form)
+                __syncwarp();
                 asm volatile("bar.arrive 1, %0;" ::"n"(kVecLX * (kVecTY + 2)) : "memory");
             }
         }
