@@ -167,11 +167,10 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
         const int buf = s & 1, tap = s / nkb, c0 = (s - tap * nkb) * KC;
         if (s >= 2 && !mbar_wait_bounded(&s_mbar[buf], ((s - 2) >> 1) & 1)) {
             atomicOr(&g_conv_error, 1);
-            ok = false;
-            break;
+            ok = false;  // the buffer stays as it is; the block leaves together below
         }
         // A: row tid = x at the tap's neighbour, channels c0 .. c0 + KC
-        {
+        if (ok) {
             const int dy = tap / 3 - 1, dx = tap % 3 - 1;
             int yy = py + dy, xx = px + dx;
             yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
@@ -189,7 +188,7 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
             }
         }
         // B: 16-byte pieces w[tap][co][c0 + 8 k8 ..] -> [k8][co]
-        for (int e = tid; e < cout * (KC / 8); e += kConvM) {
+        for (int e = tid; ok && e < cout * (KC / 8); e += kConvM) {
             const int co = e % cout, k8 = e / cout;
             const __nv_bfloat16* g = w + ((size_t)tap * cout_all + co0 + co) * cin + c0 + 8 * k8;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -199,7 +198,8 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
         asm volatile("cp.async.commit_group;");
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
+        ok = __syncthreads_and(ok) != 0;
+        if (!ok) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t a0 = smem_u32(sA(buf)), b0 = smem_u32(sB(buf));
@@ -220,10 +220,11 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
         if (!done) atomicOr(&g_conv_error, 2);
     }
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok && done) {
+    if (__all_sync(0xffffffffu, ok && done)) {  // the loads below are the whole warp's
         float* out = y + p * cout_all + co0;
         for (int c = 0; c < cout; c += 8) {
             uint32_t r[8];
+            __syncwarp();
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                            "=r"(r[7])
@@ -474,7 +475,8 @@ __global__ void __launch_bounds__(halo_threads(MODE), MODE == kResident ? 2 : 1)
         int k = 0;
         for (int t = blockIdx.x; t < q.n_tiles; t += gridDim.x, ++k) {
             const int acc = k % q.nacc;
-            if (!mbar_wait_bounded(&s_afull[acc], (k / q.nacc) & 1)) {
+            // (the loads below are the whole warp's: its lanes go on or leave together)
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&s_afull[acc], (k / q.nacc) & 1))) {
                 atomicOr(&g_conv_error, 32);
                 break;
             }
@@ -487,6 +489,7 @@ __global__ void __launch_bounds__(halo_threads(MODE), MODE == kResident ? 2 : 1)
                 const int cw = cout - c0 < 32 ? cout - c0 : 32;  // 16 or 32 channels
                 for (int c = 0; c < cw; c += 16) {
                     uint32_t r[16];
+                    __syncwarp();
                     asm volatile(
                         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
                         "[%16];"
@@ -930,8 +933,7 @@ __global__ void __launch_bounds__(kConvM) conv3x3_wgrad_tc_kernel(const float* _
         const long long pb = p0 + (long long)s * kWgK;
         if (s >= 2 && !mbar_wait_bounded(&s_mbar[buf], ((s - 2) >> 1) & 1)) {
             atomicOr(&g_conv_error, 4);
-            ok = false;
-            break;
+            ok = false;  // the block leaves together below
         }
         if (tid < kWgK) {  // the stage's pixels and their neighbours at the tap
             const long long pp = pb + tid;
@@ -946,7 +948,8 @@ __global__ void __launch_bounds__(kConvM) conv3x3_wgrad_tc_kernel(const float* _
             }
             s_q[buf][tid] = q;
         }
-        __syncthreads();
+        ok = __syncthreads_and(ok) != 0;
+        if (!ok) break;
         // 16-byte pieces (channel row, 8 pixels) of A = dy and B = x at the
         // tap's neighbours.  Tiles of at least 128 channels: one row a thread,
         // its 64 pixels unrolled (more loads in flight); narrower tiles
@@ -1007,9 +1010,10 @@ __global__ void __launch_bounds__(kConvM) conv3x3_wgrad_tc_kernel(const float* _
         if (!done) atomicOr(&g_conv_error, 8);
     }
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok && done) {
+    if (__all_sync(0xffffffffu, ok && done)) {  // the loads below are the whole warp's
         for (int c = 0; c < nci; c += 8) {
             uint32_t r[8];
+            __syncwarp();
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                            "=r"(r[7])
@@ -1173,11 +1177,12 @@ __global__ void __launch_bounds__(kWgThreads) conv3x3_wgrad_halo_kernel(const Wg
         const bool done = mbar_wait_bounded(&s_done, 0);
         if (!done) atomicOr(&g_conv_error, 8);
         asm volatile("tcgen05.fence::after_thread_sync;");
-        if (ok && done && any) {
+        if (__all_sync(0xffffffffu, ok && done && any)) {  // the loads below are the whole warp's
             const int co = co0 + tid;  // this thread's TMEM lane = D row
             for (int tp = 0; tp < TAPS; ++tp)
                 for (int c = 0; c < q.nci; c += 16) {
                     uint32_t r[16];
+                    __syncwarp();
                     asm volatile(
                         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
                         "[%16];"

@@ -17,7 +17,7 @@ def code_lines(name):
     return [ln for ln in lines if ln]
 
 
-@pytest.mark.parametrize("name,instruction", [("vec_kernel.cuh", "bar.arrive")])
+@pytest.mark.parametrize("name,instruction", [("vec_kernel.cuh", "bar.arrive"), ("lbpf_nn.cu", "tcgen05.ld.sync")])
 def test_warp_is_converged_before(name, instruction):
     lines = code_lines(name)
     found = 0
