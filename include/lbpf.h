@@ -209,9 +209,10 @@ int lbpf_write_fields(lbpf_ctx* ctx, int domain, const void* phi, const void* u,
 /* Advance every domain by n_steps time steps (n_steps >= 0).  One step is
  * the phase-field scheme of Sec. 3.2 followed by the heat scheme of Sec. 3.1
  * with Q_u = (phi(t + dt) - phi(t)) / (2 dt), one kernel launch for all
- * domains (two where the vector form applies, see LBPF_Q_KERNEL).  On a non-default stream, runs of 16 steps are replayed from CUDA
- * graphs captured on first use (do not call lbpf_step while another capture
- * is active on the context's stream).  Asynchronous on the context's stream
+ * domains (two or more in the vector form, see LBPF_Q_STEP_FORM).  On a
+ * non-default stream, runs of 16 steps are replayed from CUDA graphs captured
+ * on first use (do not call lbpf_step while another capture is active on the
+ * context's stream).  Asynchronous on the context's stream
  * (except the first call of a context whose schedule is timed, see
  * lbpf_set_schedule); launch errors are returned, device errors surface at
  * the next synchronising call. */
@@ -316,34 +317,45 @@ typedef enum {
     LBPF_Q_DEVICE_BYTES = 3,   /* device memory held by the context                  */
     LBPF_Q_LAMBDA = 4,         /* lambda of domain 0 (after the lambda* rule)        */
     LBPF_Q_STEP_KERNELS = 5,   /* step-kernel launches issued by lbpf_step so far     */
-    LBPF_Q_TILE_ROWS = 6,      /* tile variant of the step kernel (autotuned): 8, 16 */
-    LBPF_Q_SEGMENT = 7,        /* z-planes (3D) or y-rows (2D) per work item          */
-    LBPF_Q_BLOCKS = 8,         /* resident blocks of the persistent step launch       */
-    LBPF_Q_KERNEL = 9          /* step kernel: 0 the library's choice, 1 staged.  The choice
-                                  (same results bit for bit): a march over tiles in one
-                                  launch; in 2D with few sites one launch with a block per
-                                  tile; in 3D with 16-bit deviation storage (one crystal, no
-                                  velocity, rows that fill 64-site segments) two launches
-                                  with four sites a thread.  The environment variable
-                                  LBPF_KERNEL at lbpf_create forces generic (the march),
-                                  vector (the last, wherever it can run) or staged (rows
-                                  brought to shared memory by asynchronous copies: 3D
-                                  D3Q15/D3Q19 domains with 16-bit deviation storage, nx a
-                                  multiple of 8 and >= 64, one crystal; slower on GB300) */
+    LBPF_Q_TILE_ROWS = 6,      /* tile variant of the march: 8, 16.  The other forms have
+                                  one tile each (vector 64 x 12 sites, one-tile 30 x 6):
+                                  there it is the variant last given to lbpf_set_schedule
+                                  and says nothing about the launches                 */
+    LBPF_Q_SEGMENT = 7,        /* z-planes (3D) or y-rows (2D) per work item (the mean
+                                  where items differ in length)                       */
+    LBPF_Q_BLOCKS = 8,         /* blocks of the step launch: resident blocks of the
+                                  persistent forms, one per tile in the one-tile form  */
+    LBPF_Q_KERNEL = 9,         /* step kernel: 0 the library's choice, 1 staged.  The choice
+                                  (same results bit for bit) is told by LBPF_Q_STEP_FORM.
+                                  The environment variable LBPF_KERNEL at lbpf_create forces
+                                  generic (the march), vector (wherever it can run) or
+                                  staged (rows brought to shared memory by asynchronous
+                                  copies: 3D D3Q15/D3Q19 domains with 16-bit deviation
+                                  storage, nx a multiple of 8 and >= 64, one crystal;
+                                  slower on GB300)                                    */
+    LBPF_Q_STEP_FORM = 10      /* form of the step the context takes: 0 the march over
+                                  tiles in one launch; 1 staged; 2 vector, four sites a
+                                  thread (3D, 16-bit deviation storage, one crystal, no
+                                  velocity, rows and planes that fill its tiles), one or
+                                  more heat launches (domains alike in size and walls that
+                                  follow one another share one) and a phase-field launch
+                                  a step; 3 one tile a block (2D, few sites, no velocity,
+                                  LBPF_AUTOTUNE not set to 1)                          */
 } lbpf_query_t;
 
 /* Override the work schedule of the step kernel.  Normally lbpf_create takes
  * a choice cached for the configuration (file LBPF_TUNE_CACHE, default
  * ~/.cache/lbpf_tune.txt) or a rule; configurations of >= 4e6 sites (or any,
- * with LBPF_AUTOTUNE=1; none with LBPF_AUTOTUNE=0) are then timed at the
- * first lbpf_step, on the live state, which that call leaves unchanged (it
+ * with LBPF_AUTOTUNE=1, which also keeps 2D contexts on the march: only its
+ * schedules are timed; none with LBPF_AUTOTUNE=0) are then timed at the first
+ * lbpf_step, on the live state, which that call leaves unchanged (it
  * synchronises the stream once and caches the choice).  The kernel marches
  * a tile along z (3D) or y (2D).  tile_rows is 8 or 16: in 3D the tile is 32
  * sites along x by tile_rows along y; in 2D it is one row of 16 * tile_rows
  * sites (128 or 256) along x.  segment (>= 1) is the number of z-planes (3D)
  * or y-rows (2D) per work item (tile_rows = 16 exists only for periodic
- * domains and the march).  The four-sites-a-thread form (LBPF_Q_KERNEL) has
- * one tile, 64 x 12 sites: there tile_rows has no effect.  A context on the
+ * domains and the march).  The four-sites-a-thread form (LBPF_Q_STEP_FORM 2)
+ * has one tile, 64 x 12 sites: there tile_rows has no effect.  A context on the
  * block-per-tile form in 2D goes back to the march, with the schedule given.
  * Results do not depend on the schedule; only speed does.  A performance knob
  * with no counterpart in the paper.

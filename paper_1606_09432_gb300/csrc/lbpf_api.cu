@@ -1033,6 +1033,7 @@ extern "C" int lbpf_query(const lbpf_ctx* c, int what, double* value)
     case LBPF_Q_SEGMENT: v = c->seg_len; break;
     case LBPF_Q_BLOCKS: v = c->n_blocks; break;
     case LBPF_Q_KERNEL: v = c->staged ? 1 : 0; break;
+    case LBPF_Q_STEP_FORM: v = c->staged ? 1 : c->vec ? 2 : c->tile ? 3 : 0; break;
     default: return fail(const_cast<lbpf_ctx*>(c), LBPF_EINVAL, "lbpf_query: unknown property %d", what);
     }
     *value = v;

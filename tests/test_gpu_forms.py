@@ -1,0 +1,88 @@
+"""Which form of the step a context takes (LBPF_Q_STEP_FORM): the bit-for-bit
+comparisons of test_gpu_vec.py and test_gpu_tile.py are worth something only
+where the two contexts take different forms, and the rules that choose a form
+are stated in sizes."""
+import pytest
+
+import test_gpu_vec as V
+from helpers import gpu_run
+from paper_1606_09432_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+MARCH, STAGED, VECTOR, TILE = range(4)
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_1606_09432_gb300 import build as B
+    from paper_1606_09432_gb300 import lbpf
+    B.build()
+    lbpf.load()
+    return lbpf
+
+
+def make(L, shapes, precision, lattice=None, bcs=None):
+    """A context of the given (nz, ny, nx) domains, unseeded."""
+    d3 = shapes[0][0] > 1
+    prm = {k: v for k, v in (W.C3D_PARAMS if d3 else W.C1_PARAMS).items() if k != "lam"}
+    cr = L.make_crystal(**(V.FORM if d3 else dict(kind=0, eps=0.05)))
+    doms = [L.make_domain(s[2], s[1], s[0], lam=10.0, crystals=[cr], bc=bcs[k] if bcs else 0, **dict(prm, delta=0.4))
+            for k, s in enumerate(shapes)]
+    return L.Solver(doms, (1 if d3 else 0) if lattice is None else lattice, L.LBPF_GRAD_DD, precision)
+
+
+def form(L, *args, **kw):
+    s = make(L, *args, **kw)
+    try:
+        return int(s.query(L.LBPF_Q_STEP_FORM))
+    finally:
+        s.close()
+
+
+@pytest.mark.parametrize("lattice", [1, 2, 3])
+@pytest.mark.parametrize("shape", V.SHAPES + [(9, 14, 74), (40, 37, 67), (256, 256, 256)])
+def test_comparisons_of_the_vector_step_compare_two_forms(L, monkeypatch, shape, lattice):
+    forms = []
+    for kernel in ("vector", "generic"):
+        monkeypatch.setenv("LBPF_KERNEL", kernel)
+        s = make(L, [shape], 2, lattice)
+        n0 = s.query(L.LBPF_Q_STEP_KERNELS)
+        s.step(3)
+        forms.append((int(s.query(L.LBPF_Q_STEP_FORM)), int(s.query(L.LBPF_Q_STEP_KERNELS) - n0)))
+        s.close()
+    assert forms == [(VECTOR, 6), (MARCH, 3)]
+
+
+@pytest.mark.parametrize("precision", range(5))
+@pytest.mark.parametrize("shape", [(1, 2, 2), (1, 7, 31), (1, 25, 61), (1, 40, 95), (1, 64, 128)])
+def test_comparisons_of_the_one_tile_step_compare_two_forms(L, monkeypatch, shape, precision):
+    forms = []
+    for kernel in ("", "generic"):
+        monkeypatch.setenv("LBPF_KERNEL", kernel)
+        forms.append(form(L, [shape], precision))
+    assert forms == [TILE, MARCH]
+
+
+def test_schedule_given_returns_to_the_march(L, monkeypatch):
+    monkeypatch.setenv("LBPF_KERNEL", "")
+    s = make(L, [(1, 33, 70)], 1)
+    assert s.query(L.LBPF_Q_STEP_FORM) == TILE
+    L.lbpf_set_schedule(s.ctx, 16, 5)
+    assert s.query(L.LBPF_Q_STEP_FORM) == MARCH and s.query(L.LBPF_Q_TILE_ROWS) == 16
+
+
+def test_cached_2d_schedule_is_taken_again(L, tmp_path, monkeypatch):
+    """A schedule timed on the 2D march is cached and read by the next context."""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("LBPF_TUNE_CACHE", str(cache))
+    monkeypatch.setenv("LBPF_KERNEL", "generic")
+    monkeypatch.setenv("LBPF_AUTOTUNE", "1")
+    s = gpu_run(L, 0, (1, 90, 130), W.C1_PARAMS, [dict(kind=0, eps=0.05)], seeds=[(65.0, 45.0, 0.0, 6.0, 0)], precision=1)
+    s.step(2)
+    key, v, seg = cache.read_text().split()
+    cache.write_text(f"{key} 1 {int(seg) + 3}\n")  # unlike any rule's choice
+    monkeypatch.setenv("LBPF_AUTOTUNE", "0")
+    s = gpu_run(L, 0, (1, 90, 130), W.C1_PARAMS, [dict(kind=0, eps=0.05)], seeds=[(65.0, 45.0, 0.0, 6.0, 0)], precision=1)
+    assert s.query(L.LBPF_Q_TILE_ROWS) == 16 and s.query(L.LBPF_Q_SEGMENT) == int(seg) + 3
+    assert s.query(L.LBPF_Q_STEP_FORM) == MARCH
