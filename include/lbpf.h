@@ -466,6 +466,13 @@ int lbpf_net_range_check(const float* phi, long long sites, float lo, float hi, 
  * LBPF_EINVAL; LBPF_ECUDA if the launch fails. */
 int lbpf_nn_conv3x3(const float* x, const void* wt, const float* bias, float* y, int n, int H, int W, int cin,
                     int cout, int relu, void* stream);
+/* The kernel lbpf_nn_conv3x3 takes for these sizes (host arithmetic, no GPU
+ * call): *form = 1 or 2 the halo kernel (an image tile with its rim in shared
+ * memory once for all taps; 1: the weights stay resident, 2: they stream), for H
+ * a multiple of 16, W of 8 and a halo that fits beside two stages of weights
+ * (362 cin + 256 (cout tile + 1) <= 209920 bytes is enough); 0 the gather
+ * kernel (a quarter of the speed at 384 -> 256).  Errors as above. */
+int lbpf_nn_conv3x3_form(int H, int W, int cin, int cout, int* form);
 /* Weight gradient of that layer, added to dwt:
  *   dwt[tap][co][ci] += sum_n,h,w dy[n][h][w][co] x[n][h'][w'][ci]
  * (h', w' as above), on the tensor cores with x and dy rounded to BF16 (to

@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
 }
 
 // Halo form of the same convolution for images whose H is a multiple of 16
-// and W of 8.  A tile is 16 x 8 pixels (M = 128: tile row = 8-row group, pixel
+// and W of 8, and layers whose halo fits in shared memory beside two stages of
+// weights (halo_plan: cin up to 512).  A tile is 16 x 8 pixels (M = 128: tile row = 8-row group, pixel
 // in the row = row of the core matrix); its 18 x 10 halo of all cin channels
 // is converted to BF16 once (layout [8-channel slice][halo pixel][8]), and
 // every tap is a matrix descriptor over it: start at the tap's offset, SBO =
@@ -758,10 +759,13 @@ static bool halo_plan(HaloArgs& q, size_t& smem, int& per_sm)
     smem = q.nbuf * halo + all_w + out;
     if (smem > kSmemMax) {
         // the weights stream; a second halo buffer only beside four stages (and
-        // 1 KB for the TMA form's alignment)
+        // 1 KB for the TMA form's alignment).  Two stages of a wide tile beside one
+        // halo are enough (us at 256^2, gather kernel / this: 384 -> 256 565 / 135,
+        // 320 -> 256 478 / 117, 384 -> 512 1033 / 224, 448 -> 128 559 / 125, 512 -> 64
+        // 670 / 121); below that only the gather kernel's small stages fit
         const size_t rest = kSmemMax - out - 1024;
         q.nbuf = 2 * halo + 4 * st <= rest ? 2 : 1;
-        if (q.nbuf * halo + 3 * st > rest) return false;
+        if (q.nbuf * halo + 2 * st > rest) return false;
         const size_t n = (rest - q.nbuf * halo) / st;
         q.wst = (int)(n < kMaxWStages ? n : kMaxWStages);
         smem = q.nbuf * halo + q.wst * st + out + 1024;
@@ -777,6 +781,20 @@ static bool halo_plan(HaloArgs& q, size_t& smem, int& per_sm)
     const size_t least = (size_t)(228 * 1024) / (per_sm + 1) - 1024;  // no more blocks than that fit
     if (smem < least) smem = least;
     return true;
+}
+
+int conv3x3_form(int H, int W, int cin, int cout_all)
+{
+    const int n_tiles = (cout_all + 255) / 256;
+    HaloArgs q;
+    q.H = H;
+    q.W = W;
+    q.cin = cin;
+    q.cout = cout_all / n_tiles;
+    q.KC = conv_kc(cin);
+    size_t smem = 0;
+    int per_sm = 1;
+    return !halo_plan(q, smem, per_sm) ? 0 : q.wst ? 2 : 1;
 }
 
 cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, const __nv_bfloat16* w, const float* bias,

@@ -11,8 +11,13 @@ namespace lbpf_nn {
 // channels, each a multiple of 16.  w: BF16 [tap][cout][cin].
 cudaError_t conv3x3_fwd(const float* x, const __nv_bfloat16* w, const float* bias, float* y, int N, int H, int W,
                         int cin, int cout, int relu, cudaStream_t s);
-// Error word of the convolution kernels (1, 2: a bounded wait of a block
-// gave up; -1: unreadable); 0 when every wait completed.
+// The kernel conv3x3_fwd takes for these (valid) sizes: 0 the gather kernel, 1
+// the halo kernel with resident weights, 2 with streamed weights.
+int conv3x3_form(int H, int W, int cin, int cout);
+// Error word of the convolution kernels, a bit mask of the waits that gave up
+// (forward: 1, 2 gather kernel, 16 halo loaders, 32 epilogue, 64 MMA issue, 128
+// weight stream; weight gradient: 4 loaders, 8 the sums, 256 MMA issue); 0 when
+// every wait completed, -1 when it cannot be read.
 int conv_error();
 // wt[tap][ci][co] = w[8 - tap][co][ci]: weights of the data-gradient convolution.
 cudaError_t flip_weights(const __nv_bfloat16* w, __nv_bfloat16* wt, int cin, int cout, cudaStream_t s);

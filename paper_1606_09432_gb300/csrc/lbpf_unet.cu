@@ -449,6 +449,14 @@ extern "C" int lbpf_nn_conv3x3(const float* x, const void* wt, const float* bias
                : LBPF_ECUDA;
 }
 
+extern "C" int lbpf_nn_conv3x3_form(int H, int W, int cin, int cout, int* form)
+{
+    const int n_tiles = (cout + 255) / 256;
+    if (!form || H < 1 || W < 1 || cin < 16 || cout < 16 || cin % 16 || cout % (16 * n_tiles)) return LBPF_EINVAL;
+    *form = conv3x3_form(H, W, cin, cout);
+    return LBPF_OK;
+}
+
 extern "C" int lbpf_nn_conv3x3_wgrad(const float* x, const float* dy, float* dwt, int n, int H, int W, int cin,
                                      int cout, void* stream)
 {

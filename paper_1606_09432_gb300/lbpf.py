@@ -33,7 +33,7 @@ EXPORTED = ["lbpf_create", "lbpf_seed", "lbpf_write_fields", "lbpf_step", "lbpf_
             "lbpf_net_create", "lbpf_net_create_arch", "lbpf_net_destroy", "lbpf_net_last_error", "lbpf_net_num_params",
             "lbpf_net_get_params", "lbpf_net_set_params", "lbpf_net_forward", "lbpf_net_backward",
             "lbpf_net_train_step", "lbpf_net_assemble", "lbpf_net_apply", "lbpf_net_delta",
-            "lbpf_net_range_check", "lbpf_net_set_loss_weight", "lbpf_nn_conv3x3", "lbpf_nn_conv3x3_wgrad",
+            "lbpf_net_range_check", "lbpf_net_set_loss_weight", "lbpf_nn_conv3x3", "lbpf_nn_conv3x3_form", "lbpf_nn_conv3x3_wgrad",
             "lbpf_nn_conv_error"]
 
 
@@ -105,6 +105,7 @@ def load(path: str = LIB_PATH):
     lib.lbpf_net_delta.argtypes = [vp, vp, vp, vp, vp, C.c_longlong, vp]
     lib.lbpf_net_range_check.argtypes = [vp, C.c_longlong, C.c_float, C.c_float, vp, vp]
     lib.lbpf_nn_conv3x3.argtypes = [vp, vp, vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, vp]
+    lib.lbpf_nn_conv3x3_form.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
     lib.lbpf_nn_conv3x3_wgrad.argtypes = [vp, vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, vp]
     lib.lbpf_nn_conv_error.argtypes = [C.POINTER(C.c_int)]
     for name in EXPORTED:
@@ -452,6 +453,16 @@ def nn_conv3x3(x, wt, bias, y, relu=False, stream=None):
                                 cin, cout, int(bool(relu)), C.c_void_p(stream) if stream else None)
     if rc != LBPF_OK:
         raise LbpfError(rc, "lbpf_nn_conv3x3 failed")
+
+
+def nn_conv3x3_form(H, W, cin, cout):
+    """Kernel nn_conv3x3 takes for these sizes: 0 gather, 1 halo with resident
+    weights, 2 halo with streamed weights."""
+    f = C.c_int(0)
+    rc = load().lbpf_nn_conv3x3_form(H, W, cin, cout, C.byref(f))
+    if rc != LBPF_OK:
+        raise LbpfError(rc, "lbpf_nn_conv3x3_form failed")
+    return f.value
 
 
 def nn_conv3x3_wgrad(x, dy, dwt, stream=None):
