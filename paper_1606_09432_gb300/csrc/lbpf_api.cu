@@ -729,13 +729,31 @@ extern "C" int lbpf_seed(lbpf_ctx* c, int domain, const lbpf_seed_t* seeds, int 
 // Sites of a domain (its arrays may hold row padding besides).
 static long long sites_of(const DomainDev& h) { return (long long)h.nx * h.ny * h.nz; }
 
-// A field of the arithmetic type between arrays of row pitches dp and sp (elements).
-static cudaError_t copy_rows(lbpf_ctx* c, const DomainDev& h, void* dst, int dp, const void* src, int sp,
-                             cudaMemcpyKind kind)
+// A field of the arithmetic type between an array of the context (own, row pitch
+// h.px) and a dense one of the caller's, host or device.  Padded rows (only with
+// FP32 arithmetic) go through the context's scratch on their way from or to the
+// host, in one dense copy.
+static cudaError_t put_field(lbpf_ctx* c, const DomainDev& h, void* own, const void* from, cudaMemcpyKind kind)
 {
-    const size_t row = (size_t)h.nx * c->rsize, rows = (size_t)h.ny * h.nz;
-    if (dp == sp) return cudaMemcpyAsync(dst, src, row * rows, kind, c->stream);
-    return cudaMemcpy2DAsync(dst, (size_t)dp * c->rsize, src, (size_t)sp * c->rsize, row, rows, kind, c->stream);
+    const size_t bytes = (size_t)sites_of(h) * c->rsize;
+    if (h.px == h.nx) return cudaMemcpyAsync(own, from, bytes, kind, c->stream);
+    if (kind == cudaMemcpyHostToDevice || ((uintptr_t)from & 3)) {
+        const cudaError_t e = cudaMemcpyAsync(c->scratch, from, bytes, kind, c->stream);
+        if (e != cudaSuccess) return e;
+        from = c->scratch;
+    }
+    return launch_copy_rows(static_cast<float*>(own), h.px, static_cast<const float*>(from), h.nx, h.nx,
+                            (long long)h.ny * h.nz, c->stream);
+}
+static cudaError_t get_field(lbpf_ctx* c, const DomainDev& h, void* to, const void* own, cudaMemcpyKind kind)
+{
+    const size_t bytes = (size_t)sites_of(h) * c->rsize;
+    if (h.px == h.nx) return cudaMemcpyAsync(to, own, bytes, kind, c->stream);
+    const bool direct = kind == cudaMemcpyDeviceToDevice && !((uintptr_t)to & 3);
+    const cudaError_t e = launch_copy_rows(static_cast<float*>(direct ? to : c->scratch), h.nx,
+                                           static_cast<const float*>(own), h.px, h.nx, (long long)h.ny * h.nz, c->stream);
+    if (e != cudaSuccess || direct) return e;
+    return cudaMemcpyAsync(to, c->scratch, bytes, kind, c->stream);
 }
 
 extern "C" int lbpf_write_fields(lbpf_ctx* c, int domain, const void* phi, const void* u, const int* index,
@@ -747,8 +765,8 @@ extern "C" int lbpf_write_fields(lbpf_ctx* c, int domain, const void* phi, const
     if ((rc = sync_state(c))) return rc;
     const DomainDev& h = c->dd[domain];
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(copy_rows(c, h, h.phi[c->cur], h.px, phi, h.nx, kind));
-    CK(copy_rows(c, h, h.aux[c->acur], h.px, u, h.nx, kind));
+    CK(put_field(c, h, h.phi[c->cur], phi, kind));
+    CK(put_field(c, h, h.aux[c->acur], u, kind));
     if (h.use_index) {
         if (index) {
             CK(cudaMemcpyAsync(c->scratch, index, sizeof(int) * h.n, kind, c->stream));
@@ -873,7 +891,7 @@ extern "C" int lbpf_read_fields(lbpf_ctx* c, int domain, unsigned mask, void* ou
         void* dst = out_on_device ? static_cast<void*>(o) : c->scratch;
         switch (bit) {
         case LBPF_READ_PHI:
-            CK(copy_rows(c, h, o, h.nx, h.phi[c->cur], h.px, kind));
+            CK(get_field(c, h, o, h.phi[c->cur], kind));
             dst = nullptr;
             break;
         case LBPF_READ_U: CK(c->L->read_u(c->d_dd + domain, c->cur, c->fcur, c->acur, dst, c->stream)); break;

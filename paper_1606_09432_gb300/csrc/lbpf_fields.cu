@@ -145,6 +145,25 @@ cudaError_t launch_reduce(const void* phi, const void* u, long long n, int preci
     return cudaGetLastError();
 }
 
+// A field between arrays of row pitches dp and sp: 64 threads a row, four rows a
+// block.  Memory bound; it replaces pitched copies, whose rows the copy engines
+// take one by one (351^3, rows of 351 in 352 floats, phi and u from pinned host
+// memory 12.3 ms, 3.4 with this behind a dense copy, 3.25 where rows are dense;
+// phi to the host 1.1, 1.0 and 0.9).
+__global__ void __launch_bounds__(256) copy_rows_kernel(float* __restrict__ dst, int dp, const float* __restrict__ src,
+                                                        int sp, int nx, long long rows)
+{
+    for (long long r = blockIdx.x * 4LL + threadIdx.y; r < rows; r += gridDim.x * 4LL)
+        for (int x = threadIdx.x; x < nx; x += 64) dst[r * dp + x] = src[r * sp + x];
+}
+
+cudaError_t launch_copy_rows(float* dst, int dp, const float* src, int sp, int nx, long long rows, cudaStream_t s)
+{
+    const long long b = (rows + 3) / 4;
+    copy_rows_kernel<<<(unsigned)(b < 152 * 16 ? b : 152 * 16), dim3(64, 4), 0, s>>>(dst, dp, src, sp, nx, rows);
+    return cudaGetLastError();
+}
+
 // Tip crossings: block w scans the ray of axis w/2, sign +1 (even w) or -1,
 // k = 0 .. len-1 with len = half the domain length along the axis; the
 // outermost k with phi_k >= 0 > phi_{k+1} gives k + phi_k / (phi_k - phi_{k+1}).

@@ -526,6 +526,8 @@ constexpr int kReduceBlocks = 304;
 // walled coordinate (they lie on the mirror planes).
 cudaError_t launch_reduce(const void* phi, const void* u, long long n, int precision, double* partial, double* out,
                           cudaStream_t s, int nx = 0, int ny = 0, int nz = 0, int bc = 0, int dim = 3, int px = 0);
+// rows of nx floats from row pitch sp to row pitch dp (device memory)
+cudaError_t launch_copy_rows(float* dst, int dp, const float* src, int sp, int nx, long long rows, cudaStream_t s);
 // Tip crossings along +-x, +-y, +-z from (cx, cy, cz); out[6].  Rays cover
 // half the domain on periodic axes and run to the wall on walled ones.
 cudaError_t launch_tips(const void* phi, int nx, int ny, int nz, int cx, int cy, int cz, int dim, int precision,

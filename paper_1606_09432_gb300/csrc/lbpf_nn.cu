@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kConvM) conv3x3_tc_kernel(const float* __restr
 
 // Halo form of the same convolution for images whose H is a multiple of 16
 // and W of 8, and layers whose halo fits in shared memory beside two stages of
-// weights (halo_plan: cin up to 512).  A tile is 16 x 8 pixels (M = 128: tile row = 8-row group, pixel
+// weights (halo_plan).  A tile is 16 x 8 pixels (M = 128: tile row = 8-row group, pixel
 // in the row = row of the core matrix); its 18 x 10 halo of all cin channels
 // is converted to BF16 once (layout [8-channel slice][halo pixel][8]), and
 // every tap is a matrix descriptor over it: start at the tap's offset, SBO =
