@@ -485,11 +485,20 @@ struct LauncherImpl {
         }
         return nb > 0 ? nb : 1;
     }
-    static cudaError_t heat_sync(const DomainDev* d, int n, int cur, int fcur, int acur, cudaStream_t s)
+    // One launch for the domains (grid y), each with blocks for the largest: up
+    // to eight an SM, and where there are many domains a block for 2048 sites of
+    // it, but one an SM at least (a read after a step of 384^3 FP32 beside four
+    // domains of 32^3: 4.61 ms with 152 blocks a domain, 2.18 with 1216)
+    static cudaError_t heat_sync(const DomainDev* h, const DomainDev* d, int n, int cur, int fcur, int acur,
+                                 cudaStream_t s)
     {
-        for (int k = 0; k < n; k += 65535) {  // one launch for the domains (grid y)
+        for (int k = 0; k < n; k += 65535) {
             const int m = n - k < 65535 ? n - k : 65535;
-            heat_sync_kernel<PL, UL, S><<<dim3(m > 4 ? 152 : 152 * 8, m), 256, 0, s>>>(d + k, cur, fcur, acur);
+            long long most = 0;
+            for (int j = k; j < k + m; ++j) most = h[j].n > most ? h[j].n : most;
+            const long long want = m > 4 ? (most + 2047) / 2048 : 152 * 8;
+            const unsigned bx = (unsigned)(want < 152 ? 152 : want > 152 * 8 ? 152 * 8 : want);
+            heat_sync_kernel<PL, UL, S><<<dim3(bx, m), 256, 0, s>>>(d + k, cur, fcur, acur);
         }
         return cudaGetLastError();
     }

@@ -682,7 +682,7 @@ static int sync_state(lbpf_ctx* c)
         a.collide = 1;
         CK(c->L->heat_vec(c->dd.data(), c->d_dd, c->n_domains, a, c->stream));
     } else {
-        CK(c->L->heat_sync(c->d_dd, c->n_domains, c->cur, c->fcur, c->acur, c->stream));
+        CK(c->L->heat_sync(c->dd.data(), c->d_dd, c->n_domains, c->cur, c->fcur, c->acur, c->stream));
     }
     c->fcur ^= 1;
     if (c->Sg != c->Qg) c->acur ^= 1;

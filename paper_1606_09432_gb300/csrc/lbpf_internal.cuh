@@ -490,9 +490,9 @@ struct Launchers {
     // The one-tile step (tile_kernel.cuh) over n_items tiles of 30 x 6 sites;
     // nullptr in 3D.
     cudaError_t (*tile_step)(int walls, const StepArgs& a, cudaStream_t s);
-    // Heat step alone, lagged -> synced state of n domains (f^{n-1}, aux^{n-1},
-    // phi^n -> f^n [+ aux^n]).
-    cudaError_t (*heat_sync)(const DomainDev* d, int n, int cur, int fcur, int acur, cudaStream_t s);
+    // Heat step alone, lagged -> synced state of n domains (host copies h, d on
+    // the device; f^{n-1}, aux^{n-1}, phi^n -> f^n [+ aux^n]).
+    cudaError_t (*heat_sync)(const DomainDev* h, const DomainDev* d, int n, int cur, int fcur, int acur, cudaStream_t s);
     // Populations at equilibrium from the phi field in phi[cur] and u in
     // aux[acur] (index in I[cur]); writes g[cur], f[fcur] (+ aux in place).
     cudaError_t (*equilibrate)(const DomainDev* d, int cur, int fcur, int acur, int grad, int finalize_index,
