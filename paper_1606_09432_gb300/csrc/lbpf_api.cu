@@ -438,7 +438,11 @@ static int autotune(lbpf_ctx* c)
 // rows and planes within a launch grid's limits; it pays where its 64-site row segments are at least 0.6 full and there is work
 // for more than a wave of blocks (FP16, us a step, one launch / vector: 32^3 14.5
 // / 25.1, 64^3 29.7 / 29.1, 96^3 56.0 / 52.8, 128^3 115 / 85, 207x174x190 397 /
-// 296, 351^3 walls 2307 / 1682; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201).
+// 296, 351^3 walls 2307 / 1682; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201),
+// and where the domains share their heat launches (heat_grid): one more launch a
+// step costs 3 to 6 us, which takes half a million sites to earn (one launch /
+// vector with a heat launch a domain, walls alternating: 64 domains of 48^3 549 /
+// 547, 64 of 64^3 902 / 983, 16 of 96^3 755 / 746, 8 of 128^3 866 / 674).
 // LBPF_KERNEL: "vector" wherever it can, any other value never.
 static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_domains)
 {
@@ -446,6 +450,7 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
     const bool forced = kenv && strcmp(kenv, "vector") == 0;
     if (!L->heat_vec || (kenv && *kenv && !forced)) return false;
     double sites = 0, slots = 0;
+    std::vector<DomainDev> sizes(n_domains);  // what heat_grid looks at
     for (int k = 0; k < n_domains; ++k) {
         const lbpf_domain& d = domains[k];
         if (d.nx < 8 || (long long)((d.nx + 3) / 4 * 4) * d.ny * d.nz >= (1LL << 31) || d.n_crystals > 1 ||
@@ -453,8 +458,13 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
             return false;
         sites += (double)d.nx * d.ny * d.nz;
         slots += (double)((d.nx + kVecTX - 1) / kVecTX * kVecTX) * d.ny * d.nz;
+        sizes[k].px = (d.nx + 3) / 4 * 4;
+        sizes[k].ny = d.ny;
+        sizes[k].nz = d.nz;
+        sizes[k].bc = d.bc;
     }
-    return forced || (sites >= 2e5 && sites >= 0.6 * slots);
+    return forced || (sites >= 2e5 && sites >= 0.6 * slots &&
+                      L->heat_vec_launches(sizes.data(), n_domains) - 1 <= sites / 5e5);
 }
 
 // lbpf_create with the vector step where it applies, or (vec false) never.

@@ -86,3 +86,15 @@ def test_cached_2d_schedule_is_taken_again(L, tmp_path, monkeypatch):
     s = gpu_run(L, 0, (1, 90, 130), W.C1_PARAMS, [dict(kind=0, eps=0.05)], seeds=[(65.0, 45.0, 0.0, 6.0, 0)], precision=1)
     assert s.query(L.LBPF_Q_TILE_ROWS) == 16 and s.query(L.LBPF_Q_SEGMENT) == int(seg) + 3
     assert s.query(L.LBPF_Q_STEP_FORM) == MARCH
+
+
+@pytest.mark.parametrize("shapes,bcs,want", [
+    ([(64, 64, 64)] * 64, [7 * (k % 2) for k in range(64)], MARCH),  # a heat launch a domain: more than they earn
+    ([(64, 64, 64)] * 64, None, VECTOR),
+    ([(64, 64, 64)] * 64, [7 * (k // 32) for k in range(64)], VECTOR),
+    ([(64, 64, 64), (8, 12, 64)] * 32, None, VECTOR),  # pairs of unlike domains share a launch
+    ([(128, 128, 128)] * 8, [7 * (k % 2) for k in range(8)], VECTOR),
+])
+def test_heat_launches_count_in_the_choice_of_the_vector_step(L, monkeypatch, shapes, bcs, want):
+    monkeypatch.setenv("LBPF_KERNEL", "")
+    assert form(L, shapes, 2, bcs=bcs) == want
