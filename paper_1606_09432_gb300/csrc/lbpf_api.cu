@@ -435,10 +435,13 @@ static int autotune(lbpf_ctx* c)
 
 // Whether the context takes the vector step.  It can where every domain is 3D
 // with 16-bit deviations, one crystal, no advection, site indices in 31 bits and
-// rows and planes within a launch grid's limits; it pays where its 64-site row segments are at least 0.6 full and there is work
-// for more than a wave of blocks (FP16, us a step, one launch / vector: 32^3 14.5
+// rows and planes within a launch grid's limits; it pays where its 64-site row
+// segments are at least 0.6 full and its 64 x 12 tiles 0.5, and there is work for
+// more than a wave of blocks (FP16, us a step, one launch / vector: 32^3 14.5
 // / 25.1, 64^3 29.7 / 29.1, 96^3 56.0 / 52.8, 128^3 115 / 85, 207x174x190 397 /
-// 296, 351^3 walls 2307 / 1682; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201),
+// 296, 351^3 walls 2307 / 1682; nx = 24, 24x400x400, 266 / 325; nx = 40 271 / 201;
+// rows in y: 512x2x500 55 / 71, 128x2x1000 D3Q27 45 / 73, 512x4x500 71 / 80, 512x6x500
+// 94 / 86, 256x13x256 62 / 56),
 // and where the domains share their heat launches (heat_grid): one more launch a
 // step costs 3 to 6 us, which takes half a million sites to earn (one launch /
 // vector with a heat launch a domain, walls alternating: 64 domains of 48^3 549 /
@@ -449,7 +452,7 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
     const char* kenv = getenv("LBPF_KERNEL");
     const bool forced = kenv && strcmp(kenv, "vector") == 0;
     if (!L->heat_vec || (kenv && *kenv && !forced)) return false;
-    double sites = 0, slots = 0;
+    double sites = 0, slots = 0, tiles = 0;
     std::vector<DomainDev> sizes(n_domains);  // what heat_grid looks at
     for (int k = 0; k < n_domains; ++k) {
         const lbpf_domain& d = domains[k];
@@ -457,13 +460,15 @@ static bool vec_applies(const Launchers* L, const lbpf_domain* domains, int n_do
             d.adv[0] != 0.0 || d.adv[1] != 0.0 || d.adv[2] != 0.0 || d.ny > 65535 * kHeatY || d.nz > 65535)
             return false;
         sites += (double)d.nx * d.ny * d.nz;
-        slots += (double)((d.nx + kVecTX - 1) / kVecTX * kVecTX) * d.ny * d.nz;
+        const double segments = (double)((d.nx + kVecTX - 1) / kVecTX) * d.nz;
+        slots += segments * kVecTX * d.ny;
+        tiles += segments * ((d.ny + kVecTY - 1) / kVecTY);
         sizes[k].px = (d.nx + 3) / 4 * 4;
         sizes[k].ny = d.ny;
         sizes[k].nz = d.nz;
         sizes[k].bc = d.bc;
     }
-    return forced || (sites >= 2e5 && sites >= 0.6 * slots &&
+    return forced || (sites >= 2e5 && sites >= 0.6 * slots && sites >= 0.5 * kVecTX * kVecTY * tiles &&
                       L->heat_vec_launches(sizes.data(), n_domains) - 1 <= sites / 5e5);
 }
 

@@ -98,3 +98,12 @@ def test_cached_2d_schedule_is_taken_again(L, tmp_path, monkeypatch):
 def test_heat_launches_count_in_the_choice_of_the_vector_step(L, monkeypatch, shapes, bcs, want):
     monkeypatch.setenv("LBPF_KERNEL", "")
     assert form(L, shapes, 2, bcs=bcs) == want
+
+
+@pytest.mark.parametrize("shape,want", [((500, 2, 512), MARCH), ((1000, 2, 128), MARCH), ((300, 5, 200), MARCH),
+                                        ((500, 6, 512), VECTOR), ((256, 13, 256), VECTOR), ((64, 64, 64), VECTOR),
+                                        ((400, 400, 40), VECTOR), ((400, 400, 24), MARCH), ((40, 40, 40), MARCH)])
+@pytest.mark.parametrize("lattice", [1, 3])
+def test_vector_step_where_its_tiles_are_full(L, monkeypatch, shape, lattice, want):
+    monkeypatch.setenv("LBPF_KERNEL", "")
+    assert form(L, [shape], 2, lattice) == want
