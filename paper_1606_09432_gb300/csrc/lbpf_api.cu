@@ -265,13 +265,41 @@ static int set_schedule(lbpf_ctx* c, int v, int seg)
 // with walls 1000^2 49.0 / 45.8, 3000^2 330 / 373; FP16 512^2 19.5 / 10.9, 2048^2
 // 166 / 156, 4096^2 554 / 606; FP64 (bound by FP64 arithmetic) with walls 128^2 28
 // / 14, 800^2 240 / 193, 2000^2 1080 / 1146, periodic 1500^2 612 / 534.
+// Within that, where its estimated time is the shorter one, since domains that
+// fill neither the tiles' 30 x 6 sites nor the march's 128-site strips cost each
+// form differently.  A tile costs FP32 5.95 ns, 16 bits 6.9, FP64 41 (with walls 1.3
+// times that), whatever its columns, up to a quarter less with fewer rows.  The
+// march costs its rows (an item's and three before them) on all resident blocks,
+// each the more the more warps of the strip have sites (FP32 1.9 + 0.6 us a warp, 16
+// bits 1.8 + 0.8, FP64 4 + 7.5; with walls 1.25 times that), and at least one item.
+// Batches, march / tile: FP32 3000 of 128 x 7 102 / 164, 200 of 128^2 124 / 132, 1000
+// of 64^2 191 / 197, 60 of 256^2 143 / 138, 1000 of 32^2 93 / 71; FP16 107 / 195, 130 /
+// 151, 203 / 231, 158 / 160, 84 / 69; FP64 1500 of 128 x 7 427 / 453, 500 of 64^2 612 /
+// 701, 1000 of 32^2 416 / 481, 100 of 128^2 491 / 471; FP32 31 x 100000 247 / 178,
+// 100000 x 7 38 / 30; with walls FP32 1200^2 80 / 64, 1400^2 90 / 85, 30 of 256^2 94 /
+// 92, FP16 1400^2 97 / 78.
 static bool tile_applies(const lbpf_ctx* c)
 {
     const char *kenv = getenv("LBPF_KERNEL"), *tenv = getenv("LBPF_AUTOTUNE");
     if (!c->L->tile_step || (c->kind & kStepAdvect) || (kenv && *kenv) || (tenv && atoi(tenv))) return false;
-    double sites = 0;
-    for (const DomainDev& d : c->dd) sites += (double)d.n;
-    return sites <= (c->rsize == 8 ? 2.5e6 : c->kind & kStepWalls ? 2.0e6 : 4.5e6);
+    const bool walls = (c->kind & kStepWalls) != 0;
+    const int type = c->rsize == 8 ? 0 : c->ssize == 4 ? 1 : 2;
+    const double tile_us[3] = {0.041, 0.00595, 0.0069}, row_us[3] = {4.0, 1.9, 1.8}, warp_us[3] = {7.5, 0.6, 0.77};
+    const int seg = default_segment(c, 0), TX = kTileRX - 2, TY = kTileRY - 2, SX = kStripX[0];
+    auto strip_row = [&](int w) { return w > 0 ? row_us[type] + (w + 31) / 32 * warp_us[type] : 0.0; };
+    double sites = 0, tile = 0, march = 0, item = 0;
+    for (const DomainDev& d : c->dd) {
+        sites += (double)d.n;
+        // full tile rows, and the last one
+        const int th = d.ny % TY;
+        tile += (d.nx + TX - 1) / TX * (d.ny / TY + (th ? 0.6 + 0.4 * (th + 2) / kTileRY : 0.0));
+        march += (d.ny + 3.0 * ((d.ny + seg - 1) / seg)) * (d.nx / SX * strip_row(SX) + strip_row(d.nx % SX));
+        item = std::max(item, (std::min(seg, d.ny) + 3) * strip_row(std::min(d.nx, SX)));
+    }
+    if (sites > (c->rsize == 8 ? 2.5e6 : walls ? 2.0e6 : 4.5e6)) return false;
+    tile *= tile_us[type] * (walls ? 1.3 : 1.0);
+    march = std::max(march / ((double)blocks_per_sm(c, 0) * c->sms), item) * (walls ? 1.25 : 1.0);
+    return tile <= march;
 }
 
 static std::string tune_key(const lbpf_ctx* c)

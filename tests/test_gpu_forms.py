@@ -107,3 +107,26 @@ def test_heat_launches_count_in_the_choice_of_the_vector_step(L, monkeypatch, sh
 def test_vector_step_where_its_tiles_are_full(L, monkeypatch, shape, lattice, want):
     monkeypatch.setenv("LBPF_KERNEL", "")
     assert form(L, [shape], 2, lattice) == want
+
+
+BATCHES = [((1, 7, 128), 3000, (MARCH, MARCH, MARCH)), ((1, 128, 128), 200, (None, MARCH, MARCH)),
+           ((1, 64, 64), 500, (MARCH, None, MARCH)), ((1, 32, 32), 1000, (MARCH, TILE, TILE)),
+           ((1, 256, 256), 30, (TILE, TILE, TILE)), ((1, 64, 64), 1, (TILE, TILE, TILE)), ((1, 2, 2), 1, (TILE, TILE, TILE)),
+           ((1, 800, 800), 1, (TILE, TILE, TILE)), ((1, 2048, 2048), 1, (MARCH, TILE, TILE)),
+           ((1, 3000, 3000), 1, (MARCH, MARCH, MARCH)), ((1, 100000, 31), 1, (None, TILE, TILE))]
+
+
+@pytest.mark.parametrize("shape,count,want", BATCHES)
+def test_one_tile_step_where_its_tiles_cost_less(L, monkeypatch, shape, count, want):
+    """FP64, FP32, FP16; None: over the FP64 limit of sites, or too close to call."""
+    monkeypatch.setenv("LBPF_KERNEL", "")
+    for precision, w in enumerate(want):
+        if w is not None:
+            assert form(L, [shape] * count, precision) == w, precision
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_one_tile_step_with_walls(L, monkeypatch, precision):
+    monkeypatch.setenv("LBPF_KERNEL", "")
+    assert form(L, [(1, 1000, 1000)], precision, bcs=[3]) == TILE
+    assert form(L, [(1, 7, 128)] * 1500, precision, bcs=[3] * 1500) == MARCH
