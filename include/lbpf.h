@@ -424,7 +424,8 @@ int lbpf_net_set_params(lbpf_net* net, const float* host);
 /* y (N, H, W, 2) = network(x (N, H, W, 5)); y may be NULL (output kept). */
 int lbpf_net_forward(lbpf_net* net, const float* x, float* y);
 /* Parameter gradients of sum(out * dy) after a forward pass (read them with
- * lbpf_net_get_params(which = 1)). */
+ * lbpf_net_get_params(which = 1)).  Bias and head gradients repeat bit for bit;
+ * the 3x3 weights' sums vary in order from call to call (FP32 atomics). */
 int lbpf_net_backward(lbpf_net* net, const float* dy);
 /* One Adam step (beta 0.9, 0.999) on the mean squared error to `target`
  * (N, H, W, 2), weighted per site (see lbpf_net_set_loss_weight); *loss (may

@@ -1336,7 +1336,7 @@ __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<floa
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // Sum of v over the block's threads with the same tid % q4 (q4 a power of two
-// dividing 256), added to out[4 (tid % q4) ..] by the first q4 threads.
+// dividing 256) into out[4 (tid % q4) ..], by the first q4 threads.
 __device__ __forceinline__ void block_sum4(float4 v, int q4, float* out, float4* red)
 {
     __syncthreads();
@@ -1348,15 +1348,51 @@ __device__ __forceinline__ void block_sum4(float4 v, int q4, float* out, float4*
     }
     if ((int)threadIdx.x < q4) {
         const float4 t = red[threadIdx.x];
-        atomicAdd(out + 4 * threadIdx.x, t.x);
-        atomicAdd(out + 4 * threadIdx.x + 1, t.y);
-        atomicAdd(out + 4 * threadIdx.x + 2, t.z);
-        atomicAdd(out + 4 * threadIdx.x + 3, t.w);
+        out[4 * threadIdx.x] = t.x;
+        out[4 * threadIdx.x + 1] = t.y;
+        out[4 * threadIdx.x + 2] = t.z;
+        out[4 * threadIdx.x + 3] = t.w;
     }
 }
 
+// Bias and head gradients repeat bit for bit: each block of the backward element
+// passes writes its sums as a row of partials, and one launch at the end of the
+// backward pass adds the rows of every gradient in a fixed order, a block per 32
+// columns, 32 rows at a time.  (Float atomics of up to 608 blocks on each value,
+// besides leaving the order open, took longer: the backward pass of 8 x 128^2 with
+// its forward 612 us, 576 this way.)
+__global__ void __launch_bounds__(1024) sum_partials_kernel(const PartialSums q)
+{
+    __shared__ float red[32][33];
+    int k = 0, b = blockIdx.x;
+    while (b >= (q.s[k].width + 31) / 32) b -= (q.s[k++].width + 31) / 32;
+    const PartialSums::Sum m = q.s[k];
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, col = 32 * b + l;
+    float t = 0.f;
+    if (col < m.width) {
+#pragma unroll 4
+        for (int r = w; r < m.rows; r += 32) t += m.part[(size_t)r * m.pitch + col];
+    }
+    red[w][l] = t;
+    __syncthreads();
+    if (w > 0 || col >= m.width) return;
+    t = red[0][l];
+#pragma unroll
+    for (int r = 1; r < 32; ++r) t += red[r][l];
+    m.out[col] += t;
+}
+
+cudaError_t sum_partials(const PartialSums& q, cudaStream_t s)
+{
+    int blocks = 0;
+    for (int k = 0; k < q.n; ++k) blocks += (q.s[k].width + 31) / 32;
+    if (blocks > 0) sum_partials_kernel<<<blocks, 1024, 0, s>>>(q);
+    return cudaGetLastError();
+}
+
 // Gradient before a layer's ReLU and the layer's bias gradient, in one pass:
-//   dst[p][ch] = y[p][ch] > 0 ? g[p][ch] : 0,   db[ch] += sum_p dst[p][ch],
+//   dst[p][ch] = y[p][ch] > 0 ? g[p][ch] : 0,   db[ch] += sum_p dst[p][ch]
+// (the block's part of the sum: part[block][ch], added up by sum_partials),
 // where g is, by `from`:
 //   kFromSame   src[p][ch] (dst may be src);
 //   kFromUp     the sum over the pixel's 2 x 2 children in src (N, 2H, 2W, sc),
@@ -1364,13 +1400,13 @@ __device__ __forceinline__ void block_sum4(float4 v, int q4, float* out, float4*
 //   kFromPool   0.25 src[parent][ch] (N, H/2, W/2, c: backward of the pooling)
 //               + skip[p][so + ch] (N, H, W, sc: the decoder's skip gradient).
 // Bound by memory: 12 to 17 bytes an element.  A thread keeps one channel quad
-// (c / 4 a power of two) and sums it over its pixels; a block adds once.
+// (c / 4 a power of two) and sums it over its pixels.
 // Replaces a ReLU, a pooling or upsampling, an addition and a one-block-a-channel
 // sum (for 16 channels at 8 x 128^2: 76 us of 90, now 8 in all).
 enum { kFromSame, kFromUp, kFromPool };
 template <int FROM>
 __global__ void __launch_bounds__(256) act_bwd_kernel(const float* y, const float* src, const float* skip, float* dst,
-                                                      float* db, long long P, int H, int W, int c, int sc, int so)
+                                                      float* part, long long P, int H, int W, int c, int sc, int so)
 {
     __shared__ float4 red[256];
     const int q4 = c / 4, ch = 4 * ((int)threadIdx.x % q4), ppb = 256 / q4;
@@ -1402,32 +1438,32 @@ __global__ void __launch_bounds__(256) act_bwd_kernel(const float* y, const floa
         st4(dst + p * c + ch, g);
         sum = add4(sum, g);
     }
-    block_sum4(sum, q4, db, red);
+    block_sum4(sum, q4, part + (size_t)blockIdx.x * c, red);
 }
 
-static int act_blocks(long long P, int c)
+int act_blocks(long long P, int c)
 {
     const long long b = (P + 256 / (c / 4) - 1) / (256 / (c / 4));
     return (int)(b < 1 ? 1 : (b > 152 * 4 ? 152 * 4 : b));
 }
 
-cudaError_t act_bwd(const float* y, float* dy, float* db, long long P, int c, cudaStream_t s)
+cudaError_t act_bwd(const float* y, float* dy, float* part, long long P, int c, cudaStream_t s)
 {
-    act_bwd_kernel<kFromSame><<<act_blocks(P, c), 256, 0, s>>>(y, dy, nullptr, dy, db, P, 1, 1, c, 0, 0);
+    act_bwd_kernel<kFromSame><<<act_blocks(P, c), 256, 0, s>>>(y, dy, nullptr, dy, part, P, 1, 1, c, 0, 0);
     return cudaGetLastError();
 }
-cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* db, int N, int H, int W, int c, int sc,
+cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* part, int N, int H, int W, int c, int sc,
                        cudaStream_t s)
 {
     const long long P = (long long)N * H * W;
-    act_bwd_kernel<kFromUp><<<act_blocks(P, c), 256, 0, s>>>(y, src, nullptr, dst, db, P, H, W, c, sc, 0);
+    act_bwd_kernel<kFromUp><<<act_blocks(P, c), 256, 0, s>>>(y, src, nullptr, dst, part, P, H, W, c, sc, 0);
     return cudaGetLastError();
 }
-cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* db, int N, int H, int W,
+cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* part, int N, int H, int W,
                          int c, int sc, int so, cudaStream_t s)
 {
     const long long P = (long long)N * H * W;
-    act_bwd_kernel<kFromPool><<<act_blocks(P, c), 256, 0, s>>>(y, src, skip, dst, db, P, H, W, c, sc, so);
+    act_bwd_kernel<kFromPool><<<act_blocks(P, c), 256, 0, s>>>(y, src, skip, dst, part, P, H, W, c, sc, so);
     return cudaGetLastError();
 }
 
@@ -1500,10 +1536,10 @@ cudaError_t head_fwd(const float* x, const float* w, const float* b, const float
 
 // The head, backward, with the gate and the last layer's ReLU and bias in the
 // same pass: g = (dy0 (1 - phi^2), dy1); dw += g x^T, db += g; dx = w^T g where
-// x > 0 (x is that layer's output), else 0; db_last += sum dx.
+// x > 0 (x is that layer's output), else 0; db_last += sum dx.  The block's parts
+// of the sums are a row of 3 c + 2 partials: dw, db, db_last.
 __global__ void __launch_bounds__(256) head_bwd_kernel(const float* x, const float* dy, const float* w, const float* xin,
-                                                       int cx, float* dx, float* dw, float* db, float* db_last,
-                                                       long long P, int c)
+                                                       int cx, float* dx, float* part, long long P, int c)
 {
     __shared__ float4 red[256];
     const int q4 = c / 4, ch = 4 * ((int)threadIdx.x % q4), ppb = 256 / q4;
@@ -1533,9 +1569,10 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float* x, const flo
             sb.y += g1;
         }
     }
-    block_sum4(s0, q4, dw, red);
-    block_sum4(s1, q4, dw + c, red);
-    block_sum4(sl, q4, db_last, red);
+    float* row = part + (size_t)blockIdx.x * (3 * c + 2);
+    block_sum4(s0, q4, row, red);
+    block_sum4(s1, q4, row + c, red);
+    block_sum4(sl, q4, row + 2 * c + 2, red);
     // db: the first quad's threads hold the two sums
     __syncthreads();
     red[threadIdx.x] = sb;
@@ -1545,15 +1582,15 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float* x, const flo
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        atomicAdd(db, red[0].x);
-        atomicAdd(db + 1, red[0].y);
+        row[2 * c] = red[0].x;
+        row[2 * c + 1] = red[0].y;
     }
 }
 
-cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* dw,
-                     float* db, float* db_last, long long P, int c, cudaStream_t s)
+cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* part,
+                     long long P, int c, cudaStream_t s)
 {
-    head_bwd_kernel<<<act_blocks(P, c), 256, 0, s>>>(x, dy, w, xin, cx, dx, dw, db, db_last, P, c);
+    head_bwd_kernel<<<act_blocks(P, c), 256, 0, s>>>(x, dy, w, xin, cx, dx, part, P, c);
     return cudaGetLastError();
 }
 

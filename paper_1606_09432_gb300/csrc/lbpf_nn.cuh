@@ -35,18 +35,33 @@ cudaError_t conv3x3_wgrad_src(const float* a, const float* b, int ca, int cb, co
 // Gradient through a layer's ReLU and its bias gradient (act_bwd_kernel): in
 // place; from the 2 x 2 children in src (sc channels a pixel); from the pooled
 // gradient src plus the skip gradient (sc channels a pixel, from so on; may be
-// NULL).  c a power of two, 16 .. 256.
-cudaError_t act_bwd(const float* y, float* dy, float* db, long long P, int c, cudaStream_t s);
-cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* db, int N, int H, int W, int c, int sc,
+// NULL).  c a power of two, 16 .. 256.  The bias gradient comes as act_blocks(P, c)
+// rows of c partial sums in part.
+int act_blocks(long long P, int c);
+cudaError_t act_bwd(const float* y, float* dy, float* part, long long P, int c, cudaStream_t s);
+cudaError_t act_bwd_up(const float* y, const float* src, float* dst, float* part, int N, int H, int W, int c, int sc,
                        cudaStream_t s);
-cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* db, int N, int H, int W,
-                         int c, int sc, int so, cudaStream_t s);
+cudaError_t act_bwd_pool(const float* y, const float* src, const float* skip, float* dst, float* part, int N, int H,
+                         int W, int c, int sc, int so, cudaStream_t s);
+// Sums of partials, s[k].out[j] += sum over rows r of s[k].part[r * pitch + j], in
+// an order that depends on the sizes alone.
+struct PartialSums {
+    struct Sum {
+        const float* part;
+        float* out;
+        int rows, pitch, width;
+    };
+    Sum s[20];  // a layer's each, and the head's
+    int n;
+};
+cudaError_t sum_partials(const PartialSums& q, cudaStream_t s);
 cudaError_t pool_fwd(const float* x, float* y, int N, int H, int W, int c, cudaStream_t s);
 // 1x1 head with the interface gate, c <= 64 channels in, 2 out; y may be NULL.
 cudaError_t head_fwd(const float* x, const float* w, const float* b, const float* xin, int cx, float* out, float* y,
                      long long P, int c, cudaStream_t s);
-cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* dw,
-                     float* db, float* db_last, long long P, int c, cudaStream_t s);
+// part: act_blocks(P, c) rows of 3 c + 2 partial sums: dw, db, the last layer's db.
+cudaError_t head_bwd(const float* x, const float* dy, const float* w, const float* xin, int cx, float* dx, float* part,
+                     long long P, int c, cudaStream_t s);
 cudaError_t mse(const float* p, const float* t, const float* x, int cin, int cout, float alpha, float* dp, double* loss,
                 long long n, cudaStream_t s);
 cudaError_t adam(float* w, const float* g, float* m, float* v, __nv_bfloat16* wb, long long n, float lr, float b1,

@@ -30,6 +30,7 @@ struct Conv {
     long long off_w, off_b;  // offsets in the flat FP32 parameter vector
     __nv_bfloat16* wb = nullptr;   // BF16 copy [tap][cout][cin]
     __nv_bfloat16* wt = nullptr;   // flipped BF16 weights for the data gradient
+    float* part = nullptr;         // partial sums of the bias gradient
 };
 
 }  // namespace
@@ -52,6 +53,10 @@ struct lbpf_net {
     // gradient scratch per level (two of the level's widest channel count)
     std::vector<float*> ga, gb;
     float* g_out = nullptr;
+    // partial sums of the head's gradients (and the last layer's bias), and the
+    // table by which they and the layers' are added up
+    float* head_part = nullptr;
+    PartialSums sums{};
     double* d_loss = nullptr;
     std::vector<void*> allocs;
     std::string err;
@@ -198,6 +203,18 @@ extern "C" int lbpf_net_create_arch(int H, int W, int batch, int levels, int bas
         if (ok && l + 1 < levels)
             ok = (net->da[l] = alloc_f(net, Pl * c)) && (net->d[l] = alloc_f(net, Pl * c));
     }
+    // level of conv k: pairs down the encoder, then pairs up the decoder
+    auto level = [&](int k) { return k < 2 * levels ? k / 2 : 2 * levels - 2 - k / 2; };
+    const int nc = (int)net->conv.size(), c0 = net->ch(0), hb = act_blocks(P0, c0);
+    ok = ok && (net->head_part = alloc_f(net, (long long)hb * (3 * c0 + 2)));
+    for (int k = 0; k + 1 < nc && ok; ++k) {
+        Conv& c = net->conv[k];
+        const int rows = act_blocks(P0 >> (2 * level(k)), c.cout);
+        ok = (c.part = alloc_f(net, (long long)rows * c.cout)) != nullptr;
+        net->sums.s[net->sums.n++] = {c.part, net->g + c.off_b, rows, c.cout, c.cout};
+    }
+    net->sums.s[net->sums.n++] = {net->head_part, net->g + net->off_hw, hb, 3 * c0 + 2, 2 * c0 + 2};
+    net->sums.s[net->sums.n++] = {net->head_part + 2 * c0 + 2, net->g + net->conv[nc - 1].off_b, hb, 3 * c0 + 2, c0};
     void* dl = nullptr;
     ok = ok && cudaMalloc(&dl, sizeof(double)) == cudaSuccess;
     if (dl) {
@@ -310,14 +327,15 @@ int forward(lbpf_net* net, const float* x, float* y)
 // Backward from dy (dL/d out); accumulates parameter gradients into g.
 // Mirrors the forward pass: decoder levels from the top down, then the encoder
 // from the deepest level up.  A layer's gradient arrives masked by its ReLU,
-// with its bias gradient already summed (head_bwd, act_bwd*).
+// with the partial sums of its bias gradient taken (head_bwd, act_bwd*), which
+// the last launch adds up.
 int backward(lbpf_net* net, const float* dy)
 {
     const int N = net->N, H = net->H, W = net->W, lv = net->levels;
     const long long P0 = (long long)N * H * W;
     cudaStream_t s = net->stream;
     float* g = net->g;
-    auto bias = [&](int k) { return g + net->conv[k].off_b; };
+    auto bias = [&](int k) { return net->conv[k].part; };
     // weight gradient and data gradient (dx may be NULL) of conv k at level l
     // from the masked gradient dyk of its output
     auto cvb = [&](int k, const float* a, const float* b, int ca, int cb, const float* dyk, float* dx, int l) -> int {
@@ -329,8 +347,7 @@ int backward(lbpf_net* net, const float* dy)
     };
     int rc;
     int k = (int)net->conv.size();
-    NK(head_bwd(net->top(), dy, net->p + net->off_hw, net->xin, kInPad, net->ga[0], g + net->off_hw, g + net->off_hb,
-                bias(k - 1), P0, net->ch(0), s));
+    NK(head_bwd(net->top(), dy, net->p + net->off_hw, net->xin, kInPad, net->ga[0], net->head_part, P0, net->ch(0), s));
     for (int l = 0; l + 1 < lv; ++l) {  // decoder: the masked gradient of d[l] is in ga[l]
         k -= 2;
         const int c = net->ch(l), h = H >> l, w = W >> l;
@@ -360,6 +377,7 @@ int backward(lbpf_net* net, const float* dy)
         if ((rc = cvb(k, l > 0 ? net->pl[l] : net->xin, nullptr, cin, 0, b, l > 0 ? a : nullptr, l))) return rc;
         if (l > 0 && a != net->gb[l]) std::swap(net->ga[l], net->gb[l]);  // level l - 1 reads gb[l]
     }
+    NK(sum_partials(net->sums, s));
     return LBPF_OK;
 }
 
