@@ -284,11 +284,17 @@ constexpr int kOutPitch = 36;  // floats a pixel of the store staging (32 + 4)
 
 // Channels of the convolution's input: all cin from a, or (b set) the first ca
 // from a at half the resolution (nearest 2x upsampling), the others from b.
+// near: offsets of a tile's halo pixels fit in 32 bits (fill_halo_table).
 struct ConvSrc {
     const float* a;
     const float* b;
     int ca, cb;
+    bool near;
 };
+static ConvSrc conv_src(const float* a, const float* b, int ca, int cb, int W)
+{
+    return ConvSrc{a, b, ca, cb, (long long)W * (ca > cb ? ca : cb) <= 0x7fffffff / kHaloY};
+}
 
 __device__ __forceinline__ const float* src_at(const ConvSrc& s, int img, int y, int x, int H, int W, int c)
 {
@@ -309,8 +315,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* b)
 // Offsets (floats) of the halo pixels from the tile's first pixel in the full
 // resolution source and in the half resolution one, for tiles whose halo does
 // not wrap: filled once a block, so that a piece's address is one table entry.
+// Images so wide that an offset may not fit (rows of 1.2e8 floats) go without.
 __device__ __forceinline__ void fill_halo_table(int* tab, const ConvSrc& s, int W, int t, int nt)
 {
+    if (!s.near) return;
     for (int hp = t; hp < kHaloP; hp += nt) {
         const int hy = hp / kHaloX - 1, hx = hp % kHaloX - 1;
         tab[hp] = (hy * W + hx) * (s.b ? s.cb : s.ca);
@@ -329,7 +337,7 @@ __device__ __forceinline__ void load_halo(const ConvSrc& src, const int* tab, un
     const int dq = nt / k8n;
     if (t >= dq * k8n) return;
     const int p0 = t / k8n, k8 = t - p0 * k8n, c = c0 + 8 * k8, end = rows * kHaloX;
-    const bool inside = ty0 > 0 && tx0 > 0 && ty0 + 16 < H && tx0 + 8 < W;
+    const bool inside = src.near && ty0 > 0 && tx0 > 0 && ty0 + 16 < H && tx0 + 8 < W;
     const bool half = src.b && c < src.ca;
     const float* base;
     if (!src.b)
@@ -806,7 +814,7 @@ cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, cons
     if (cin % 16 || ca % 8 || cout_all % (16 * n_tiles) || cin < 16 || cout_all < 16 || H < 1 || W < 1)
         return cudaErrorInvalidValue;
     HaloArgs q;
-    q.src = ConvSrc{a, b, ca, cb};
+    q.src = conv_src(a, b, ca, cb, W);
     q.w = w;
     q.bias = bias;
     q.y = y;
@@ -830,6 +838,8 @@ cudaError_t conv3x3_fwd_src(const float* a, const float* b, int ca, int cb, cons
         CUtensorMap map = {};
         if (q.wst) {
             if (q.KC == 64 && weight_map(q, map)) return launch_halo<4, kTma>(q, map, grid, smem, s);
+            // (blocks of 64 channels by pieces: only where the driver has no tensor-map
+            // encoder, which no test meets)
             return q.KC == 64 ? launch_halo<4, kStream>(q, map, grid, smem, s)
                               : launch_halo<0, kStream>(q, map, grid, smem, s);
         }
@@ -1298,7 +1308,7 @@ cudaError_t conv3x3_wgrad_src(const float* a, const float* b, int ca, int cb, co
     const int n_ntiles = (cin + 255) / 256;
     if (cin % 16 || cout % 16 || cin < 16 || cout < 16 || cin % (16 * n_ntiles)) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
-    if (wgrad_halo(ConvSrc{a, b, ca, cb}, dy, dw, N, H, W, cin, cout, s, e)) return e;
+    if (wgrad_halo(conv_src(a, b, ca, cb, W), dy, dw, N, H, W, cin, cout, s, e)) return e;
     if (b) return cudaErrorInvalidValue;
     const int nci = cin / n_ntiles, n_mtiles = (cout + kConvM - 1) / kConvM;
     const long long P = (long long)N * H * W;
