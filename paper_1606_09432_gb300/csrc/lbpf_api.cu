@@ -688,7 +688,7 @@ extern "C" int lbpf_create(const lbpf_domain* domains, int n_domains, int lattic
 {
     bool vec = true;
     int rc = create(domains, n_domains, lattice, grad, precision, stream, &vec, out);
-    if (rc == LBPF_ENOMEM && vec) {  // its work field and row padding (4 to 8 % of the state) may be what does not fit
+    if (rc == LBPF_ENOMEM && vec) {  // its work field (4 B a site) and row padding may be what does not fit
         vec = false;
         rc = create(domains, n_domains, lattice, grad, precision, stream, &vec, out);
     }

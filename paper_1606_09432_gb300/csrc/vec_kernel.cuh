@@ -22,7 +22,8 @@
 // D3Q27 1260 / 980.  Rows that are not whole vectors are padded in memory
 // (DomainDev::px); a row's last partial vector is computed whole, what falls into
 // the padding is never read.  Full (FP32) storage measured 2-8 % slower this way
-// (the vectors in flight need twice the registers) and stays with step_kernel.
+// (the vectors in flight need twice the registers) and stays with step_kernel;
+// the heat launch apart before a one-site phase-field march was not measured.
 #pragma once
 
 #include <algorithm>
