@@ -50,8 +50,8 @@ __device__ __forceinline__ SiteNb site_nb(const DomainDev& d, long long s, int& 
 __device__ __forceinline__ long long dense_index(const DomainDev& d, long long s)
 {
     if (d.px == d.nx) return s;
-    const long long row = s / d.px, x = s - row * d.px;
-    return x < d.nx ? row * d.nx + x : -1;
+    const uint32_t t = (uint32_t)s, row = t / (uint32_t)d.px, x = t - row * (uint32_t)d.px;  // (padded: n < 2^31)
+    return x < (uint32_t)d.nx ? (long long)(row * (uint32_t)d.nx + x) : -1;
 }
 
 // Gradient of phi at site s in lattice units (Sec. 4.2), global-memory stencil.

@@ -82,7 +82,12 @@ __global__ void __launch_bounds__(256) reduce_kernel(const R* __restrict__ phi, 
     double sf = 0.0, cs = 0.0, bad = 0.0;
     const long long nxy = (long long)nx * ny;
     for (long long s = blockIdx.x * 256LL + threadIdx.x; s < n; s += (long long)gridDim.x * 256) {
-        const double p = (double)phi[px == nx ? s : s / nx * px + s % nx], v = (double)u[s];
+        long long sp = s;
+        if (px != nx) {  // (padded rows: fewer than 2^31 sites)
+            const uint32_t t = (uint32_t)s, row = t / (uint32_t)nx;
+            sp = row * (uint32_t)px + (t - row * (uint32_t)nx);
+        }
+        const double p = (double)phi[sp], v = (double)u[s];
         if (!isfinite(p) || !isfinite(v)) {
             bad += 1.0;
             continue;
@@ -145,22 +150,36 @@ cudaError_t launch_reduce(const void* phi, const void* u, long long n, int preci
     return cudaGetLastError();
 }
 
-// A field between arrays of row pitches dp and sp: 64 threads a row, four rows a
-// block.  Memory bound; it replaces pitched copies, whose rows the copy engines
-// take one by one (351^3, rows of 351 in 352 floats, phi and u from pinned host
-// memory 12.3 ms, 3.4 with this behind a dense copy, 3.25 where rows are dense;
-// phi to the host 1.1, 1.0 and 0.9).
+// A field of rows * nx < 2^31 floats between arrays of row pitches dp and sp, a
+// site a thread in the dense order.  Memory bound; it replaces pitched copies, whose
+// rows the copy engines take one by one (351^3, rows of 351 in 352 floats, phi and
+// u from pinned host memory 12.3 ms, 3.4 with this behind a dense copy, 3.25 where
+// rows are dense; phi to the host 1.1, 1.0 and 0.9).
 __global__ void __launch_bounds__(256) copy_rows_kernel(float* __restrict__ dst, int dp, const float* __restrict__ src,
-                                                        int sp, int nx, long long rows)
+                                                        int sp, int nx, uint32_t n)
 {
-    for (long long r = blockIdx.x * 4LL + threadIdx.y; r < rows; r += gridDim.x * 4LL)
-        for (int x = threadIdx.x; x < nx; x += 64) dst[r * dp + x] = src[r * sp + x];
+    constexpr int B = 4;  // loads in flight
+    const uint32_t step = gridDim.x * 256;
+    for (uint32_t e = blockIdx.x * 256 + threadIdx.x; e < n; e += B * step) {
+        float v[B];
+        uint32_t row[B], x[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            row[k] = (e + k * step) / (uint32_t)nx;
+            x[k] = e + k * step - row[k] * (uint32_t)nx;
+            if (e + k * step < n) v[k] = src[(size_t)row[k] * sp + x[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+            if (e + k * step < n) dst[(size_t)row[k] * dp + x[k]] = v[k];
+    }
 }
 
 cudaError_t launch_copy_rows(float* dst, int dp, const float* src, int sp, int nx, long long rows, cudaStream_t s)
 {
-    const long long b = (rows + 3) / 4;
-    copy_rows_kernel<<<(unsigned)(b < 152 * 16 ? b : 152 * 16), dim3(64, 4), 0, s>>>(dst, dp, src, sp, nx, rows);
+    const long long n = rows * nx, b = (n + 1023) / 1024;
+    if (n >= 1LL << 31) return cudaErrorInvalidValue;
+    copy_rows_kernel<<<(unsigned)(b < 152 * 32 ? b : 152 * 32), 256, 0, s>>>(dst, dp, src, sp, nx, (uint32_t)n);
     return cudaGetLastError();
 }
 
